@@ -8,6 +8,8 @@ import os
 import shutil
 import subprocess
 
+from . import maxwell
+
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
@@ -18,7 +20,8 @@ SOURCES = ["rt_abi.cu", "rt_sample.cu", "rt_trace.cu", "rt_trace_mixed.cu", "rt_
            "rt_flops.cu", "rt_adjoint.cu", "rt_tail.cu", "rt_trace_rot.cu", "rt_peak.cu",
            "rt_rhs.cu", "rt_trace_df.cu"]
 HEADERS = ["rt_device.cuh", "rt_internal.h", "rt_integrator.cuh", "rt_sample_core.cuh",
-           "rt_dual.cuh", "rt_backward.cuh", "rt_df.cuh"]
+           "rt_sample_types.cuh", "rt_maxwell.cuh", "rt_tail.cuh", "rt_dual.cuh",
+           "rt_backward.cuh", "rt_df.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVFLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr",
            "-Xptxas", "-v"]
@@ -46,14 +49,17 @@ def build(force: bool = False, verbose: bool = False) -> str:
     """Compile every CUDA source for sm_103a and link the shared library."""
     nvcc = _nvcc()
     os.makedirs(BUILD, exist_ok=True)
-    hdrs = [os.path.join(CSRC, h) for h in HEADERS] + [os.path.join(INCLUDE, "rt.h")]
+    table = os.path.join(BUILD, "maxwell_table.inc")
+    if force or _stale(table, [maxwell.__file__]):
+        maxwell.write(table)
+    hdrs = [os.path.join(CSRC, h) for h in HEADERS] + [os.path.join(INCLUDE, "rt.h"), table]
     objs, jobs = [], []
     for src in SOURCES:
         s = os.path.join(CSRC, src)
         o = os.path.join(BUILD, src.replace(".cu", ".o"))
         objs.append(o)
         if force or _stale(o, [s] + hdrs):
-            cmd = [nvcc, *ARCH, *NVFLAGS, "-I", INCLUDE, "-I", CSRC, "-c", s, "-o", o]
+            cmd = [nvcc, *ARCH, *NVFLAGS, "-I", INCLUDE, "-I", CSRC, "-I", BUILD, "-c", s, "-o", o]
             jobs.append((src, cmd))
     logs = {}
     with cf.ThreadPoolExecutor(max_workers=max(1, len(jobs))) as ex:

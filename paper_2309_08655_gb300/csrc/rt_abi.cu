@@ -265,10 +265,12 @@ rt_status rt_sample_conversion_surface_part(const rt_star* s, int64_t n, int64_t
   if ((st = check_dev_ptr(d_weight, "d_weight")) != RT_OK) return st;
   if ((st = check_dev_ptr(d_status, "d_status")) != RT_OK) return st;
   rtk::SampleParams p;
-  p.s = s->h;
-  p.n = n;
+  p.stars = s->d;
+  p.nstars = 1;
+  p.begin[0] = 0;
+  p.begin[1] = n;
+  p.norm[0] = n_norm;
   p.ld = n;
-  p.n_norm = n_norm;
   p.u = d_u;
   p.state = d_state;
   p.weight = d_weight;
@@ -1052,14 +1054,18 @@ rt_status rt_sample_batch(rt_batch* b, const double* d_u, double* d_state, doubl
   if ((st = check_dev_ptr(d_state, "d_state")) != RT_OK) return st;
   if ((st = check_dev_ptr(d_weight, "d_weight")) != RT_OK) return st;
   if ((st = check_dev_ptr(d_status, "d_status")) != RT_OK) return st;
-  for (size_t s = 0; s < b->stars.size(); ++s) {
-    const int64_t o = b->off[s], cnt = b->off[s + 1] - o;
-    if (cnt == 0) continue;
+  for (size_t s0 = 0; s0 < b->stars.size(); s0 += rtk::SAMPLE_STARS) {
+    const size_t left = b->stars.size() - s0;
     rtk::SampleParams p;
-    p.s = b->stars[s]->h;
-    p.n = cnt;
+    p.stars = b->d_stars + s0;
+    p.nstars = left < rtk::SAMPLE_STARS ? (int)left : rtk::SAMPLE_STARS;
+    const int64_t o = b->off[s0];
+    for (int s = 0; s < p.nstars; ++s) {
+      p.begin[s] = b->off[s0 + s] - o;
+      p.norm[s] = b->norm.empty() ? b->off[s0 + s + 1] - b->off[s0 + s] : b->norm[s0 + s];
+    }
+    p.begin[p.nstars] = b->off[s0 + p.nstars] - o;
     p.ld = b->N;
-    p.n_norm = b->norm.empty() ? cnt : b->norm[s];
     p.u = d_u + o;
     p.state = d_state + o;
     p.weight = d_weight + o;

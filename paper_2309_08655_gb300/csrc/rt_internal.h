@@ -7,7 +7,7 @@
 #include "rt.h"
 #include "rt_device.cuh"
 #include "rt_dual.cuh"
-#include "rt_sample_core.cuh"
+#include "rt_sample_types.cuh"
 
 #include <nvtx3/nvToolsExt.h>
 
@@ -97,12 +97,15 @@ enum {
 // rt_trace_backward uses slot 5 for its FP64 extremum searches (grazing pairs)
 constexpr int CTR_SEARCH = CTR_PROMOTED_STEPS;
 
+// Sampling of up to SAMPLE_STARS consecutive stars in one launch.
+constexpr int SAMPLE_STARS = 32;
 struct SampleParams {
-  StarDev s;
-  int64_t n;                // samples
-  int64_t ld;               // SoA row stride of u and state (>= n)
-  int64_t n_norm;           // the weights are normalised by n_norm (n, or the
-                            // samples of all shards of one workload)
+  const StarDev* stars;     // device, nstars descriptors
+  int nstars;
+  int64_t begin[SAMPLE_STARS + 1];  // samples of star s: [begin[s], begin[s + 1])
+  int64_t norm[SAMPLE_STARS];       // its weights are normalised by norm[s] (its
+                                    // samples, or those of all shards of one workload)
+  int64_t ld;               // SoA row stride of u and state
   const double* u;
   double* state;
   double* weight;

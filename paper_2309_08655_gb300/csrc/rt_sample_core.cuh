@@ -34,65 +34,11 @@
 
 #include "rt_device.cuh"
 #include "rt_dual.cuh"
+#include "rt_maxwell.cuh"
+#include "rt_sample_types.cuh"
 
 namespace rtk {
 namespace sampling {
-
-constexpr double TWO_OVER_SQRTPI = 1.12837916709551257390;
-
-// Inverse CDF of the Maxwellian speed x = |k_inf| / k0, density
-// (4/sqrt(pi)) x^2 exp(-x^2).  Lower half: erf(x) - c x e^{-x^2} = u; upper
-// half: erfc(x) + c x e^{-x^2} = 1 - u (exact for u >= 1/2), which keeps the
-// tail well conditioned.  Safeguarded Newton iteration.
-// The start of the FP64 iteration: the same safeguarded Newton iteration in
-// FP32 (FP32 exp, erf and erfc issue on the fast pipe) to ~1e-5.  Where FP32
-// cannot resolve the equation (u below ~1e-8: erf(x) and x e^{-x^2} cancel) the
-// FP64 iteration starts from a poor point and takes more steps, nothing else.
-__device__ __forceinline__ float maxwell_seed(bool upper, float v) {
-  const float c = (float)TWO_OVER_SQRTPI;
-  float lo = 0.0f, hi = 30.0f;
-  float x = 1.0876520317f;   // median
-  for (int it = 0; it < 40; ++it) {
-    const float ex = expf(-x * x);
-    const float q = upper ? erfcf(x) + c * x * ex : erff(x) - c * x * ex;
-    const float dq = 2.0f * c * x * x * ex * (upper ? -1.0f : 1.0f);
-    const bool below = upper ? (q > v) : (q < v);
-    if (below) lo = x; else hi = x;
-    float xn = x - (q - v) / dq;
-    if (!(xn > lo && xn < hi)) xn = 0.5f * (lo + hi);
-    if (fabsf(xn - x) <= 1e-5f * x || hi - lo <= 1e-6f * hi) return xn;
-    x = xn;
-  }
-  return x;
-}
-
-__device__ __forceinline__ double maxwell_speed(int fa_model, double u) {
-  if (fa_model == FA_DELTA) return 1.0;
-  const bool upper = u > 0.5;
-  const double v = upper ? 1.0 - u : u;
-  double lo = 0.0, hi = 30.0;
-  double x = (double)maxwell_seed(upper, (float)v);
-  if (!(x > lo && x < hi)) x = 1.0876520317;   // median
-  for (int it = 0; it < 200; ++it) {
-    const double ex = exp(-x * x);
-    const double q = upper ? erfc(x) + TWO_OVER_SQRTPI * x * ex
-                           : erf(x) - TWO_OVER_SQRTPI * x * ex;
-    const double dq = 2.0 * TWO_OVER_SQRTPI * x * x * ex * (upper ? -1.0 : 1.0);
-    // bracket update: the CDF increases with x, the tail decreases
-    const bool below = upper ? (q > v) : (q < v);
-    if (below) lo = x; else hi = x;
-    double xn = x - (q - v) / dq;
-    if (!(xn > lo && xn < hi)) xn = 0.5 * (lo + hi);
-    // converged: a Newton step of a few ulps (one of exactly 1-2 ulps can
-    // recur for ever where q - v is a rounding-level difference)
-    if (fabs(xn - x) <= 1e-15 * x || hi - lo <= 4e-16 * hi) {
-      x = xn;
-      break;
-    }
-    x = xn;
-  }
-  return x;
-}
 
 struct Line {
   int disp, plasma;
@@ -169,27 +115,6 @@ __device__ __forceinline__ double line_G(const Line& L, double r, double* dG) {
 }
 
 
-// Sample constants in the working type T: double for sampling, a dual number
-// for the derivatives of the initial state and the weight with respect to the
-// star parameters (the adjoint).  Only the fields a parameter can move are T.
-template <class T>
-struct SampConst {
-  T rs, cp, sin_tm, cos_tm, B0_eV2, R_eV, n_inf, ma_eV;
-  double v0, psi_fixed, plasma_a, g_eV, w_unit;
-  double rlc;     // light-cylinder radius / R (twisted model: open field lines excluded)
-  double per_cm3; // 1 cm^-3 in eV^3 (the renormalised weights)
-  int disp, plasma, fa_model, phase_mode;
-  int weight_mode;
-};
-
-template <class T>
-struct SampOut {
-  T x[3], k[3];   // scaled state: x / R, covariant k / m_a
-  T w;            // weight [W]
-  double delta, psi;
-  bool ok;
-};
-
 __device__ __forceinline__ double val(double x) { return x; }
 __device__ __forceinline__ double tabs(double x) { return fabs(x); }
 
@@ -223,6 +148,83 @@ __device__ __forceinline__ void line_plasma_t(int plasma, const T& PR, double pa
     }
     default: P = T(0.0); dP = T(0.0); break;
   }
+}
+
+// The root of G on the line for the profiles that fall as a power of r, where
+// G decreases through a single root (0: not found this way).  The bracket and
+// the Newton iteration run in FP32, to ~1e-6; in FP64 G alone is evaluated,
+// and its quotient with the FP32 slope (good to 1e-6) converges in two steps.
+// Every lane does the same two or three FP64 evaluations of G, where the
+// bracketing in FP64 and a Newton iteration to the last bit took five to ten,
+// each with its own count.
+__device__ __forceinline__ double line_root_power(const Line& L, float W2m1) {
+  if (L.plasma != PLASMA_GJ && L.plasma != PLASMA_RADIAL && L.plasma != PLASMA_TWISTED)
+    return 0.0;
+  float lo = 1.0f, hi = 2.0f, dG = 0.0f;
+  for (int it = 0; !(line_G32(L, W2m1, hi, &dG) < 0.0f); ++it) {
+    if (it > 40) return 0.0;
+    lo = hi;
+    hi *= 2.0f;
+  }
+  float x = 0.5f * (lo + hi);
+  for (int it = 0; it < 40; ++it) {
+    const float g = line_G32(L, W2m1, x, &dG);
+    if (g > 0.0f) lo = x; else hi = x;
+    float xn = x - g / dG;
+    if (!(xn > lo && xn < hi)) xn = 0.5f * (lo + hi);
+    const bool done = fabsf(xn - x) <= 1e-5f * x || hi - lo <= 1e-6f * hi;
+    x = xn;
+    if (done) break;
+  }
+  (void)line_G32(L, W2m1, x, &dG);
+  if (!(dG < 0.0f)) return 0.0;
+  const float idG = 1.0f / dG;
+  double r = (double)x;
+  for (int it = 0; it < 8; ++it) {
+    const float step = (float)line_G(L, r, nullptr) * idG;
+    r = fmax(r - (double)step, 1.0);
+    if (fabsf(step) <= 1e-10f * x) return r;
+  }
+  return 0.0;
+}
+
+// The root of G for any profile (0: G does not change sign): bracketed by
+// doubling, then safeguarded Newton to a few ulps from a start that the same
+// iteration finds in FP32.
+static __device__ __noinline__ double line_root(const Line L, float W2m1) {
+  double lo = 1.0, hi = 2.0;
+  int n = 0;
+  while (!(line_G(L, hi, nullptr) < 0.0)) {
+    lo = hi;
+    hi *= 2.0;
+    if (++n > 60) return 0.0;
+  }
+  double r = 0.5 * (lo + hi);
+  {
+    float flo = (float)lo, fhi = (float)hi, fr = (float)r;
+    for (int it = 0; it < 40; ++it) {
+      float dG;
+      const float g = line_G32(L, W2m1, fr, &dG);
+      if (g > 0.0f) flo = fr; else fhi = fr;
+      float rn = fr - g / dG;
+      if (!(rn > flo && rn < fhi)) rn = 0.5f * (flo + fhi);
+      const bool done = fabsf(rn - fr) <= 1e-5f * fr || fhi - flo <= 1e-6f * fhi;
+      fr = rn;
+      if (done) break;
+    }
+    if ((double)fr > lo && (double)fr < hi) r = (double)fr;
+  }
+  for (int it = 0; it < 200; ++it) {
+    double dG;
+    const double g = line_G(L, r, &dG);
+    if (g > 0.0) lo = r; else hi = r;
+    double rn = r - g / dG;
+    if (!(rn > lo && rn < hi)) rn = 0.5 * (lo + hi);
+    const bool done = fabs(rn - r) <= 1e-15 * r || hi - lo <= 4e-16 * hi;
+    r = rn;
+    if (done) break;
+  }
+  return r;
 }
 
 // Gradient of G (units 1/R) at the point x (units of R) of the leaf selected by
@@ -286,9 +288,11 @@ __device__ void sample_core(const SampConst<T>& s, const double* u, double nsamp
   const double kinf = xs * s.v0;
   const double delta = kinf * kinf / (sqrt(1.0 + kinf * kinf) + 1.0);
   const double om = 1.0 + delta;
-  const double psi = (s.phase_mode == PHASE_UNIFORM) ? 2.0 * PI * u[5] : s.psi_fixed;
+  const bool uniform_phase = s.phase_mode == PHASE_UNIFORM;
+  const double psi = uniform_phase ? 2.0 * PI * u[5] : s.psi_fixed;
   double sps, cps;
-  sincos(psi, &sps, &cps);
+  if (uniform_phase) sincospi(2.0 * u[5], &sps, &cps);   // no argument reduction by pi
+  else sincos(psi, &sps, &cps);
   const T m0 = s.sin_tm * T(cps), m1 = s.sin_tm * T(sps), m2 = s.cos_tm;
   // dipole direction b = 3 (m.n) n - m (depends on n only)
   const T mu = m0 * T(n0) + m1 * T(n1) + m2 * T(n2);
@@ -314,42 +318,13 @@ __device__ void sample_core(const SampConst<T>& s, const double* u, double nsamp
   o.delta = delta;
   o.psi = psi;
   o.ok = line_G(L, 1.0, nullptr) > 0.0;
-  double lo = 1.0, hi = 2.0;
-  if (o.ok) {
-    int it = 0;
-    while (!(line_G(L, hi, nullptr) < 0.0)) {
-      lo = hi;
-      hi *= 2.0;
-      if (++it > 60) { o.ok = false; break; }
-    }
-  }
   if (!o.ok) return;
-  // safeguarded Newton on G, from a start the same iteration finds in FP32
-  double r = 0.5 * (lo + hi);
-  {
-    const float W2m1 = (float)(delta * (2.0 + delta));
-    float flo = (float)lo, fhi = (float)hi, fr = (float)r;
-    for (int it = 0; it < 40; ++it) {
-      float dG;
-      const float g = line_G32(L, W2m1, fr, &dG);
-      if (g > 0.0f) flo = fr; else fhi = fr;
-      float rn = fr - g / dG;
-      if (!(rn > flo && rn < fhi)) rn = 0.5f * (flo + fhi);
-      const bool done = fabsf(rn - fr) <= 1e-5f * fr || fhi - flo <= 1e-6f * fhi;
-      fr = rn;
-      if (done) break;
-    }
-    if ((double)fr > lo && (double)fr < hi) r = (double)fr;
-  }
-  for (int it = 0; it < 200; ++it) {
-    double dG;
-    const double g = line_G(L, r, &dG);
-    if (g > 0.0) lo = r; else hi = r;
-    double rn = r - g / dG;
-    if (!(rn > lo && rn < hi)) rn = 0.5 * (lo + hi);
-    const bool done = fabs(rn - r) <= 1e-15 * r || hi - lo <= 4e-16 * hi;
-    r = rn;
-    if (done) break;
+  const float W2m1 = (float)(delta * (2.0 + delta));   // omega_inf^2 - 1
+  double r = line_root_power(L, W2m1);
+  if (r == 0.0) r = line_root(L, W2m1);
+  if (r == 0.0) {
+    o.ok = false;
+    return;
   }
   // twisted magnetosphere: no conversion on open field lines, the dipole
   // lines r / sin^2(theta) = L that reach the light cylinder (L >= r_LC)
@@ -358,10 +333,12 @@ __device__ void sample_core(const SampConst<T>& s, const double* u, double nsamp
     return;
   }
   // G in the working type at the root, for the root's dependence on the constants
-  double dGr;
-  line_G(L, r, &dGr);
   T rT;
-  {
+  if constexpr (std::is_same<T, double>::value) {
+    rT = r;
+  } else {
+    double dGr;
+    line_G(L, r, &dGr);
     T P, dP;
     line_plasma_t(s.plasma, PR, s.plasma_a, n2, T(r), P, dP);
     T G;
@@ -374,36 +351,41 @@ __device__ void sample_core(const SampConst<T>& s, const double* u, double nsamp
     }
     rT = root_of(r, G, dGr);
   }
-  // quantities at the resonance
+  // quantities at the resonance.  One reciprocal each for r and A, one rsqrt
+  // for E and one quotient for the whole weight: an FP64 division is ten
+  // instructions of a pipe that takes 64 cycles for each.
   T P, dP;
   line_plasma_t(s.plasma, PR, s.plasma_a, n2, rT, P, dP);
-  const T A = T(1.0) - s.rs / rT;
-  const T K2 = T(L.W2) / A - T(1.0);
+  const T ir = rt_rcp(rT);
+  const T rsr = s.rs * ir;
+  const T A = T(1.0) - rsr;
+  const T qA = rt_rsqrt(A);
+  const T iA = qA * qA;
+  const T K2 = T(L.W2) * iA - T(1.0);          // on shell with the rounded omega_inf^2
   const T E2 = T(1.0) + K2;
-  const T E = rt_sqrt(E2);
-  T dhdr, shape, hden;   // hden: dh = dG / hden
-  if (s.disp == DISP_ISO) {
-    dhdr = dP / (T(2.0) * E);
-    hden = T(2.0) * E;
-    shape = s2;
-  } else {
-    const T dK2 = -T(L.W2) * s.rs / (rT * rT * A * A);
-    const T dG = dP * (T(1.0) + K2 * s2) + P * s2 * dK2 - dK2;
-    const T ym = K2 * P * c2 / E2;
-    dhdr = dG / (T(2.0) * E * (E2 - ym));
-    hden = T(2.0) * E * (E2 - ym);
-    const T D = c2 * P * (P - T(2.0) * E2) + E2 * E2;
-    shape = E2 * E2 * s2 / D;
-  }
   const T kloc = rt_sqrt(K2);
-  const T ir = T(1.0) / rT;
-  const T Bmag = s.B0_eV2 * T(0.5) * ir * ir * ir * rt_sqrt(bb);
-  const T Psi = T(0.5 * PI * s.g_eV * s.g_eV) * Bmag * Bmag * shape * (E * s.ma_eV);
-  const T r_eV = rT * s.R_eV;
-  const T dh_eV = tabs(dhdr) * s.ma_eV / s.R_eV;
-  // the weight per unit of Psi (the conversion probability's numerator)
-  const T W1 = T(4.0 * PI) * r_eV * r_eV * (kloc / T(kinf)) * s.n_inf / (A * dh_eV);
-  o.w = W1 * Psi / T(nsamp) * T(s.w_unit);
+  // dh/dr = dG / hden with hden = 2 E (E^2 - y_minus) = 2 hE / E (isotropic: 2 E),
+  // the shape factor E^4 s2 / D = shape / D
+  T dG, hE, shape, D;
+  if (s.disp == DISP_ISO) {
+    dG = dP;
+    hE = E2;
+    shape = s2;
+    D = T(1.0);
+  } else {
+    const T dK2 = -T(L.W2) * rsr * ir * iA * iA;
+    const T E4 = E2 * E2;
+    dG = dP * (T(1.0) + K2 * s2) + P * s2 * dK2 - dK2;
+    hE = E4 - K2 * P * c2;
+    D = c2 * P * (P - T(2.0) * E2) + E4;
+    shape = E4 * s2;
+  }
+  // w = W1 Psi, W1 = 4 pi r^2 (kloc / kinf) n_inf / (A |dh/dr|) and
+  // Psi = (pi/2) g^2 (B0/2)^2 r^-6 bb (shape / D) E, the sizes in eV
+  const T pre = T(PI * PI * s.g_eV * s.g_eV * s.w_unit) * s.n_inf * s.B0_eV2 * s.B0_eV2 *
+                (s.R_eV * s.R_eV * s.R_eV);
+  const T ir2 = ir * ir;
+  o.w = pre * (ir2 * ir2) * bb * kloc * hE * shape / (T(nsamp * kinf) * A * tabs(dG) * D);
   if constexpr (std::is_same<T, double>::value) {
     if (s.weight_mode == WEIGHT_UNIT_P || s.weight_mode == WEIGHT_RENORM) {
       // conversion probability set to one (Sec. 5.1): divide by
@@ -421,8 +403,10 @@ __device__ void sample_core(const SampConst<T>& s, const double* u, double nsamp
         const double ni = (i == 0) ? n0 : (i == 1) ? n1 : n2;
         kg += q[i] * (g[i] + (sA - 1.0) * gn * ni);
       }
-      const double kdE = kloc * s.ma_eV * fabs(kg / hden) * s.ma_eV / s.R_eV;   // [eV^3]
-      o.w = W1 * kdE / nsamp * s.w_unit;
+      // W1 |k . dE|: the factor 1 / hden of dE and of dh cancel
+      const double r_eV = rT * s.R_eV;
+      const double W1 = 4.0 * PI * r_eV * r_eV * (kloc / kinf) * s.n_inf / (A * fabs(dG));
+      o.w = W1 * (kloc * s.ma_eV * fabs(kg)) / nsamp * s.w_unit;
       if (s.weight_mode == WEIGHT_RENORM) {
         // Eq. reweight: x (1 cm^-3 / n_a(r)) (m_a / |k_a|) / sqrt(1 - r_s / r), the
         // focused density of the monochromatic distribution n_inf k_c / k0,
@@ -435,7 +419,7 @@ __device__ void sample_core(const SampConst<T>& s, const double* u, double nsamp
   // photon phase-space point: orthonormal k = |k| khat; covariant Cartesian
   // k = k_o + (1/sqrt(A) - 1) (n.k_o) n
   const T nko = kloc * T(n0 * q0 + n1 * q1 + n2 * q2);
-  const T cr = (T(1.0) / rt_sqrt(A) - T(1.0)) * nko;
+  const T cr = (qA - T(1.0)) * nko;
   o.x[0] = rT * T(n0);
   o.x[1] = rT * T(n1);
   o.x[2] = rT * T(n2);
