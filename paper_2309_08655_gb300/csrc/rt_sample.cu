@@ -20,59 +20,105 @@ namespace {
 
 using namespace sampling;
 
-__global__ void __launch_bounds__(128) sample_kernel(const SampleParams p) {
+__device__ __forceinline__ SampConst<double> sample_const(const StarDev& s) {
+  SampConst<double> c;
+  c.rs = s.rs;
+  c.cp = s.cp;
+  c.sin_tm = s.sin_tm;
+  c.cos_tm = s.cos_tm;
+  c.B0_eV2 = s.B0_eV2;
+  c.R_eV = s.R_eV;
+  c.n_inf = s.n_inf;
+  c.ma_eV = s.ma_eV;
+  c.v0 = s.v0;
+  c.psi_fixed = s.psi_fixed;
+  c.plasma_a = s.plasma_a;
+  c.rlc = s.rlc;
+  c.g_eV = s.g_eV;
+  c.w_unit = s.w_unit;
+  c.disp = s.dispersion;
+  c.plasma = s.plasma;
+  c.fa_model = s.fa_model;
+  c.phase_mode = s.phase_mode;
+  c.weight_mode = s.weight_mode;
+  c.per_cm3 = PER_CM3_EV3;
+  return c;
+}
+
+__device__ __forceinline__ int star_of_sample(const SampleParams& p, int64_t i) {
+  int star = 0;                                  // begin[star] <= i < begin[star + 1]
+  for (int hi = p.nstars - 1; star < hi;) {
+    const int mid = (star + hi + 1) >> 1;
+    if (p.begin[mid] <= i) star = mid; else hi = mid - 1;
+  }
+  return star;
+}
+
+__device__ __forceinline__ void store_state(const SampleParams& p, const StarDev& s, int64_t i,
+                                            const SampOut<double>& o) {
+  const int64_t ld = p.ld;
+  p.state[6 * ld + i] = o.delta;
+  p.state[7 * ld + i] = o.psi;
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    p.state[j * ld + i] = o.ok ? o.x[j] * s.R_km : 0.0;
+    p.state[(3 + j) * ld + i] = o.ok ? o.k[j] * s.ma_eV : 0.0;
+  }
+  p.status[i] = o.ok ? RAY_READY : RAY_NO_ROOT;
+}
+
+// The samples next to the null cone (about 2 % of a Goldreich-Julian star's) are
+// listed by their block and sampled once more by sample_state_iterated, a full
+// block of them at a time: scattered over the warps, their iterations would hold
+// every warp for a lane or two.
+constexpr int SAMPLE_BLOCK = 128;
+constexpr int LISTED = 2 * SAMPLE_BLOCK;
+
+__global__ void __launch_bounds__(SAMPLE_BLOCK) sample_kernel(const SampleParams p) {
+  __shared__ int64_t listed[LISTED];
+  __shared__ int nlisted;
+  if (threadIdx.x == 0) nlisted = 0;
+  __syncthreads();
   const int64_t n = p.begin[p.nstars], ld = p.ld;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    int star = 0;                                // begin[star] <= i < begin[star + 1]
-    for (int hi = p.nstars - 1; star < hi;) {
-      const int mid = (star + hi + 1) >> 1;
-      if (p.begin[mid] <= i) star = mid; else hi = mid - 1;
-    }
-    const StarDev& s = p.stars[star];
-    SampConst<double> c;
-    c.rs = s.rs;
-    c.cp = s.cp;
-    c.sin_tm = s.sin_tm;
-    c.cos_tm = s.cos_tm;
-    c.B0_eV2 = s.B0_eV2;
-    c.R_eV = s.R_eV;
-    c.n_inf = s.n_inf;
-    c.ma_eV = s.ma_eV;
-    c.v0 = s.v0;
-    c.psi_fixed = s.psi_fixed;
-    c.plasma_a = s.plasma_a;
-    c.rlc = s.rlc;
-    c.g_eV = s.g_eV;
-    c.w_unit = s.w_unit;
-    c.disp = s.dispersion;
-    c.plasma = s.plasma;
-    c.fa_model = s.fa_model;
-    c.phase_mode = s.phase_mode;
-    c.weight_mode = s.weight_mode;
-    c.per_cm3 = PER_CM3_EV3;
-    double u[6];
+  for (int64_t base = blockIdx.x * (int64_t)SAMPLE_BLOCK;; base += (int64_t)gridDim.x * SAMPLE_BLOCK) {
+    const int64_t i = base + threadIdx.x;
+    if (i < n) {
+      const int star = star_of_sample(p, i);
+      const StarDev& s = p.stars[star];
+      const SampConst<double> c = sample_const(s);
+      double u[6];
 #pragma unroll
-    for (int j = 0; j < 6; ++j) u[j] = p.u[j * ld + i];
-    SampOut<double> o;
-    sample_core(c, u, (double)p.norm[star], o);
-    p.state[6 * ld + i] = o.delta;
-    p.state[7 * ld + i] = o.psi;
-    if (!o.ok) {
-#pragma unroll
-      for (int j = 0; j < 6; ++j) p.state[j * ld + i] = 0.0;
-      p.weight[i] = 0.0;
-      p.status[i] = RAY_NO_ROOT;
-      continue;
+      for (int j = 0; j < 6; ++j) u[j] = p.u[j * ld + i];
+      SampOut<double> o;
+      sample_core(c, u, (double)p.norm[star], o);
+      store_state(p, s, i, o);
+      p.weight[i] = o.ok ? o.w : 0.0;
+      if (o.ok && next_to_null_cone(c, o.x, o.psi)) listed[atomicAdd(&nlisted, 1)] = i;
     }
-    p.weight[i] = o.w;
-    p.state[i] = o.x[0] * s.R_km;
-    p.state[ld + i] = o.x[1] * s.R_km;
-    p.state[2 * ld + i] = o.x[2] * s.R_km;
-    p.state[3 * ld + i] = o.k[0] * s.ma_eV;
-    p.state[4 * ld + i] = o.k[1] * s.ma_eV;
-    p.state[5 * ld + i] = o.k[2] * s.ma_eV;
-    p.status[i] = RAY_READY;
+    // (base is the block's: every thread leaves the loop in the same pass)
+    const bool last = base + (int64_t)gridDim.x * SAMPLE_BLOCK >= n;
+    __syncthreads();
+    const int m = nlisted;
+    __syncthreads();
+    if (m < SAMPLE_BLOCK && !last) continue;     // at most LISTED - SAMPLE_BLOCK remain
+    // entry j to warp j mod 4: a few entries take a warp each, on four schedulers
+    constexpr int WARPS = SAMPLE_BLOCK / 32;
+    for (int j = (threadIdx.x & 31) * WARPS + (threadIdx.x >> 5); j < m; j += SAMPLE_BLOCK) {
+      const int64_t q = listed[j];
+      const StarDev& s = p.stars[star_of_sample(p, q)];
+      const SampConst<double> c = sample_const(s);
+      double u[6];
+#pragma unroll
+      for (int k = 0; k < 6; ++k) u[k] = p.u[k * ld + q];
+      SampOut<double> o;
+      sample_state_iterated(c, u, o);
+      store_state(p, s, q, o);
+      if (!o.ok) p.weight[q] = 0.0;
+    }
+    if (last) break;
+    __syncthreads();
+    if (threadIdx.x == 0) nlisted = 0;
+    __syncthreads();
   }
 }
 
@@ -86,11 +132,15 @@ cudaError_t launch_sample(const SampleParams& p, cudaStream_t stream) {
   if (e != cudaSuccess) return e;
   e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
-  const int block = 128;
-  int64_t grid = (n + block - 1) / block;
-  const int64_t cap = (int64_t)nsm * 64;
+  // resident blocks only, so that each gathers enough samples next to the cone
+  // to fill its warps with them
+  int occ = 0;
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, sample_kernel, SAMPLE_BLOCK, 0);
+  if (e != cudaSuccess) return e;
+  int64_t grid = (n + SAMPLE_BLOCK - 1) / SAMPLE_BLOCK;
+  const int64_t cap = (int64_t)nsm * (occ > 0 ? occ : 1);
   if (grid > cap) grid = cap;
-  sample_kernel<<<(unsigned)grid, block, 0, stream>>>(p);
+  sample_kernel<<<(unsigned)grid, SAMPLE_BLOCK, 0, stream>>>(p);
   return cudaGetLastError();
 }
 

@@ -428,5 +428,86 @@ __device__ void sample_core(const SampConst<T>& s, const double* u, double nsamp
   o.k[2] = kloc * T(q2) + cr * T(n2);
 }
 
+// Squared angle within which a Goldreich-Julian sample counts as next to the
+// null cone: 1e-2 rad (the cost-ordered claims' two nearest buckets), with room
+// for this test's FP32 rounding.
+constexpr float GUIDED_DIST2 = 1.05e-4f;
+
+// Whether a sample lies within GUIDED_DIST2 of the null cone, (F / |grad_n F|)^2 as
+// cone_dist2 of rt_integrator.cuh, in FP32.
+__device__ __forceinline__ bool next_to_null_cone(const SampConst<double>& s, const double* x,
+                                                  double psi) {
+  if (s.plasma != PLASMA_GJ) return false;
+  const float x0 = (float)x[0], x1 = (float)x[1], x2 = (float)x[2];
+  float sp, cp;
+  sincosf((float)psi, &sp, &cp);
+  const float st = (float)s.sin_tm, m2 = (float)s.cos_tm;
+  const float ir = rsqrtf(x0 * x0 + x1 * x1 + x2 * x2), n2 = x2 * ir;
+  const float mu = st * (cp * x0 + sp * x1) * ir + m2 * n2;
+  const float F = 3.0f * n2 * mu - m2, c = 6.0f * mu * n2;
+  const float g2 = 9.0f * (mu * mu + n2 * n2) + 18.0f * mu * n2 * m2 - c * c;
+  return F * F < GUIDED_DIST2 * g2;
+}
+
+// The state of one sample (not its weight) by iterating the speed and the
+// resonance radius to the last bit in FP64.  For the samples next to the null
+// cone: a ray guided along it for thousands of steps carries a last-bit change of
+// its start to another end point (in the mixed-precision trace, to another bin or
+// fate), so these starts keep this arithmetic, operation for operation.
+__device__ __forceinline__ void sample_state_iterated(const SampConst<double>& s, const double* u,
+                                                      SampOut<double>& o) {
+  const double ct = 1.0 - 2.0 * u[0];
+  const double st = sqrt(fmax(0.0, (1.0 - ct) * (1.0 + ct)));
+  double sph, cph;
+  sincospi(2.0 * u[1], &sph, &cph);
+  const double n0 = st * cph, n1 = st * sph, n2 = ct;
+  const double ck = 1.0 - 2.0 * u[2];
+  const double sk = sqrt(fmax(0.0, (1.0 - ck) * (1.0 + ck)));
+  double spk, cpk;
+  sincospi(2.0 * u[3], &spk, &cpk);
+  const double q0 = sk * cpk, q1 = sk * spk, q2 = ck;
+  const double kinf = (s.fa_model == FA_DELTA ? 1.0 : maxwell_newton(u[4])) * s.v0;
+  const double delta = kinf * kinf / (sqrt(1.0 + kinf * kinf) + 1.0);
+  const double om = 1.0 + delta;
+  const double psi = (s.phase_mode == PHASE_UNIFORM) ? 2.0 * PI * u[5] : s.psi_fixed;
+  double sps, cps;
+  sincos(psi, &sps, &cps);
+  const double m0 = s.sin_tm * cps, m1 = s.sin_tm * sps, m2 = s.cos_tm;
+  const double mu = m0 * n0 + m1 * n1 + m2 * n2;
+  const double b0 = 3.0 * mu * n0 - m0, b1 = 3.0 * mu * n1 - m1, b2 = 3.0 * mu * n2 - m2;
+  const double bb = 3.0 * mu * mu + 1.0;
+  const double kb = q0 * b0 + q1 * b1 + q2 * b2;
+  const double c2 = kb * kb / bb;
+  Line L;
+  L.disp = s.disp;
+  L.plasma = s.plasma;
+  L.rs = s.rs;
+  L.W2 = om * om;
+  L.s2 = 1.0 - c2;
+  L.PR = s.cp * fabs(3.0 * n2 * mu - m2);
+  L.pa = s.plasma_a;
+  L.nz = n2;
+  o.delta = delta;
+  o.psi = psi;
+  o.ok = line_G(L, 1.0, nullptr) > 0.0;
+  if (!o.ok) return;
+  const double r = line_root(L, (float)(delta * (2.0 + delta)));
+  if (r == 0.0) {
+    o.ok = false;
+    return;
+  }
+  const double A = 1.0 - s.rs / r;
+  const double K2 = L.W2 / A - 1.0;
+  const double kloc = sqrt(K2);
+  const double nko = kloc * (n0 * q0 + n1 * q1 + n2 * q2);
+  const double cr = (1.0 / sqrt(A) - 1.0) * nko;
+  o.x[0] = r * n0;
+  o.x[1] = r * n1;
+  o.x[2] = r * n2;
+  o.k[0] = kloc * q0 + cr * n0;
+  o.k[1] = kloc * q1 + cr * n1;
+  o.k[2] = kloc * q2 + cr * n2;
+}
+
 }  // namespace sampling
 }  // namespace rtk

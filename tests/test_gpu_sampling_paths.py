@@ -87,3 +87,20 @@ def test_conversion_next_to_the_surface(oracle, scale):
     assert np.array_equal(s, s_o) and (s == oracle.RAY_READY).all()
     assert G.rel_state_diff(st, st_o).max() < 1e-12
     assert np.abs(w / w_o - 1).max() < 1e-11
+
+
+@pytest.mark.parametrize("n,theta", [(1, 0.0), (130, 0.0), (1000, 0.0), (70001, 0.5)])
+def test_samples_next_to_the_null_cone(oracle, n, theta):
+    """Every sample within 1e-2 rad of the cone: the blocks' lists fill and flush, the
+    last one partly filled; and an inclined star, whose lists gather a few of many."""
+    kw = dict(I.star_config0(), theta_m=theta, psi=0.0, phase_mode=0)
+    u = I.sample_uniforms(5, n)
+    if theta == 0.0:                     # the cone of the aligned star: cos^2 = 1/3
+        u[0] = 0.5 * (1 - np.cos(np.arccos(1 / np.sqrt(3)) + 5e-3 * (2 * u[0] - 1)))
+    _, st, w, s, _ = G.gpu_sample(kw, u)
+    st_o, w_o, s_o = oracle.sample(oracle.star_vector(**kw), u)
+    st, w, s = G.to_np(st, w, s)
+    assert np.array_equal(s, s_o)
+    ok = s_o == oracle.RAY_READY
+    assert G.rel_state_diff(st[:, ok], st_o[:, ok]).max(initial=0.0) < 1e-12
+    assert np.abs(w[ok] / w_o[ok] - 1).max(initial=0.0) < 1e-11
