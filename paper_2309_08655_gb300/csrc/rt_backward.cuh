@@ -17,7 +17,7 @@
 // not certain); the slope of the screened quantity along th, also in FP32,
 // brackets the extrema of g that turn toward zero, and where a tangent-line
 // bound lets such a dip reach zero the extremum is located in FP64 by
-// bisection on the sign of dg/dth.  Every root is located by FP64 bisection.
+// Illinois on dg/dth.  Every root is located in FP64.
 
 #pragma once
 #include <cuda_runtime.h>
@@ -34,6 +34,7 @@ constexpr int BACK_SUBDIV = 16;
 // (far from the resonance N ~ -1; a smooth dip of N by more than 0.5 within a
 // sixteenth of a step that resolves the ray to rtol does not occur).
 constexpr float SLOPE_NEAR = 0.5f;
+constexpr double ROOT_TOL = 0x1p-49;
 
 struct BackParams {
   StarDev s;
@@ -398,17 +399,30 @@ struct CrossingAcc {
     sum += sA * Psi * ratio;
   }
 
-  // Locates the sign change of g on [lo, hi] (g(lo) < 0 iff negA) by FP64
-  // bisection on dense64 and adds its contribution.
+  // Locates the sign change of g on [lo, hi] (g(lo) < 0 iff negA) in FP64 on
+  // dense64 and adds its contribution: Illinois to ROOT_TOL (below the rounding
+  // of g over its slope), bisection-guarded where that stalls.  About nine
+  // evaluations of g, ~70 FP64 instructions each at one or two live lanes,
+  // where bisection to the last bit took about fifty.
   template <class Dense64>
   __device__ void root(const RayConst<double>& c, double lo, double hi, bool negA,
                        Dense64& dense64) {
     double yd[6];
-    for (int it = 0; it < 200; ++it) {
-      const double mid = 0.5 * (lo + hi);
-      if (mid <= lo || mid >= hi) break;
-      dense64(mid, yd, nullptr);
-      if ((crossing_g(c, W, yd) < 0.0) == negA) lo = mid; else hi = mid;
+    // s g, of the start's sign (>= 0) at lo and of the other at hi; -g and g
+    // share their sign test: g = 0 counts as the positive side
+    auto side = [&](double th) {
+      dense64(th, yd, nullptr);
+      const double g = crossing_g(c, W, yd);
+      return negA ? (g < 0.0 ? -g : fmin(-g, -1e-300)) : g;
+    };
+    double flo = side(lo), fhi = side(hi);
+    if (!(flo >= 0.0)) flo = 0.0;
+    if (!(fhi < 0.0)) fhi = -1e-300;
+    illinois(side, lo, hi, flo, fhi, ROOT_TOL, 40);
+    if (hi - lo > ROOT_TOL * hi) {
+      double h2;
+      lo = last_nonneg(side, flo, fhi, &h2, lo, hi);
+      hi = h2;
     }
     dense64(0.5 * (lo + hi), yd, nullptr);
     contribution(c, yd);
@@ -460,7 +474,7 @@ struct CrossingAcc {
   // sign of g at BACK_SUBDIV + 1 points, screened in FP32 on the pieces
   // p2..p5 of y(th) - y = th (p2 + (1 - th) (p3 + th (p4 + (1 - th) p5)))
   // about y32, evaluated in FP64 at dense64(th) where the screen leaves it
-  // open; every sign change located by FP64 bisection; and between two
+  // open; every sign change located in FP64; and between two
   // samples of one sign, an extremum of g turning toward zero (bracketed by
   // the FP32 slope of the screened N) searched in FP64 where the two tangent
   // lines at the samples meet within the screen's margin of zero.

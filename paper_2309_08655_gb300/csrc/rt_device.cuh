@@ -232,6 +232,151 @@ RT_HD __forceinline__ void ham_rhs(const RayConst<T>& c, const T x0, const T x1,
   dk2 = -gx2;
 }
 
+// Small exact factors and summands.  Overloaded for the composite scalars
+// (rt_df.cuh, rt_dual.cuh), which take them without a full product or sum.
+template <class T>
+RT_HD __forceinline__ T rt_twice(const T& x) { return x + x; }
+template <class T>
+RT_HD __forceinline__ T rt_times(const T& x, int c) { return T(c) * x; }
+template <class T>
+RT_HD __forceinline__ T rt_plus_one(const T& x) { return T(1) + x; }
+
+// The Hamiltonian's derivatives with respect to the constants that a star's
+// parameters move: cp dH/dcp, dH/drs, and dH/dm . dm for a given turn dm of the
+// magnetic axis.
+template <class T>
+struct ConstGrad {
+  T dm0, dm1, dm2;   // in
+  T cp, rs, m;       // out
+};
+
+// The right-hand side of ham_rhs in fewer operations, for the scalars whose
+// arithmetic is the kernel's time: FP64 (one warp instruction holds its
+// sub-partition for 64 cycles here), double-float (7-20 FP32 instructions an
+// operation, and code size) and their dual numbers.  Every vector of Hamilton's
+// equations is a combination of n, k, m and e_z, so the scalar coefficients
+// are summed first and the vectors formed once:
+//
+//   dx/dl =  2 k + bx n + gm m,        gm = 2 P A Kp / (W2 |b|), c1 = mu (1 + 2 sqrt(A)),
+//                                      bx = -2 (rs/r) kr - gm c1
+//   dk/dl = -(Cn n + (bx/r) k + Cm m + Cz e_z)
+//
+// with the plasma's gradient as dP = t (qn n + qm m + qz e_z).  That the
+// coefficient of k is bx/r follows from rotational symmetry about n.  About 105
+// FP64 instructions for the Goldreich-Julian anisotropic medium where ham_rhs
+// takes about 170; the results differ by rounding.  DW: *dw = dH/dW2, as
+// ham_rhs.  CG: *cg = the derivatives with respect to the star's constants
+// (with dual numbers in the direction u, their tangents are u . grad_y of them:
+// the parameter part of a Jacobian product without a tangent per parameter).
+template <class T, bool DW = false, bool CG = false>
+RT_HD __forceinline__ void ham_rhs64(const RayConst<T>& c, const T x0, const T x1, const T x2,
+                                     const T k0, const T k1, const T k2, T& dx0, T& dx1, T& dx2,
+                                     T& dk0, T& dk1, T& dk2, T* dw = nullptr,
+                                     ConstGrad<T>* cg = nullptr) {
+  const T r2 = x0 * x0 + x1 * x1 + x2 * x2;
+  const T ir = rt_rsqrt(r2);
+  const T n0 = x0 * ir, n1 = x1 * ir, n2 = x2 * ir;
+  const T ir2 = ir * ir;
+  const T u = c.rs * ir;
+  const T A = rt_plus_one(-u);
+  const T qA = rt_rsqrt(A);
+  const T iA = qA * qA;
+  const T kr = n0 * k0 + n1 * k1 + n2 * k2;
+  const T mu = c.m0 * n0 + c.m1 * n1 + c.m2 * n2;
+  const T mu3 = rt_times(mu, 3);
+  // P and dP = t (qn n + qm m + qz e_z)
+  T P = T(0), t = T(0), qn = T(0), qm = T(0), qz = T(0);
+  T dPdm = T(0);                                 // dP/dm . dm (CG)
+  if (c.plasma == PLASMA_GJ) {
+    const T g3 = c.cp * c.sig * (ir2 * ir);
+    const T mn = mu * n2;
+    const T F = rt_times(mn, 3) - c.m2;
+    P = g3 * F;
+    t = g3 * ir;
+    qn = rt_times(c.m2, 3) - rt_times(mn, 15);
+    qm = rt_times(n2, 3);
+    qz = mu3;
+    if (CG) dPdm = g3 * (qm * (n0 * cg->dm0 + n1 * cg->dm1 + n2 * cg->dm2) - cg->dm2);
+  } else if (c.plasma == PLASMA_TWISTED) {
+    const T g4 = c.cp * (ir2 * ir2);
+    const T mm = mu * mu;
+    P = g4 * rt_plus_one(-mm);
+    t = rt_twice(g4 * ir);
+    qn = rt_times(mm, 3) - T(2);
+    qm = -mu;
+    if (CG) dPdm = -rt_twice(g4 * mu) * (n0 * cg->dm0 + n1 * cg->dm1 + n2 * cg->dm2);
+  } else if (c.plasma == PLASMA_RADIAL) {
+    P = c.pa * (ir2 * ir);
+    t = P * ir;
+    qn = T(-3);
+  } else if (c.plasma == PLASMA_LINEAR_Z) {
+    P = c.pa * x2;
+    t = c.pa;
+    qz = T(1);
+  } else if (c.plasma == PLASMA_HOMOG) {
+    P = c.pa;
+  }
+  const T v = c.rs * ir2;                        // dA/dr
+  const T iA2 = iA * iA;
+  // dH/dr of the metric part: v (W2/A^2 + kr^2) and the turn of n, 2 v kr^2
+  T s = c.W2 * iA2 + rt_times(kr * kr, 3);
+  const T bx0 = -rt_twice(u * kr);
+  if (c.disp == DISP_ISO) {
+    const T Cn = v * s + t * qn, Ck = bx0 * ir, Cm = t * qm;
+    dx0 = rt_twice(k0) + bx0 * n0;
+    dx1 = rt_twice(k1) + bx0 * n1;
+    dx2 = rt_twice(k2) + bx0 * n2;
+    dk0 = -(Cn * n0 + Ck * k0 + Cm * c.m0);
+    dk1 = -(Cn * n1 + Ck * k1 + Cm * c.m1);
+    dk2 = -(Cn * n2 + Ck * k2 + Cm * c.m2 + t * qz);
+    if (DW) *dw = -iA;
+    if (CG) {
+      cg->cp = (c.plasma == PLASMA_GJ || c.plasma == PLASMA_TWISTED) ? P : T(0);
+      cg->rs = -(ir * (c.W2 * iA2 + kr * kr));   // dA/drs = -1/r
+      cg->m = dPdm;
+    }
+    return;
+  }
+  const T ib = rt_rsqrt(rt_plus_one(mu3 * mu));
+  const T sA = A * qA;
+  const T opsA = rt_plus_one(rt_twice(sA));
+  const T km = k0 * c.m0 + k1 * c.m1 + k2 * c.m2;
+  const T c1 = mu * opsA;
+  const T U = c1 * kr - km;
+  const T Kp = U * ib;
+  const T q = Kp * c.iW2;
+  const T Kq = Kp * q;                           // Kp^2 / W2
+  const T one_m = rt_plus_one(-(A * Kq));
+  const T gm = (P * A) * (rt_twice(q) * ib);
+  const T bx = bx0 - gm * c1;
+  dx0 = rt_twice(k0) + bx * n0 + gm * c.m0;
+  dx1 = rt_twice(k1) + bx * n1 + gm * c.m1;
+  dx2 = rt_twice(k2) + bx * n2 + gm * c.m2;
+  const T ib2 = ib * ib;
+  const T okr = opsA * kr;
+  const T a1 = okr - (mu3 * U) * ib2;            // |b| dKp/dmu at fixed kr, km
+  const T a3 = (mu * kr) * (v * qA);             // |b| dKp/dr through sqrt(A)
+  const T gmr = gm * ir;
+  const T w = t * one_m;
+  s = s - P * Kq;
+  const T Cn = v * s + w * qn + gmr * (a1 * mu + c1 * kr) - gm * a3;
+  const T Ck = bx * ir;
+  const T Cm = w * qm - gmr * a1;
+  dk0 = -(Cn * n0 + Ck * k0 + Cm * c.m0);
+  dk1 = -(Cn * n1 + Ck * k1 + Cm * c.m1);
+  dk2 = -(Cn * n2 + Ck * k2 + Cm * c.m2 + w * qz);
+  if (DW) *dw = (P * A) * (Kq * c.iW2) - iA;
+  if (CG) {
+    cg->cp = (c.plasma == PLASMA_GJ || c.plasma == PLASMA_TWISTED) ? P * one_m : T(0);
+    // dH/dA = W2/A^2 + kr^2 - P Kq - (P A 2 Kp/W2) dKp/dA, dKp/dA = mu kr / (sqrt(A) |b|)
+    cg->rs = -(ir * ((c.W2 * iA2 + kr * kr) - P * Kq - gm * ((mu * kr) * qA)));
+    // U = k.b + ..: dU/dm . dm = opsA kr dmu - k.dm, d|b|^2 = 6 mu dmu
+    const T dmu = n0 * cg->dm0 + n1 * cg->dm1 + n2 * cg->dm2;
+    const T dkm = k0 * cg->dm0 + k1 * cg->dm1 + k2 * cg->dm2;
+    cg->m = dPdm * one_m - gm * (a1 * dmu - dkm);
+  }
+}
+
 // The value of H (diagnostics).
 template <class T>
 __device__ __forceinline__ T ham_value(const RayConst<T>& c, const T* x, const T* k) {

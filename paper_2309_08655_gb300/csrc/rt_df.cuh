@@ -109,6 +109,11 @@ RT_HD __forceinline__ bool operator>=(DF a, DF b) { return !(a < b); }
 RT_HD __forceinline__ bool operator==(DF a, DF b) { return a.hi == b.hi && a.lo == b.lo; }
 RT_HD __forceinline__ bool operator!=(DF a, DF b) { return !(a == b); }
 
+// exact, and without a full product (ham_rhs64)
+RT_HD __forceinline__ DF rt_twice(const DF& x) { return DF(2.0f * x.hi, 2.0f * x.lo); }
+RT_HD __forceinline__ DF rt_times(const DF& x, int c) { return x * (float)c; }
+RT_HD __forceinline__ DF rt_plus_one(const DF& x) { return x + 1.0f; }
+
 // hi is the rounding of hi + lo to FP32
 RT_HD __forceinline__ float df_f(DF a) { return a.hi; }
 RT_HD __forceinline__ double df_d(DF a) { return (double)a.hi + (double)a.lo; }

@@ -75,6 +75,28 @@ RT_HD __forceinline__ Dual<N, T> operator/(const Dual<N, T>& a, const Dual<N, T>
   return r;
 }
 template <int N, class T>
+RT_HD __forceinline__ Dual<N, T> rt_twice(const Dual<N, T>& a) {
+  Dual<N, T> r;
+  r.v = rt_twice(a.v);
+#pragma unroll
+  for (int i = 0; i < N; ++i) r.d[i] = rt_twice(a.d[i]);
+  return r;
+}
+template <int N, class T>
+RT_HD __forceinline__ Dual<N, T> rt_times(const Dual<N, T>& a, int c) {
+  Dual<N, T> r;
+  r.v = rt_times(a.v, c);
+#pragma unroll
+  for (int i = 0; i < N; ++i) r.d[i] = rt_times(a.d[i], c);
+  return r;
+}
+template <int N, class T>
+RT_HD __forceinline__ Dual<N, T> rt_plus_one(const Dual<N, T>& a) {
+  Dual<N, T> r = a;
+  r.v = rt_plus_one(a.v);
+  return r;
+}
+template <int N, class T>
 RT_HD __forceinline__ Dual<N, T>& operator+=(Dual<N, T>& a, const Dual<N, T>& b) {
   a = a + b;
   return a;
@@ -115,7 +137,7 @@ RT_HD __forceinline__ Dual<N, T> rt_sqrt(const Dual<N, T>& a) {
 }
 template <int N, class T>
 RT_HD __forceinline__ Dual<N, T> rt_rsqrt(const Dual<N, T>& a) {
-  const T q = T(1) / rt_sqrt(a.v);
+  const T q = rt_rsqrt(a.v);
   return chain(a, q, T(-0.5) * q * q * q);
 }
 template <int N, class T>

@@ -71,7 +71,7 @@ extern "C" rt_status rt_flops_per_step(int32_t dispersion, int32_t plasma, doubl
   c.m0 = 0.3; c.m1 = 0.1; c.m2 = 0.9; c.sig = 1.0; c.disp = dispersion; c.plasma = plasma;
   g_t = Tally();
   Cnt d[6];
-  rtk::ham_rhs<Cnt>(c, Cnt(20.0), Cnt(3.0), Cnt(-5.0), Cnt(0.3), Cnt(-0.4), Cnt(0.8), d[0], d[1],
+  rtk::ham_rhs64<Cnt>(c, Cnt(20.0), Cnt(3.0), Cnt(-5.0), Cnt(0.3), Cnt(-0.4), Cnt(0.8), d[0], d[1],
                     d[2], d[3], d[4], d[5]);
   const double rhs = g_t.flops, rhs_special = g_t.special;
   // Stage inputs y + h * sum_j a_sj k_j for stages 2..6 with 1..5 nonzero
@@ -102,7 +102,7 @@ extern "C" rt_status rt_flops_per_step_df(int32_t dispersion, int32_t plasma, do
   c.m0 = 0.3; c.m1 = 0.1; c.m2 = 0.9; c.sig = 1.0; c.disp = dispersion; c.plasma = plasma;
   g_t = Tally();
   CntD d[6];
-  rtk::ham_rhs<CntD>(c, CntD(20.0), CntD(3.0), CntD(-5.0), CntD(0.3), CntD(-0.4), CntD(0.8), d[0],
+  rtk::ham_rhs64<CntD>(c, CntD(20.0), CntD(3.0), CntD(-5.0), CntD(0.3), CntD(-0.4), CntD(0.8), d[0],
                      d[1], d[2], d[3], d[4], d[5]);
   const double rhs = g_t.flops;
   // stage inputs y + h (sum_j a_sj k_j): nnz products and nnz - 1 sums of

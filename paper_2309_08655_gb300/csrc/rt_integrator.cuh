@@ -15,7 +15,45 @@ namespace {
 constexpr unsigned FULL = 0xffffffffu;
 
 __device__ __forceinline__ void rhs64(const RayConst<double>& c, const double* y, double* f) {
-  ham_rhs<double>(c, y[0], y[1], y[2], y[3], y[4], y[5], f[0], f[1], f[2], f[3], f[4], f[5]);
+  ham_rhs64<double>(c, y[0], y[1], y[2], y[3], y[4], y[5], f[0], f[1], f[2], f[3], f[4], f[5]);
+}
+
+// FP32 <-> FP64 by integer operations.  The conversion instructions issue on
+// the FP64 pipe at its rate (64 cycles a warp); these cost it nothing.
+// narrow(): toward zero; below 2^-126 zero, above FP32's range infinity, NaN
+// stays NaN.  widen(): exact for zero and normal values; infinity and NaN stay
+// what they are (a subnormal float becomes zero).
+__device__ __forceinline__ float narrow(double d) {
+  const int hi = __double2hiint(d), a = hi & 0x7fffffff;
+  int f = __funnelshift_l(__double2loint(d), a - 0x38000000, 3);
+  if (a < 0x38100000) f = 0;
+  if (a >= 0x47f00000) f = (a > 0x7ff00000 || (a == 0x7ff00000 && __double2loint(d))) ? 0x7fc00000
+                                                                                      : 0x7f800000;
+  return __int_as_float(f | (hi & 0x80000000));
+}
+__device__ __forceinline__ double widen(float v) {
+  const int b = __float_as_int(v), a = b & 0x7fffffff;
+  int hi = (a >> 3) + 0x38000000;
+  if (a < 0x00800000) hi = 0;
+  if (a >= 0x7f800000) hi = 0x7ff00000 | (a > 0x7f800000 ? 0x80000 : 0);
+  return __hiloint2double(hi | (b & 0x80000000),
+                          (a < 0x00800000 || a >= 0x7f800000) ? 0 : (a << 29));
+}
+// the larger magnitude, compared as integers (a comparison of doubles is an
+// FP64-pipe instruction)
+__device__ __forceinline__ double max_abs(double a, double b) {
+  const long long x = __double_as_longlong(a) & 0x7fffffffffffffffll;
+  const long long y = __double_as_longlong(b) & 0x7fffffffffffffffll;
+  return __longlong_as_double(x > y ? x : y);
+}
+// 1/x to rounding for normal x: the hardware's coarse reciprocal r (about 2^-20
+// off) corrected by the geometric series in the residual d = 1 - x r,
+// r (1 + d + d^2); the rest is d^3 ~ 2^-60.
+__device__ __forceinline__ double recip_series(double x) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  const double d = fma(-x, r, 1.0);
+  return fma(r, fma(d, d, d), r);
 }
 
 // err^(-1/5) to within an ulp or two: a single-precision estimate refined by
@@ -37,6 +75,29 @@ __device__ __forceinline__ double step_factor(double err, bool accepted, bool la
   double fac = (err > 1e6) ? 0.0 : (err >= 1e-6) ? 0.9 * pow_m1_5(err) : 5.0;
   fac = fmin(5.0, fmax(0.2, fac));
   if (!accepted || last_rej) fac = fmin(fac, 1.0);
+  return fac;
+}
+
+// step_factor() of err = sqrt(q), without the root: err^(-1/5) = q^(-1/10), a
+// single-precision estimate y corrected by the series of (1 - r)^(-1/10) in the
+// residual r = 1 - q y^10 (at most ~1e-5), y (1 + r/10 + 11 r^2/200).  The clamp
+// to [0.2, 5] is decided on the high words (positive numbers order like their
+// bits).
+__device__ __forceinline__ double step_factor_sq(double q, bool accepted, bool last_rej) {
+  const int hq = __double2hiint(q);
+  double fac = 5.0;
+  if (hq >= 0x426d1a94) {                         // q > 1e12
+    fac = 0.2;
+  } else if (hq >= 0x3d719799) {                  // q > 1e-12
+    const double y = widen(exp2f(-0.1f * log2f(narrow(q))));
+    const double y2 = y * y, y4 = y2 * y2;
+    const double r = fma(-q, (y4 * y) * (y4 * y), 1.0);
+    fac = 0.9 * fma(y, r * fma(0.055, r, 0.1), y);
+    const int hf = __double2hiint(fac);
+    if (hf >= 0x40140000) fac = 5.0;
+    if (__double_as_longlong(fac) < __double_as_longlong(0.2)) fac = 0.2;
+  }
+  if ((!accepted || last_rej) && __double2hiint(fac) >= 0x3ff00000) fac = 1.0;
   return fac;
 }
 
@@ -203,49 +264,43 @@ __device__ __forceinline__ void illinois(const S& side, T& lo, T& hi, T& flo, T&
   }
 }
 
-// Event location on the continuous extension: the last th in [0, 1] on the
-// non-negative side of a function given in FP64 (f64) and, to FP32 rounding,
-// by a cheap FP32 model (f32), with f64(0) = flo >= 0 > fhi = f64(1).  The FP32
-// model's root (plain Illinois to 2^-22 relative) is widened by SEED_WIDEN on
-// each side; FP64 values at the two ends confirm that the root lies inside
-// (else the part of [0, 1] left or right of it holds one), and FP64 Illinois
-// narrows that bracket to SEED_TOL64 relative, far below the 1e-10 relative
-// overshoot of a switch and below the rounding of an escape point.  About six
-// FP64 evaluations where bisection-guarded Illinois from [0, 1] to the last
-// bit takes twenty or more.  Returns lo; *hi_out the end past it.
+// Event location on the continuous extension: the root th in [0, 1] of a
+// function given in FP64 (f64) and, to FP32 rounding, by a cheap FP32 model
+// (f32), with f64(0) = flo >= 0 > fhi = f64(1).  The FP32 model's root (plain
+// Illinois to 2^-22 relative) is widened by SEED_WIDEN on each side; where FP64
+// values at the two ends confirm it, the secant through them is off by
+// ~SEED_WIDEN^2 times the relative curvature, and one more secant step from an
+// FP64 value there leaves only rounding.  Otherwise (a grazing crossing, or
+// rounding of the model) last_nonneg from [0, 1].
+//
+// On this GPU a search runs at one or two live lanes of its warp while every
+// FP64 instruction costs the same 64 cycles: three FP64 evaluations and two
+// divisions, against fifteen or more evaluations, each with a division, of the
+// guarded Illinois from [0, 1].  The FP32 part costs the FP64 pipe nothing (the
+// model is built with narrow()).
 constexpr float SEED_TOL32 = 0x1p-22f;
-constexpr double SEED_WIDEN = 0x1p-16;
-constexpr double SEED_TOL64 = 0x1p-44;
+constexpr float SEED_WIDEN = 0x1p-19f;
 template <class S64, class S32>
-__device__ __forceinline__ double last_nonneg_seeded(const S64& f64, const S32& f32, double flo,
-                                                     double fhi, double* hi_out) {
-  float l = 0.0f, u = 1.0f, fl = (float)flo, fu = (float)fhi;
+__device__ __forceinline__ double event_root(const S64& f64, const S32& f32, double flo,
+                                             double fhi) {
+  float l = 0.0f, u = 1.0f, fl = narrow(flo), fu = narrow(fhi);
   if (!(fl >= 0.0f)) fl = 0.0f;
   if (!(fu < 0.0f)) fu = -1e-30f;
   illinois(f32, l, u, fl, fu, SEED_TOL32, 40);
-  double lo = 0.0, hi = 1.0;
-  const double a = fmax(0.0, (double)l - SEED_WIDEN), b = fmin(1.0, (double)u + SEED_WIDEN);
-  const double fa = (a > 0.0) ? f64(a) : flo;
-  if (fa < 0.0) {
-    hi = a;                                        // the root lies left of the FP32 bracket
-    fhi = fa;
-  } else {
-    lo = a;
-    flo = fa;
-    const double fb = (b < 1.0) ? f64(b) : fhi;
-    if (fb >= 0.0) {
-      lo = b;                                      // right of it
-      flo = fb;
-    } else {
-      hi = b;
-      fhi = fb;
-    }
+  const double a = widen(fmaxf(0.0f, l - SEED_WIDEN)), b = widen(fminf(1.0f, u + SEED_WIDEN));
+  const double fa = f64(a), fb = f64(b);
+  if (fa >= 0.0 && fb < 0.0) {
+    const double slope = (b - a) * recip_series(fa - fb);      // -1 / f'
+    double th = fma(fa, slope, a);
+    th = fma(f64(th), slope, th);
+    if (th >= a && th <= b) return th;
   }
-  illinois(f64, lo, hi, flo, fhi, SEED_TOL64, 40);
-  if (hi - lo > SEED_TOL64 * hi) return last_nonneg(f64, flo, fhi, hi_out, lo, hi);
-  *hi_out = hi;
-  return lo;
+  double hi;
+  return last_nonneg(f64, flo, fhi, &hi);
 }
+
+__device__ __forceinline__ float to_f32(float v) { return v; }
+__device__ __forceinline__ float to_f32(double v) { return narrow(v); }
 
 // FP32 model of the null-cone side function sig F(x(th)), F = 3 z (m.x) -
 // m_z |x|^2, along the continuous extension x(th) = y + d(th), d(th) =
@@ -263,17 +318,17 @@ struct ConeModel32 {
     m0 = cm0;
     m1 = cm1;
     m2 = cm2;
-    const float y0 = (float)y[0], y1 = (float)y[1], y2 = (float)y[2];
+    const float y0 = to_f32(y[0]), y1 = to_f32(y[1]), y2 = to_f32(y[2]);
     const float mx = m0 * y0 + m1 * y1 + m2 * y2;
     gF[0] = 3.0f * y2 * m0 - 2.0f * m2 * y0;
     gF[1] = 3.0f * y2 * m1 - 2.0f * m2 * y1;
     gF[2] = 3.0f * mx + 3.0f * y2 * m2 - 2.0f * m2 * y2;
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-      r2[i] = (float)R2[i];
-      r3[i] = (float)R3[i];
-      r4[i] = (float)R4[i];
-      r5[i] = (float)R5[i];
+      r2[i] = to_f32(R2[i]);
+      r3[i] = to_f32(R3[i]);
+      r4[i] = to_f32(R4[i]);
+      r5[i] = to_f32(R5[i]);
     }
   }
   __device__ __forceinline__ float operator()(float th) const {
@@ -297,11 +352,11 @@ struct EscapeModel32 {
     c0 = c0f;
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-      y[i] = (float)yd[i];
-      r2[i] = (float)R2[i];
-      r3[i] = (float)R3[i];
-      r4[i] = (float)R4[i];
-      r5[i] = (float)R5[i];
+      y[i] = to_f32(yd[i]);
+      r2[i] = to_f32(R2[i]);
+      r3[i] = to_f32(R3[i]);
+      r4[i] = to_f32(R4[i]);
+      r5[i] = to_f32(R5[i]);
     }
   }
   __device__ __forceinline__ float operator()(float th) const {
@@ -363,21 +418,23 @@ __device__ int advance(const TraceParams& p, Lane& L, Hook& hook) {
   for (int i = 0; i < 6; ++i) {
     const double e = h * (DP::e1 * k1[i] + DP::e3 * k3[i] + DP::e4 * k4[i] + DP::e5 * k5[i] +
                           DP::e6 * k6[i] + DP::e7 * k7[i]);
-    const double sc = p.atol + p.rtol * fmax(fabs(y[i]), fabs(yn[i]));
-    s += (e / sc) * (e / sc);
+    const double q = e * recip_series(p.atol + p.rtol * max_abs(y[i], yn[i]));
+    s += q * q;
   }
-  const double en = sqrt(s / 6.0);
-  if (!isfinite(en)) {
+  // the squared error norm; <= 1 accepts
+  const double en2 = s * (1.0 / 6.0);
+  if ((__double2hiint(en2) & 0x7ff00000) == 0x7ff00000) {   // infinite or NaN
     ++L.nr;
     L.h = h * 0.2;
     L.last_rej = true;
     return (L.h < 1e-12) ? RAY_NAN : -1;
   }
+  const bool ok = en2 <= 1.0;
   const bool gj = (L.c.plasma == PLASMA_GJ);
-  if (en <= 1.0 && gj && !L.switching &&
+  if (ok && gj && !L.switching &&
       L.c.sig * gj_side<double>(L.c.m0, L.c.m1, L.c.m2, yn[0], yn[1], yn[2]) < 0.0) {
-    // the step crossed the null cone: largest th with the start side on the
-    // continuous extension (bisection), then redo the step to end just past it
+    // the step crossed the null cone: the crossing on the continuous extension,
+    // then redo the step to end just past it
     double r3[3], r4[3], r5[3], r2[3];
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
@@ -387,10 +444,7 @@ __device__ int advance(const TraceParams& p, Lane& L, Hook& hook) {
       r5[i] = h * (DP::d1 * k1[i] + DP::d3 * k3[i] + DP::d4 * k4[i] + DP::d5 * k5[i] +
                    DP::d6 * k6[i] + DP::d7 * k7[i]);
     }
-    // largest th with the start side on the continuous extension: Illinois
-    // (regula falsi with halving) on s(th) = sig (3 z (m.x) - m_z |x|^2), whose
-    // sign is the side, bracketed on [0, 1]; a bisection step whenever the
-    // bracket did not halve, to the last representable th
+    // s(th) = sig (3 z (m.x) - m_z |x|^2), whose sign is the side
     const double sgn = L.c.sig;
     auto side_val = [&](double th) {
       double xd[3];
@@ -402,10 +456,12 @@ __device__ int advance(const TraceParams& p, Lane& L, Hook& hook) {
       return sgn * (3.0 * xd[2] * mx - L.c.m2 * rr);
     };
     double flo = side_val(0.0), fhi = side_val(1.0);
+    ConeModel32 m32;
+    m32.init(narrow(sgn), narrow(sgn * flo), narrow(L.c.m0), narrow(L.c.m1), narrow(L.c.m2), y, r2,
+             r3, r4, r5);
     if (!(flo >= 0.0)) flo = 0.0;                  // the start is on its own side
     if (!(fhi < 0.0)) fhi = -1e-300;
-    double hi;
-    const double lo = last_nonneg(side_val, flo, fhi, &hi);
+    const double lo = event_root(side_val, m32, flo, fhi);
     ++L.nr;
     if (lo < SWITCH_MIN_FRACTION) {
       L.c.sig = -L.c.sig;             // already at the cone: switch here
@@ -418,7 +474,7 @@ __device__ int advance(const TraceParams& p, Lane& L, Hook& hook) {
     }
     return -1;
   }
-  if (en <= 1.0) {
+  if (ok) {
     ++L.na;
     hook.on_accept(L, y, yn, k1, k2, k3, k4, k5, k6, k7, h);
     const double rnew2 = yn[0] * yn[0] + yn[1] * yn[1] + yn[2] * yn[2];
@@ -434,8 +490,7 @@ __device__ int advance(const TraceParams& p, Lane& L, Hook& hook) {
                      DP::d6 * k6[i] + DP::d7 * k7[i]);
         t[i] = r2;
       }
-      // r_out^2 - |x(th)|^2 changes sign on [0, 1]: Illinois to the last
-      // representable th (the root to rounding, in ~10 evaluations)
+      // r_out^2 - |x(th)|^2 changes sign on [0, 1]
       const double ro2 = p.r_out * p.r_out;
       auto inside = [&](double th) {
         double xd[3];
@@ -448,9 +503,9 @@ __device__ int advance(const TraceParams& p, Lane& L, Hook& hook) {
       if (!(flo >= 0.0)) flo = 0.0;
       double fhi = ro2 - rnew2;
       if (!(fhi < 0.0)) fhi = -1e-300;
-      double hi;
-      const double lo = last_nonneg(inside, flo, fhi, &hi);
-      const double th = 0.5 * (lo + hi);
+      EscapeModel32 e32;
+      e32.init(narrow(flo), y, t, r3, r4, r5);
+      const double th = event_root(inside, e32, flo, fhi);
 #pragma unroll
       for (int i = 0; i < 6; ++i)
         yn[i] = y[i] + th * (t[i] + (1.0 - th) * (r3[i] + th * (r4[i] + (1.0 - th) * r5[i])));
@@ -475,13 +530,13 @@ __device__ int advance(const TraceParams& p, Lane& L, Hook& hook) {
       L.h = L.h_resume;
       L.switching = false;
     } else {
-      L.h = h * step_factor(en, true, L.last_rej);
+      L.h = h * step_factor_sq(en2, true, L.last_rej);
     }
     L.last_rej = false;
     return -1;
   }
   ++L.nr;
-  L.h = h * step_factor(en, false, L.last_rej);
+  L.h = h * step_factor_sq(en2, false, L.last_rej);
   L.last_rej = true;
   return (L.h < 1e-12) ? RAY_STIFF : -1;
 }

@@ -1,6 +1,6 @@
 // Hamilton's equations at given phase-space points: the right-hand side that
-// the FP64 integrators step with (rhs64 of rt_integrator.cuh, i.e. ham_rhs of
-// rt_device.cuh), exposed so that it can be checked point by point.
+// the FP64 integrators step with (rhs64 of rt_integrator.cuh, i.e. ham_rhs64
+// of rt_device.cuh), exposed so that it can be checked point by point.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
