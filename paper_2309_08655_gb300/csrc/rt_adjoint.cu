@@ -31,6 +31,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "rt_df.cuh"
 #include "rt_dual.cuh"
 #include "rt_integrator.cuh"
@@ -110,7 +112,7 @@ struct AdjParams {
 // Right-hand side in the sweep's precision T.
 template <class T>
 __device__ __forceinline__ void rhs_t(const RayConst<T>& c, const T* y, T* f) {
-  ham_rhs<T>(c, y[0], y[1], y[2], y[3], y[4], y[5], f[0], f[1], f[2], f[3], f[4], f[5]);
+  ham_rhs64<T>(c, y[0], y[1], y[2], y[3], y[4], y[5], f[0], f[1], f[2], f[3], f[4], f[5]);
 }
 
 // The ray's constants in the sweep's precision.
@@ -137,28 +139,15 @@ __device__ __forceinline__ RayConst<T> cast_const(const RayConst<double>& c) {
 constexpr int NQ = 3;
 enum { Q_RS = 0, Q_CP, Q_THM };
 
-// J^T v and v . df/dq at y, from one dual evaluation in the scalar type T
-// with 1 + NQ tangents: the direction Omega v, and q (m along dm).
+// J^T v and v . df/dq at y, from one dual evaluation in the scalar type T with
+// one tangent, the direction u = Omega v = (v_k, -v_x).  With f = (dH/dk,
+// -dH/dx), v . f = -u . grad H, so J^T v = Omega (J u) and v . df/dq = -u . grad
+// (dH/dq): the tangents of the right-hand side and of the three scalars dH/dq.
+// A product costs 3 operations of T, against 9 with a tangent for each q.
 template <class T>
 __device__ __noinline__ void rhs_vjp(const RayConst<T>& c, const T* dm, const T* y, const T* v,
                                      T* out, T* qbar) {
-  typedef Dual<1 + NQ, T> DT;
-  RayConst<DT> cd;
-  cd.rs = DT::var(c.rs, 1 + Q_RS);
-  cd.cp = DT::var(c.cp, 1 + Q_CP);
-  cd.pa = DT(c.pa);
-  cd.W2 = DT(c.W2);
-  cd.iW2 = DT(c.iW2);
-  cd.m0 = DT(c.m0);
-  cd.m1 = DT(c.m1);
-  cd.m2 = DT(c.m2);
-  cd.m0.d[1 + Q_THM] = dm[0];
-  cd.m1.d[1 + Q_THM] = dm[1];
-  cd.m2.d[1 + Q_THM] = dm[2];
-  cd.sig = DT(c.sig);
-  cd.disp = c.disp;
-  cd.plasma = c.plasma;
-  // u = Omega v = (v_k, -v_x)
+  typedef Dual<1, T> DT;
   DT yd[6];
 #pragma unroll
   for (int j = 0; j < 3; ++j) {
@@ -168,20 +157,21 @@ __device__ __noinline__ void rhs_vjp(const RayConst<T>& c, const T* dm, const T*
     yd[3 + j].d[0] = -v[j];
   }
   DT f[6];
-  ham_rhs<DT>(cd, yd[0], yd[1], yd[2], yd[3], yd[4], yd[5], f[0], f[1], f[2], f[3], f[4], f[5]);
+  ConstGrad<DT, T> cg;
+  cg.dm0 = dm[0];
+  cg.dm1 = dm[1];
+  cg.dm2 = dm[2];
+  ham_rhs64<DT, false, true, T>(c, yd[0], yd[1], yd[2], yd[3], yd[4], yd[5], f[0], f[1], f[2],
+                                f[3], f[4], f[5], nullptr, &cg);
   // J^T v = Omega (J u) = ((Ju)_k, -(Ju)_x)
 #pragma unroll
   for (int j = 0; j < 3; ++j) {
     out[j] = f[3 + j].d[0];
     out[3 + j] = -f[j].d[0];
   }
-#pragma unroll
-  for (int m = 1; m <= NQ; ++m) {
-    T s = T(0);
-#pragma unroll
-    for (int j = 0; j < 6; ++j) s += v[j] * f[j].d[m];
-    qbar[m - 1] += s;
-  }
+  qbar[Q_RS] -= cg.rs.d[0];
+  qbar[Q_CP] -= cg.cp.d[0];
+  qbar[Q_THM] -= cg.m.d[0];
 }
 
 // Dual number of the mixed sweep: the value and the state-direction tangent in
@@ -398,20 +388,31 @@ __device__ void step_adjoint(const RayConst<T>& c, const T* dm, const T* y, T h,
       r5[i] = h * (d1 * K[0][i] + d3 * K[2][i] + d4 * K[3][i] + d5 * K[4][i] + d6 * K[5][i] +
                    d7 * K[6][i]);
     }
-    // the same bisection as the forward step
-    T lo = T(0), hi = T(1);
-    for (int it = 0; it < 200; ++it) {
-      const T mid = T(0.5) * (lo + hi);
-      if (mid <= lo || mid >= hi) break;
+    // the escape point of the forward step
+    auto inside = [&](T at) {
       T xd[3];
 #pragma unroll
       for (int i = 0; i < 3; ++i)
-        xd[i] = y[i] + mid * (r2v[i] + (T(1) - mid) * (r3[i] + mid * (r4[i] + (T(1) - mid) *
-                                                                             r5[i])));
-      const T rd2 = xd[0] * xd[0] + xd[1] * xd[1] + xd[2] * xd[2];
-      if (rd2 < r_out * r_out) lo = mid; else hi = mid;
+        xd[i] = y[i] + at * (r2v[i] + (T(1) - at) * (r3[i] + at * (r4[i] + (T(1) - at) * r5[i])));
+      return r_out * r_out - (xd[0] * xd[0] + xd[1] * xd[1] + xd[2] * xd[2]);
+    };
+    T th;
+    if constexpr (std::is_same<T, double>::value) {
+      double flo = inside(0.0), fhi = inside(1.0);
+      if (!(flo >= 0.0)) flo = 0.0;
+      if (!(fhi < 0.0)) fhi = -1e-300;
+      EscapeModel32 e32;
+      e32.init(narrow(flo), y, r2v, r3, r4, r5);
+      th = event_root(inside, e32, flo, fhi);
+    } else {
+      T lo = T(0), hi = T(1);
+      for (int it = 0; it < 200; ++it) {
+        const T mid = T(0.5) * (lo + hi);
+        if (mid <= lo || mid >= hi) break;
+        if (inside(mid) > T(0)) lo = mid; else hi = mid;
+      }
+      th = T(0.5) * (lo + hi);
     }
-    const T th = T(0.5) * (lo + hi);
     const T al = th, be = th * (T(1) - th), ga = th * th * (T(1) - th),
             de = th * th * (T(1) - th) * (T(1) - th);
     const T dal = T(1), dbe = T(1) - T(2) * th, dga = T(2) * th - T(3) * th * th,

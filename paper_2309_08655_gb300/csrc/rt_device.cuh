@@ -242,11 +242,11 @@ template <class T>
 RT_HD __forceinline__ T rt_plus_one(const T& x) { return T(1) + x; }
 
 // The Hamiltonian's derivatives with respect to the constants that a star's
-// parameters move: cp dH/dcp, dH/drs, and dH/dm . dm for a given turn dm of the
+// parameters move: dH/dcp, dH/drs, and dH/dm . dm for a given turn dm of the
 // magnetic axis.
-template <class T>
+template <class T, class C = T>
 struct ConstGrad {
-  T dm0, dm1, dm2;   // in
+  C dm0, dm1, dm2;   // in
   T cp, rs, m;       // out
 };
 
@@ -268,11 +268,12 @@ struct ConstGrad {
 // ham_rhs.  CG: *cg = the derivatives with respect to the star's constants
 // (with dual numbers in the direction u, their tangents are u . grad_y of them:
 // the parameter part of a Jacobian product without a tangent per parameter).
-template <class T, bool DW = false, bool CG = false>
-RT_HD __forceinline__ void ham_rhs64(const RayConst<T>& c, const T x0, const T x1, const T x2,
+// C: the type of the ray's constants (T, or the plain scalar under a dual T).
+template <class T, bool DW = false, bool CG = false, class C = T>
+RT_HD __forceinline__ void ham_rhs64(const RayConst<C>& c, const T x0, const T x1, const T x2,
                                      const T k0, const T k1, const T k2, T& dx0, T& dx1, T& dx2,
                                      T& dk0, T& dk1, T& dk2, T* dw = nullptr,
-                                     ConstGrad<T>* cg = nullptr) {
+                                     ConstGrad<T, C>* cg = nullptr) {
   const T r2 = x0 * x0 + x1 * x1 + x2 * x2;
   const T ir = rt_rsqrt(r2);
   const T n0 = x0 * ir, n1 = x1 * ir, n2 = x2 * ir;
@@ -286,7 +287,7 @@ RT_HD __forceinline__ void ham_rhs64(const RayConst<T>& c, const T x0, const T x
   const T mu3 = rt_times(mu, 3);
   // P and dP = t (qn n + qm m + qz e_z)
   T P = T(0), t = T(0), qn = T(0), qm = T(0), qz = T(0);
-  T dPdm = T(0);                                 // dP/dm . dm (CG)
+  T dPdm = T(0), Pc = T(0);                      // dP/dm . dm and dP/dcp (CG)
   if (c.plasma == PLASMA_GJ) {
     const T g3 = c.cp * c.sig * (ir2 * ir);
     const T mn = mu * n2;
@@ -296,15 +297,21 @@ RT_HD __forceinline__ void ham_rhs64(const RayConst<T>& c, const T x0, const T x
     qn = rt_times(c.m2, 3) - rt_times(mn, 15);
     qm = rt_times(n2, 3);
     qz = mu3;
-    if (CG) dPdm = g3 * (qm * (n0 * cg->dm0 + n1 * cg->dm1 + n2 * cg->dm2) - cg->dm2);
+    if (CG) {
+      Pc = (c.sig * (ir2 * ir)) * F;
+      dPdm = g3 * (qm * (n0 * cg->dm0 + n1 * cg->dm1 + n2 * cg->dm2) - cg->dm2);
+    }
   } else if (c.plasma == PLASMA_TWISTED) {
     const T g4 = c.cp * (ir2 * ir2);
     const T mm = mu * mu;
     P = g4 * rt_plus_one(-mm);
     t = rt_twice(g4 * ir);
-    qn = rt_times(mm, 3) - T(2);
+    qn = rt_times(mm, 3) - C(2);
     qm = -mu;
-    if (CG) dPdm = -rt_twice(g4 * mu) * (n0 * cg->dm0 + n1 * cg->dm1 + n2 * cg->dm2);
+    if (CG) {
+      Pc = (ir2 * ir2) * rt_plus_one(-mm);
+      dPdm = -(rt_twice(g4 * mu) * (n0 * cg->dm0 + n1 * cg->dm1 + n2 * cg->dm2));
+    }
   } else if (c.plasma == PLASMA_RADIAL) {
     P = c.pa * (ir2 * ir);
     t = P * ir;
@@ -331,7 +338,7 @@ RT_HD __forceinline__ void ham_rhs64(const RayConst<T>& c, const T x0, const T x
     dk2 = -(Cn * n2 + Ck * k2 + Cm * c.m2 + t * qz);
     if (DW) *dw = -iA;
     if (CG) {
-      cg->cp = (c.plasma == PLASMA_GJ || c.plasma == PLASMA_TWISTED) ? P : T(0);
+      cg->cp = Pc;
       cg->rs = -(ir * (c.W2 * iA2 + kr * kr));   // dA/drs = -1/r
       cg->m = dPdm;
     }
@@ -367,7 +374,7 @@ RT_HD __forceinline__ void ham_rhs64(const RayConst<T>& c, const T x0, const T x
   dk2 = -(Cn * n2 + Ck * k2 + Cm * c.m2 + w * qz);
   if (DW) *dw = (P * A) * (Kq * c.iW2) - iA;
   if (CG) {
-    cg->cp = (c.plasma == PLASMA_GJ || c.plasma == PLASMA_TWISTED) ? P * one_m : T(0);
+    cg->cp = Pc * one_m;
     // dH/dA = W2/A^2 + kr^2 - P Kq - (P A 2 Kp/W2) dKp/dA, dKp/dA = mu kr / (sqrt(A) |b|)
     cg->rs = -(ir * ((c.W2 * iA2 + kr * kr) - P * Kq - gm * ((mu * kr) * qA)));
     // U = k.b + ..: dU/dm . dm = opsA kr dmu - k.dm, d|b|^2 = 6 mu dmu

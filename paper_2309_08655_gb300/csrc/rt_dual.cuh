@@ -74,6 +74,31 @@ RT_HD __forceinline__ Dual<N, T> operator/(const Dual<N, T>& a, const Dual<N, T>
   for (int i = 0; i < N; ++i) r.d[i] = (a.d[i] - r.v * b.d[i]) * ib;
   return r;
 }
+// with a plain scalar: no arithmetic on tangents that are zero
+template <int N, class T>
+RT_HD __forceinline__ Dual<N, T> operator*(const Dual<N, T>& a, const T& b) {
+  Dual<N, T> r;
+  r.v = a.v * b;
+#pragma unroll
+  for (int i = 0; i < N; ++i) r.d[i] = a.d[i] * b;
+  return r;
+}
+template <int N, class T>
+RT_HD __forceinline__ Dual<N, T> operator*(const T& a, const Dual<N, T>& b) {
+  return b * a;
+}
+template <int N, class T>
+RT_HD __forceinline__ Dual<N, T> operator-(const Dual<N, T>& a, const T& b) {
+  Dual<N, T> r = a;
+  r.v = a.v - b;
+  return r;
+}
+template <int N, class T>
+RT_HD __forceinline__ Dual<N, T> operator-(const T& a, const Dual<N, T>& b) {
+  Dual<N, T> r = -b;
+  r.v = a - b.v;
+  return r;
+}
 template <int N, class T>
 RT_HD __forceinline__ Dual<N, T> rt_twice(const Dual<N, T>& a) {
   Dual<N, T> r;

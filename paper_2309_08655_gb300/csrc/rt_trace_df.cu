@@ -1,5 +1,5 @@
 // Forward tracing in double-float (RT_PREC_DF): the FP64 integrator of
-// rt_integrator.cuh -- the same Hamiltonian right-hand side (ham_rhs,
+// rt_integrator.cuh -- the same Hamiltonian right-hand side (ham_rhs64,
 // instantiated on the double-float scalar of rt_df.cuh), the same
 // Dormand-Prince 5(4) step with its embedded error estimate, step-size
 // controller, step reach, Goldreich-Julian null-cone switch and escape
@@ -66,13 +66,13 @@ __constant__ DF c_E[7] = {DPD::e1, DF(0), DPD::e3, DPD::e4, DPD::e5, DPD::e6, DP
 // The Goldreich-Julian anisotropic medium (the benchmark's) has a copy with
 // the model switches fixed, free of the other media's branches.
 __device__ __noinline__ void rhs_df_any(const RayConst<DF>& c, const DF* y, DF* f) {
-  ham_rhs<DF>(c, y[0], y[1], y[2], y[3], y[4], y[5], f[0], f[1], f[2], f[3], f[4], f[5]);
+  ham_rhs64<DF>(c, y[0], y[1], y[2], y[3], y[4], y[5], f[0], f[1], f[2], f[3], f[4], f[5]);
 }
 __device__ __noinline__ void rhs_df_gj_aniso(const RayConst<DF>& c0, const DF* y, DF* f) {
   RayConst<DF> c = c0;
   c.plasma = PLASMA_GJ;
   c.disp = DISP_ANISO;
-  ham_rhs<DF>(c, y[0], y[1], y[2], y[3], y[4], y[5], f[0], f[1], f[2], f[3], f[4], f[5]);
+  ham_rhs64<DF>(c, y[0], y[1], y[2], y[3], y[4], y[5], f[0], f[1], f[2], f[3], f[4], f[5]);
 }
 __device__ __forceinline__ void rhs_df(const RayConst<DF>& c, const DF* y, DF* f) {
   if (c.plasma == PLASMA_GJ && c.disp == DISP_ANISO)

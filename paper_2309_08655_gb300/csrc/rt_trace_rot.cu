@@ -5,7 +5,7 @@
 // equations (Eq. Hamilton) carry all four canonical pairs.  State of a ray
 // (units of R and m_a): y = (x, k, t, omega) with omega = -k_t, and
 //
-//   dx/dl, dk/dl   ham_rhs with the axis m(psi0 + Omega t) and W2 = omega^2
+//   dx/dl, dk/dl   ham_rhs64 with the axis m(psi0 + Omega t) and W2 = omega^2
 //   dt/dl        = dH/dk_t = -2 omega dH/dW2
 //   domega/dl    = dH/dt   = -Omega [(x x dH/dx)_z + (k x dH/dk)_z]
 //
@@ -49,8 +49,8 @@ __device__ __forceinline__ void rhs_rot(RotLane& L, const double* y, double* f) 
   L.c.W2 = y[7] * y[7];
   L.c.iW2 = 1.0 / L.c.W2;
   double dw;
-  ham_rhs<double, false, false, true>(L.c, y[0], y[1], y[2], y[3], y[4], y[5], f[0], f[1], f[2],
-                                      f[3], f[4], f[5], 0.0, &dw);
+  ham_rhs64<double, true>(L.c, y[0], y[1], y[2], y[3], y[4], y[5], f[0], f[1], f[2], f[3], f[4],
+                          f[5], &dw);
   f[6] = -2.0 * y[7] * dw;
   // dH/dx = -(f3, f4, f5), dH/dk = (f0, f1, f2)
   f[7] = L.Om * (y[0] * f[4] - y[1] * f[3] - y[3] * f[1] + y[4] * f[0]);
