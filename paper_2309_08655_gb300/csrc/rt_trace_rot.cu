@@ -47,7 +47,7 @@ __device__ __forceinline__ void rhs_rot(RotLane& L, const double* y, double* f) 
   L.c.m0 = L.sin_tm * cp;
   L.c.m1 = L.sin_tm * sp;
   L.c.W2 = y[7] * y[7];
-  L.c.iW2 = 1.0 / L.c.W2;
+  L.c.iW2 = recip_series(L.c.W2);
   double dw;
   ham_rhs64<double, true>(L.c, y[0], y[1], y[2], y[3], y[4], y[5], f[0], f[1], f[2], f[3], f[4],
                           f[5], &dw);
@@ -154,6 +154,25 @@ __device__ void store_rot(const TraceParams& p, int64_t i, const RotLane& L, int
   if (p.nrej) p.nrej[i] = L.nr;
 }
 
+// FP32 model of the turning cone's side function along a step: that of the axis
+// at the step's start (ConeModel32) plus the axis's turn by a(th) = Omega (t(th)
+// - t_start), 3 z (dm . x), dm = m(a) - m(0) to third order.
+struct TurningConeModel32 {
+  ConeModel32 cone;
+  float y[3], a2, a3, a4, a5;
+  __device__ __forceinline__ float operator()(float th) const {
+    const float u = 1.0f - th;
+    float x[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+      x[i] = y[i] + th * (cone.r2[i] + u * (cone.r3[i] + th * (cone.r4[i] + u * cone.r5[i])));
+    const float a = th * (a2 + u * (a3 + th * (a4 + u * a5)));
+    const float s = a * (1.0f - a * a * (1.0f / 6.0f)), v = -0.5f * a * a;
+    const float dm0 = v * cone.m0 - s * cone.m1, dm1 = v * cone.m1 + s * cone.m0;
+    return cone(th) + cone.sg * 3.0f * x[2] * (dm0 * x[0] + dm1 * x[1]);
+  }
+};
+
 // One attempted step; returns -1 to continue, else the final ray status.
 __device__ int advance_rot(const TraceParams& p, RotLane& L) {
   if (L.na >= p.max_steps || L.na + L.nr >= 4 * p.max_steps) return RAY_MAXSTEPS;
@@ -200,27 +219,32 @@ __device__ int advance_rot(const TraceParams& p, RotLane& L) {
   for (int i = 0; i < 6; ++i) {
     const double e = h * (DP::e1 * k1[i] + DP::e3 * k3[i] + DP::e4 * k4[i] + DP::e5 * k5[i] +
                           DP::e6 * k6[i] + DP::e7 * k7[i]);
-    const double sc = p.atol + p.rtol * fmax(fabs(y[i]), fabs(yn[i]));
-    s += (e / sc) * (e / sc);
+    const double q = e * recip_series(p.atol + p.rtol * max_abs(y[i], yn[i]));
+    s += q * q;
   }
-  const double en = sqrt(s / 6.0);
-  if (!isfinite(en)) {
+  // the squared error norm; <= 1 accepts
+  const double en2 = s * (1.0 / 6.0);
+  if ((__double2hiint(en2) & 0x7ff00000) == 0x7ff00000) {   // infinite or NaN
     ++L.nr;
     L.h = h * 0.2;
     L.last_rej = true;
     return (L.h < 1e-12) ? RAY_NAN : -1;
   }
+  const bool ok = en2 <= 1.0;
   // continuous extension of the step: y(th) = y + th (r2 + (1-th)(r3 + th(r4 + (1-th) r5)))
   auto dense = [&](double th, double* out, double* r2, double* r3, double* r4, double* r5,
                    int nc) {
     for (int i = 0; i < nc; ++i)
       out[i] = y[i] + th * (r2[i] + (1.0 - th) * (r3[i] + th * (r4[i] + (1.0 - th) * r5[i])));
   };
-  const bool gj = (L.c.plasma == PLASMA_GJ);
-  if (en <= 1.0 && gj && !L.switching && L.c.sig * side_at(L, yn) < 0.0) {
-    // the step crossed the turning null cone: the largest th whose point (x,
-    // at its own t) is on the start side, by Illinois on the continuous
-    // extension; then redo the step to end just past it
+  // the side of the turning cone at (x, t) of yn: the last evaluation was there
+  // and left the axis at that time in L.c
+  const bool across =
+      ok && L.c.plasma == PLASMA_GJ &&
+      L.c.sig * gj_side<double>(L.c.m0, L.c.m1, L.c.m2, yn[0], yn[1], yn[2]) < 0.0;
+  if (across && !L.switching) {
+    // the step crossed the turning null cone: the crossing (x at its own t) on
+    // the continuous extension; then redo the step to end just past it
     double r2[8], r3[8], r4[8], r5[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
@@ -242,10 +266,20 @@ __device__ int advance_rot(const TraceParams& p, RotLane& L) {
       return sgn * (3.0 * yd[2] * mx - m2 * rr);
     };
     double flo = side_val(0.0), fhi = side_val(1.0);
+    double sp, cp;
+    sincos(L.psi0 + L.Om * y[6], &sp, &cp);
+    TurningConeModel32 m32;
+    m32.cone.init(narrow(sgn), narrow(sgn * flo), narrow(L.sin_tm * cp), narrow(L.sin_tm * sp),
+                  narrow(L.c.m2), y, r2, r3, r4, r5);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) m32.y[i] = narrow(y[i]);
+    m32.a2 = narrow(L.Om * r2[6]);
+    m32.a3 = narrow(L.Om * r3[6]);
+    m32.a4 = narrow(L.Om * r4[6]);
+    m32.a5 = narrow(L.Om * r5[6]);
     if (!(flo >= 0.0)) flo = 0.0;
     if (!(fhi < 0.0)) fhi = -1e-300;
-    double hi;
-    const double lo = last_nonneg(side_val, flo, fhi, &hi);
+    const double lo = event_root(side_val, m32, flo, fhi);
     ++L.nr;
     if (lo < SWITCH_MIN_FRACTION) {
       L.c.sig = -L.c.sig;
@@ -258,7 +292,7 @@ __device__ int advance_rot(const TraceParams& p, RotLane& L) {
     }
     return -1;
   }
-  if (en <= 1.0) {
+  if (ok) {
     ++L.na;
     const double rnew2 = yn[0] * yn[0] + yn[1] * yn[1] + yn[2] * yn[2];
     if (rnew2 >= p.r_out * p.r_out) {
@@ -281,9 +315,9 @@ __device__ int advance_rot(const TraceParams& p, RotLane& L) {
       if (!(flo >= 0.0)) flo = 0.0;
       double fhi = ro2 - rnew2;
       if (!(fhi < 0.0)) fhi = -1e-300;
-      double hi;
-      const double lo = last_nonneg(inside, flo, fhi, &hi);
-      const double th = 0.5 * (lo + hi);
+      EscapeModel32 e32;
+      e32.init(narrow(flo), y, r2, r3, r4, r5);
+      const double th = event_root(inside, e32, flo, fhi);
       dense(th, yn, r2, r3, r4, r5, 8);
 #pragma unroll
       for (int i = 0; i < 8; ++i) L.y[i] = yn[i];
@@ -298,7 +332,7 @@ __device__ int advance_rot(const TraceParams& p, RotLane& L) {
     L.lam += h;
     if (rnew2 <= p.r_capture * p.r_capture) return RAY_CAPTURED;
     if (clipped) return RAY_LAMBDA_END;
-    if (gj && L.c.sig * side_at(L, L.y) < 0.0) {
+    if (across) {
       L.c.sig = -L.c.sig;
       rhs_rot(L, L.y, L.f0);
     }
@@ -306,13 +340,13 @@ __device__ int advance_rot(const TraceParams& p, RotLane& L) {
       L.h = L.h_resume;
       L.switching = false;
     } else {
-      L.h = h * step_factor(en, true, L.last_rej);
+      L.h = h * step_factor_sq(en2, true, L.last_rej);
     }
     L.last_rej = false;
     return -1;
   }
   ++L.nr;
-  L.h = h * step_factor(en, false, L.last_rej);
+  L.h = h * step_factor_sq(en2, false, L.last_rej);
   L.last_rej = true;
   return (L.h < 1e-12) ? RAY_STIFF : -1;
 }
