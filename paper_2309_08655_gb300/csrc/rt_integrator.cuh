@@ -56,33 +56,22 @@ __device__ __forceinline__ double recip_series(double x) {
   return fma(r, fma(d, d, d), r);
 }
 
-// err^(-1/5) to within an ulp or two: a single-precision estimate refined by
-// two Newton steps on y^-5 = err, y <- y (6 - err y^5) / 5 (quadratic
-// convergence: 1e-7, 1e-14, rounding).  Used where the result is clamped to
-// [0.2, 5] after the factor 0.9, i.e. for err in [1.9e-4, 1.9e3].
-__device__ __forceinline__ double pow_m1_5(double err) {
-  double y = (double)exp2f(-0.2f * log2f((float)err));
-#pragma unroll
-  for (int it = 0; it < 2; ++it) {
-    const double y2 = y * y;
-    y = y * (1.2 - 0.2 * err * (y2 * y2 * y));
-  }
-  return y;
+// 1/sqrt(x) to rounding for normal positive x (NaN for negative): the hardware's
+// coarse estimate y corrected by the binomial series in e = 1 - x y^2 (~2^-19),
+// y (1 + e/2 + 3 e^2/8); the rest is O(e^3) ~ 2^-58.  Five FP64 instructions and
+// no branch.
+__device__ __forceinline__ double rsqrt_series(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-x, y * y, 1.0);
+  return fma(y * e, fma(0.375, e, 0.5), y);
 }
 
-__device__ __forceinline__ double step_factor(double err, bool accepted, bool last_rej) {
-  // outside [1e-6, 1e6] the clamp below decides: 0.9 err^-0.2 > 5 or < 0.2
-  double fac = (err > 1e6) ? 0.0 : (err >= 1e-6) ? 0.9 * pow_m1_5(err) : 5.0;
-  fac = fmin(5.0, fmax(0.2, fac));
-  if (!accepted || last_rej) fac = fmin(fac, 1.0);
-  return fac;
-}
-
-// step_factor() of err = sqrt(q), without the root: err^(-1/5) = q^(-1/10), a
+// The controller's factor 0.9 err^(-1/5), clamped to [0.2, 5] (no growth after a
+// rejection), from the squared error norm q: err^(-1/5) = q^(-1/10), a
 // single-precision estimate y corrected by the series of (1 - r)^(-1/10) in the
 // residual r = 1 - q y^10 (at most ~1e-5), y (1 + r/10 + 11 r^2/200).  The clamp
-// to [0.2, 5] is decided on the high words (positive numbers order like their
-// bits).
+// is decided on the high words (positive numbers order like their bits).
 __device__ __forceinline__ double step_factor_sq(double q, bool accepted, bool last_rej) {
   const int hq = __double2hiint(q);
   double fac = 5.0;
@@ -309,9 +298,9 @@ __device__ __forceinline__ float to_f32(double v) { return narrow(v); }
 struct ConeModel32 {
   float sg, F0, m0, m1, m2, gF[3], r2[3], r3[3], r4[3], r5[3];
   // y, R2..R5: the first three (position) components
-  template <class T>
+  template <class Y, class T>
   __device__ __forceinline__ void init(float sig, float F0f, float cm0, float cm1, float cm2,
-                                       const T* y, const T* R2, const T* R3, const T* R4,
+                                       const Y* y, const T* R2, const T* R3, const T* R4,
                                        const T* R5) {
     sg = sig;
     F0 = F0f;
@@ -346,8 +335,8 @@ struct ConeModel32 {
 // c0 = r_out^2 - |y|^2 from FP64.
 struct EscapeModel32 {
   float c0, y[3], r2[3], r3[3], r4[3], r5[3];
-  template <class T>
-  __device__ __forceinline__ void init(float c0f, const T* yd, const T* R2, const T* R3,
+  template <class Y, class T>
+  __device__ __forceinline__ void init(float c0f, const Y* yd, const T* R2, const T* R3,
                                        const T* R4, const T* R5) {
     c0 = c0f;
 #pragma unroll

@@ -14,20 +14,29 @@ namespace rtk {
 
 namespace {
 
-__global__ void __launch_bounds__(128) tail_fp64_kernel(TraceParams p) {
+// Rays left for the launch, from few to many: one group per warp and one warp per
+// scheduler (a guided ray's attempts then wait for no other group's branches and
+// for no other warp's FP64 instructions), up to five groups per warp, then every
+// resident block.
+__global__ void __launch_bounds__(128) tail_fp64_kernel(TraceParams p, int nsm) {
   const int lane = threadIdx.x & 31;
+  __shared__ double slots[GROUP_SLOTS];
   GroupCounts gc;
   if (p.xrec) {   // express records that no express group claimed
     const unsigned long long K = *p.xcount < (unsigned long long)p.xcap
                                      ? *p.xcount : (unsigned long long)p.xcap;
     const unsigned long long S = express_solo(K);
-    tail_groups(p, p.xrec, 0, S, p.xcount + 2, GROUPS_PER_WARP, gc);
-    tail_groups(p, p.xrec, S, K, p.xcount + 1, GROUPS_PER_WARP, gc);
+    tail_groups(p, p.xrec, 0, S, p.xcount + 2, GROUPS_PER_WARP, gc, slots);
+    tail_groups(p, p.xrec, S, K, p.xcount + 1, GROUPS_PER_WARP, gc, slots);
   }
   const unsigned long long nparked = *p.park_count < (unsigned long long)p.park_cap
                                          ? *p.park_count
                                          : (unsigned long long)p.park_cap;
-  tail_groups(p, p.park, 0, nparked, p.park_next, GROUPS_PER_WARP, gc);
+  const unsigned long long wave = 4ull * (unsigned)nsm;     // warps of one block per SM
+  const unsigned long long per = (nparked + wave - 1) / wave;
+  const int ngroups = per < GROUPS_PER_WARP ? (int)(per > 0 ? per : 1) : GROUPS_PER_WARP;
+  if ((int)blockIdx.x < nsm || per > GROUPS_PER_WARP)
+    tail_groups(p, p.park, 0, nparked, p.park_next, ngroups, gc, slots);
   if (p.counters && (lane % GROUP) == 0 && lane / GROUP < GROUPS_PER_WARP) {
     atomicAdd((unsigned long long*)&p.counters[CTR_ACC], (unsigned long long)gc.acc);
     atomicAdd((unsigned long long*)&p.counters[CTR_REJ], (unsigned long long)gc.rej);
@@ -55,7 +64,7 @@ cudaError_t launch_tail_fp64(const TraceParams& p, cudaStream_t stream) {
   const int64_t cap = (int64_t)nsm * (occ > 0 ? occ : 1);
   if (grid > cap) grid = cap;
   if (grid < 1) grid = 1;
-  tail_fp64_kernel<<<(unsigned)grid, 128, 0, stream>>>(p);
+  tail_fp64_kernel<<<(unsigned)grid, 128, 0, stream>>>(p, nsm);
   return cudaGetLastError();
 }
 

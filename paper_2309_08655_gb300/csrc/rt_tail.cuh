@@ -40,112 +40,226 @@ __device__ __forceinline__ int find_star_t(const TraceParams& p, int64_t i) {
   return lo;
 }
 
-// Component c (0-2: dx_c/dl, 3-5: dk_{c-3}/dl) of ham_rhs at the full state y.
-// The scalar prefix is evaluated by every lane, except that its three dot
-// products and its two independent reciprocal square roots are spread over
-// the group's lanes (one FP64 instruction sequence for all, then shuffles:
-// the same operations and operands, so the same results); each lane then
-// takes its component from coefficients that all lanes form.
-__device__ double rhs_comp(const RayConst<double>& c, const double* y, int comp, unsigned gm,
-                           int base) {
-  const double x0 = y[0], x1 = y[1], x2 = y[2], k0 = y[3], k1 = y[4], k2 = y[5];
-  const double r2 = x0 * x0 + x1 * x1 + x2 * x2;
-  const double ir = rsqrt(r2);
-  const double n0 = x0 * ir, n1 = x1 * ir, n2 = x2 * ir;
-  const double ir2 = ir * ir;
-  const double A = 1.0 - c.rs * ir;
-  const double Am1 = -c.rs * ir;
-  const int j = comp < 3 ? comp : comp - 3;
-  // n.k (lane 0), m.n (lane 1), k.m (lane 2) in one pass
-  const double a0 = j == 0 ? n0 : (j == 1 ? c.m0 : k0);
-  const double a1 = j == 0 ? n1 : (j == 1 ? c.m1 : k1);
-  const double a2 = j == 0 ? n2 : (j == 1 ? c.m2 : k2);
-  const double b0 = j == 0 ? k0 : (j == 1 ? n0 : c.m0);
-  const double b1 = j == 0 ? k1 : (j == 1 ? n1 : c.m1);
-  const double b2 = j == 0 ? k2 : (j == 1 ? n2 : c.m2);
-  const double dot = a0 * b0 + a1 * b1 + a2 * b2;
-  const double kr = __shfl_sync(gm, dot, base);
-  const double mu = __shfl_sync(gm, dot, base + 1);
-  const double km = __shfl_sync(gm, dot, base + 2);
-  // 1/sqrt(A) (lanes 0-2) and 1/sqrt(3 mu^2 + 1) (lanes 3-5) in one pass
-  const double rq = rsqrt(comp < 3 ? A : 3.0 * mu * mu + 1.0);
-  const double qA = __shfl_sync(gm, rq, base);
-  const double iA = qA * qA;
-  const double W = c.W2 * iA;
-  const double nj = j == 0 ? n0 : (j == 1 ? n1 : n2);
-  const double kj = j == 0 ? k0 : (j == 1 ? k1 : k2);
-  const double mj = j == 0 ? c.m0 : (j == 1 ? c.m1 : c.m2);
-  double P = 0.0, dPj = 0.0;
-  if (c.plasma == PLASMA_GJ) {
-    const double F = 3.0 * n2 * mu - c.m2;
-    const double ir3 = ir2 * ir;
-    P = c.cp * ir3 * (F * c.sig);
-    const double t = c.cp * ir3 * c.sig * 3.0 * ir;
-    const double m3 = -3.0 * P * ir;
-    const double two_mu_nz = 2.0 * mu * n2;
-    dPj = m3 * nj + t * (n2 * mj - two_mu_nz * nj) + (j == 2 ? t * mu : 0.0);
-  } else if (c.plasma == PLASMA_HOMOG) {
-    P = c.pa;
-  } else if (c.plasma == PLASMA_LINEAR_Z) {
-    P = c.pa * x2;
-    dPj = (j == 2) ? c.pa : 0.0;
-  } else if (c.plasma == PLASMA_RADIAL) {
-    P = c.pa * ir2 * ir;
-    dPj = -3.0 * P * ir * nj;
-  } else if (c.plasma == PLASMA_TWISTED) {
-    const double ir4 = ir2 * ir2;
-    P = c.cp * (1.0 - mu * mu) * ir4;
-    const double q = c.cp * ir4 * ir;
-    dPj = (-2.0 * q * mu) * mj + (q * (6.0 * mu * mu - 4.0)) * nj;
+// The group's right-hand side as passes over a small register file in shared
+// memory.
+//
+// An FP64 instruction costs a warp 64 cycles whether the lanes of a group do the
+// same work or six different products, and a launch of guided rays ends with its
+// longest ray: what counts is the number of FP64 instructions one after another,
+// and what stands between them.  So the scalar coefficients of the
+// Goldreich-Julian anisotropic medium (the one with rays long enough for this
+// mode) are formed in passes: in each, the six lanes take one multiply-add whose
+// operands they read from slots of their own choice, and store the result to a
+// slot.  The slot numbers are one table, read into registers at the start, so a
+// pass is three loads, the multiply-add and a store: 32 FP64 instructions a
+// right-hand side, where every lane forming every scalar takes 105.  (Operands
+// exchanged by shuffles and picked by selects took 13 other instructions for
+// each FP64 one, and 23.5 us an attempt.)
+//
+// Slots: the point, the ray's constants, plain numbers, then what the passes
+// leave.
+enum Slot : int {
+  S_X = 0,                                      // x0 x1 x2 k0 k1 k2
+  S_M = 6, S_M3 = 9,                            // m, 3 m
+  S_RS = 12, S_CPS, S_NM2, S_3M2, S_W2, S_IW2,  // rs, cp sig, -m_z, 3 m_z, W2, 1/W2
+  S_0, S_1, S_N1, S_2, S_N2, S_3, S_N15,
+  S_IR, S_DOT,                                  // 1/r; x.k, m.x, k.m, |x|^2, 3 m.x
+  S_Q = S_DOT + 6,                              // 1/sqrt(A) (0-2), 1/|b| (3-5)
+  S_P1 = S_Q + 6                                // pass n at S_P1 + 6 (n - 1)
+};
+constexpr int PASSES = 14;
+constexpr int SLOTS = S_P1 + 6 * PASSES;
+
+constexpr int res(int pass, int lane) { return S_P1 + 6 * (pass - 1) + lane; }
+
+// what the passes leave
+enum Value : int {
+  V_KR = res(1, 0), V_MU = res(1, 1), V_NZ = res(1, 2), V_IR2 = res(1, 3), V_MU3 = res(1, 4),
+  V_U = res(1, 5),
+  V_A = res(2, 0), V_QA = S_Q, V_IB = S_Q + 3,
+  V_IR3 = res(3, 0), V_MN = res(3, 1), V_UKR = res(3, 2), V_DA = res(3, 3), V_KR2 = res(3, 4),
+  V_MKR = res(3, 5),
+  V_G3 = res(4, 0), V_F = res(4, 1), V_QN = res(4, 2), V_SA = res(4, 3), V_IA = res(4, 4),
+  V_IB2 = res(4, 5),
+  V_P = res(5, 0), V_T = res(5, 1), V_BX0 = res(5, 2), V_OPSA = res(5, 3), V_IA2 = res(5, 4),
+  V_DAQ = res(5, 5),
+  V_C1 = res(6, 0), V_OKR = res(6, 1), V_PA = res(6, 2), V_QM = res(6, 3), V_W2IA2 = res(6, 4),
+  V_A3 = res(6, 5),
+  V_UU = res(7, 0), V_IBIW2 = res(7, 1), V_C1KR = res(7, 2), V_PA2 = res(7, 3), V_S1 = res(7, 4),
+  V_AIW2 = res(7, 5),
+  V_KP = res(8, 0), V_M3U = res(8, 1), V_NIB2 = res(8, 2), V_NAIW2 = res(8, 3),
+  V_NC1 = res(8, 4), V_NP = res(8, 5),
+  V_KP2 = res(9, 0), V_A1 = res(9, 1), V_QIB = res(9, 2), V_NA3 = res(9, 3),
+  V_ONEM = res(10, 0), V_GM = res(10, 1), V_D = res(10, 2), V_KQ = res(10, 3),
+  V_NA1 = res(10, 4),
+  V_W = res(11, 0), V_GMR = res(11, 1), V_BX = res(11, 2), V_S = res(11, 3), V_Z = res(11, 4),
+  V_WQM = res(12, 0), V_GMZ = res(12, 1), V_CK = res(12, 2), V_VS = res(12, 3), V_WQZ = res(12, 4),
+  V_NGA1 = res(12, 5),
+  V_CM = res(13, 0), V_E = res(13, 1),
+  V_CN = res(14, 0)
+};
+
+// Operands of pass n (2 and up to 14): result = a b + c per lane.  Pass 1 (the
+// products with 1/r) and the dot products before it are written out.
+__constant__ unsigned char c_pass[PASSES - 1][GROUP][3] = {
+    // A, and |b|^2 = 3 mu^2 + 1
+    {{V_U, S_N1, S_1}, {V_U, S_N1, S_1}, {V_U, S_N1, S_1}, {V_MU3, V_MU, S_1},
+     {V_MU3, V_MU, S_1}, {V_MU3, V_MU, S_1}},
+    // r^-3, mu n_z, (rs/r) kr, dA/dr, kr^2, mu kr
+    {{V_IR2, S_IR, S_0}, {V_MU, V_NZ, S_0}, {V_U, V_KR, S_0}, {S_RS, V_IR2, S_0},
+     {V_KR, V_KR, S_0}, {V_MU, V_KR, S_0}},
+    // g3 = cp sig r^-3, F, qn, sqrt(A), 1/A, 1/|b|^2
+    {{S_CPS, V_IR3, S_0}, {S_3, V_MN, S_NM2}, {S_N15, V_MN, S_3M2}, {V_A, V_QA, S_0},
+     {V_QA, V_QA, S_0}, {V_IB, V_IB, S_0}},
+    // P, t, -2 (rs/r) kr, 1 + 2 sqrt(A), 1/A^2, dA/dr / sqrt(A)
+    {{V_G3, V_F, S_0}, {V_G3, S_IR, S_0}, {S_N2, V_UKR, S_0}, {S_2, V_SA, S_1},
+     {V_IA, V_IA, S_0}, {V_DA, V_QA, S_0}},
+    // c1, opsA kr, P A, qm, W2/A^2, a3
+    {{V_MU, V_OPSA, S_0}, {V_OPSA, V_KR, S_0}, {V_P, V_A, S_0}, {S_3, V_NZ, S_0},
+     {S_W2, V_IA2, S_0}, {V_MKR, V_DAQ, S_0}},
+    // U, 1/(|b| W2), c1 kr, 2 P A, W2/A^2 + 3 kr^2, A/W2
+    {{V_C1, V_KR, S_DOT + 5}, {V_IB, S_IW2, S_0}, {V_C1, V_KR, S_0}, {S_2, V_PA, S_0},
+     {S_3, V_KR2, V_W2IA2}, {V_A, S_IW2, S_0}},
+    // Kp, 3 mu U, and the negatives of 1/|b|^2, A/W2, c1, P
+    {{V_UU, V_IB, S_0}, {V_MU3, V_UU, S_0}, {S_N1, V_IB2, S_0}, {S_N1, V_AIW2, S_0},
+     {S_N1, V_C1, S_0}, {S_N1, V_P, S_0}},
+    // Kp^2, a1, Kp/(|b| W2), -a3
+    {{V_KP, V_KP, S_0}, {V_M3U, V_NIB2, V_OKR}, {V_KP, V_IBIW2, S_0}, {S_N1, V_A3, S_0},
+     {S_0, S_0, S_0}, {S_0, S_0, S_0}},
+    // 1 - A Kp^2/W2, gm, a1 mu + c1 kr, Kp^2/W2, -a1
+    {{V_NAIW2, V_KP2, S_1}, {V_PA2, V_QIB, S_0}, {V_A1, V_MU, V_C1KR}, {V_KP2, S_IW2, S_0},
+     {S_N1, V_A1, S_0}, {S_0, S_0, S_0}},
+    // w, gm/r, bx, s, z = (a1 mu + c1 kr)/r - a3
+    {{V_T, V_ONEM, S_0}, {V_GM, S_IR, S_0}, {V_GM, V_NC1, V_BX0}, {V_NP, V_KQ, V_S1},
+     {S_IR, V_D, V_NA3}, {S_0, S_0, S_0}},
+    // w qm, gm z, Ck, dA/dr s, w qz, -gm a1 / r
+    {{V_W, V_QM, S_0}, {V_GM, V_Z, S_0}, {V_BX, S_IR, S_0}, {V_DA, V_S, S_0},
+     {V_W, V_MU3, S_0}, {V_GMR, V_NA1, S_0}},
+    // Cm, w qn + gm z
+    {{S_1, V_WQM, V_NGA1}, {V_W, V_QN, V_GMZ}, {S_0, S_0, S_0}, {S_0, S_0, S_0},
+     {S_0, S_0, S_0}, {S_0, S_0, S_0}},
+    // Cn
+    {{S_1, V_E, V_VS}, {S_0, S_0, S_0}, {S_0, S_0, S_0}, {S_0, S_0, S_0}, {S_0, S_0, S_0},
+     {S_0, S_0, S_0}}};
+
+// A lane's view of its group's slots: byte offsets of its operands.
+struct GroupFile {
+  double* s;                        // the group's SLOTS slots
+  unsigned off[PASSES - 1][3];
+  int cc, j;                        // component, and component mod 3
+  unsigned gm;
+};
+
+__device__ __forceinline__ void file_init(GroupFile& f, double* slots, int cc, unsigned gm) {
+  f.s = slots;
+  f.cc = cc;
+  f.j = cc < 3 ? cc : cc - 3;
+  f.gm = gm;
+#pragma unroll
+  for (int p = 0; p < PASSES - 1; ++p)
+#pragma unroll
+    for (int q = 0; q < 3; ++q) f.off[p][q] = 8u * c_pass[p][cc][q];
+}
+
+__device__ __forceinline__ double slot_at(const GroupFile& f, unsigned off) {
+  return *(const double*)((const char*)f.s + off);
+}
+
+// The ray's constants, and the plain numbers (every lane of the group).
+__device__ __forceinline__ void file_ray(const GroupFile& f, const RayConst<double>& c) {
+  __syncwarp(f.gm);
+  double* s = f.s;
+  if (f.cc == 0) {
+    s[S_M] = c.m0;
+    s[S_M + 1] = c.m1;
+    s[S_M + 2] = c.m2;
+    s[S_M3] = 3.0 * c.m0;
+    s[S_M3 + 1] = 3.0 * c.m1;
+    s[S_M3 + 2] = 3.0 * c.m2;
+    s[S_RS] = c.rs;
+    s[S_CPS] = c.cp * c.sig;
+    s[S_NM2] = -c.m2;
+    s[S_3M2] = 3.0 * c.m2;
+    s[S_W2] = c.W2;
+    s[S_IW2] = c.iW2;
+    s[S_0] = 0.0;
+    s[S_1] = 1.0;
+    s[S_N1] = -1.0;
+    s[S_2] = 2.0;
+    s[S_N2] = -2.0;
+    s[S_3] = 3.0;
+    s[S_N15] = -15.0;
   }
-  // the anisotropic scalars both kinds of component use, once
-  const bool aniso = (c.disp != DISP_ISO);
-  double ib = 0.0, sA = 0.0, U = 0.0, Kp = 0.0, fac = 0.0, opsA = 0.0;
-  if (aniso) {
-    ib = __shfl_sync(gm, rq, base + 3);
-    sA = A * qA;
-    U = 3.0 * mu * kr - km + 2.0 * mu * kr * (sA - 1.0);
-    Kp = U * ib;
-    fac = P * A * Kp * c.iW2;
-    opsA = 1.0 + 2.0 * sA;
+  __syncwarp(f.gm);
+}
+
+// Own component (0-2: dx_j/dl, 3-5: dk_j/dl) of the right-hand side at the point
+// whose own component is yc.  *r2 = |x|^2 and *F the null-cone factor there (any
+// positive multiple of it: its sign is the side; Goldreich-Julian only).
+__device__ __forceinline__ double rhs_group(const GroupFile& f, const RayConst<double>& c,
+                                            double yc, double* r2, double* F) {
+  double* s = f.s;
+  __syncwarp(f.gm);
+  s[S_X + f.cc] = yc;
+  __syncwarp(f.gm);
+  if (c.plasma != PLASMA_GJ || c.disp == DISP_ISO) {
+    // every lane evaluates the whole right-hand side and keeps its component
+    double y[6], g[6];
+#pragma unroll
+    for (int q = 0; q < 6; ++q) y[q] = s[S_X + q];
+    rhs64(c, y, g);
+    *r2 = y[0] * y[0] + y[1] * y[1] + y[2] * y[2];
+    *F = c.plasma == PLASMA_GJ ? 3.0 * y[2] * (c.m0 * y[0] + c.m1 * y[1] + c.m2 * y[2]) - c.m2 * *r2
+                               : 1.0;
+    double out = g[0];
+#pragma unroll
+    for (int q = 1; q < 6; ++q) out = f.cc == q ? g[q] : out;
+    return out;
   }
-  // Both kinds of component as out = al k_j + be n_j + ga m_j (+ dP_j one_m):
-  // every lane forms both coefficient sets (no divergence), then takes its own.
-  // position (c < 3): dH/dk_j = 2 (k_j + (A-1) kr n_j) - 2 fac ib (mu opsA n_j - m_j)
-  const double gk_be = 2.0 * Am1 * kr - 2.0 * fac * ib * mu * opsA;
-  const double gk_ga = 2.0 * fac * ib;
-  // momentum (c >= 3): -dH/dx_j, dH/dx_j = cA n_j + ckr (k_j - kr n_j)
-  //   + dP_j one_m + cdA n_j - 2 fac (a1r m_j + a2r k_j + an n_j)
-  const double cA = (W * iA + kr * kr) * c.rs * ir2;
-  const double ckr = 2.0 * Am1 * kr * ir;
-  double gx_al = ckr, gx_be = cA - ckr * kr, gx_ga = 0.0, one_m = 1.0;
-  if (aniso) {
-    const double Kp2iW2 = Kp * Kp * c.iW2;
-    const double ib3 = ib * ib * ib;
-    const double a1 = ib * opsA * kr - 3.0 * mu * U * ib3;
-    const double a2 = ib * opsA * mu;
-    const double a3 = ib * mu * kr * c.rs * ir2 * qA;
-    const double a1r = a1 * ir, a2r = a2 * ir;
-    const double an = a3 - a1r * mu - a2r * kr;
-    one_m = 1.0 - A * Kp2iW2;
-    const double cdA = -P * Kp2iW2 * c.rs * ir2;
-    const double m2f = -2.0 * fac;
-    gx_al += m2f * a2r;
-    gx_be += cdA + m2f * an;
-    gx_ga = m2f * a1r;
+  // x.k, m.x, k.m, |x|^2, 3 m.x, -k.m
+  const double* va = s + (f.cc == 2 || f.cc == 5 ? S_X + 3 : S_X);
+  const double* vb = s + (f.cc == 0 ? S_X + 3 : f.cc == 3 ? S_X : f.cc == 4 ? S_M3 : S_M);
+  double d = va[0] * vb[0] + va[1] * vb[1] + va[2] * vb[2];
+  s[S_DOT + f.cc] = f.cc == 5 ? -d : d;
+  __syncwarp(f.gm);
+  const double rr = s[S_DOT + 3];
+  const double ir = rsqrt_series(rr);
+  // kr, mu, n_z, r^-2, 3 mu, rs/r
+  const double v1 = f.cc == 2 ? s[S_X + 2] : f.cc == 3 ? ir : f.cc == 5 ? s[S_RS] : d;
+  s[S_P1 + f.cc] = ir * v1;
+  s[S_IR] = ir;                       // every lane the same value
+  const double nj = ir * s[S_X + f.j];
+  __syncwarp(f.gm);
+  auto pass = [&](int n) {
+    const unsigned* o = f.off[n - 2];
+    return fma(slot_at(f, o[0]), slot_at(f, o[1]), slot_at(f, o[2]));
+  };
+  double* out = s + S_P1 + f.cc;
+  const double p2 = pass(2);
+  out[6] = p2;
+  out[12] = pass(3);
+  s[S_Q + f.cc] = rsqrt_series(p2);
+  __syncwarp(f.gm);
+#pragma unroll
+  for (int n = 4; n <= PASSES; ++n) {
+    out[6 * (n - 1)] = pass(n);
+    __syncwarp(f.gm);
   }
-  const bool pos = comp < 3;
-  const double al = pos ? 2.0 : -gx_al;
-  const double be = pos ? gk_be : -gx_be;
-  const double ga = pos ? gk_ga : -gx_ga;
-  const double dp = pos ? 0.0 : -dPj * one_m;
-  return al * kj + be * nj + ga * mj + dp;
+  // 2 k + bx n + gm m, or -(Cn n + Ck k + Cm m + Cz e_z)
+  const bool pos = f.cc < 3;
+  const double al = s[pos ? (int)S_2 : (int)V_CK], be = s[pos ? (int)V_BX : (int)V_CN],
+               ga = s[pos ? (int)V_GM : (int)V_CM], dz = s[f.cc == 5 ? (int)V_WQZ : (int)S_0];
+  const double g = fma(be, nj, fma(al, s[S_X + 3 + f.j], fma(ga, s[S_M + f.j], dz)));
+  *r2 = rr;
+  *F = s[V_F];
+  return pos ? g : -g;
 }
 
 // Group state: lane c of a group owns component c; the rest is replicated.
 struct GLane {
   RayConst<double> c;
   double yc, f0c;      // own component of the state and of f at the state
+  double r2;           // |x|^2 at the state
   double h, h_resume, lam;
   int na, nr;
   bool last_rej, switching;
@@ -153,107 +267,110 @@ struct GLane {
   int star;
 };
 
-// The group's six values of v, in component order, to every lane of the group.
-__device__ __forceinline__ void gather6(unsigned gm, int base, double v, double* out) {
+// The group's three position values of v to every lane of the group.
+__device__ __forceinline__ void gather3d(unsigned gm, int base, double v, double* out) {
 #pragma unroll
-  for (int q = 0; q < GROUP; ++q) out[q] = __shfl_sync(gm, v, base + q);
+  for (int q = 0; q < 3; ++q) out[q] = __shfl_sync(gm, v, base + q);
+}
+
+// The other side of the null cone from here on, and the derivative there.
+__device__ __forceinline__ void flip_side(const GroupFile& f, GLane& L) {
+  L.c.sig = -L.c.sig;
+  __syncwarp(f.gm);
+  if (f.cc == 0) f.s[S_CPS] = L.c.cp * L.c.sig;
+  double F;
+  L.f0c = rhs_group(f, L.c, L.yc, &L.r2, &F);
+}
+
+// The group's three position values of v in FP32 (for the events' models).
+__device__ __forceinline__ void gather3(unsigned gm, int base, double v, float* out) {
+  const float f = narrow(v);
+#pragma unroll
+  for (int q = 0; q < 3; ++q) out[q] = __shfl_sync(gm, f, base + q);
 }
 
 // One attempted step of the group's ray; the same decisions as advance().
-__device__ int advance_group(const TraceParams& p, GLane& L, int cc, unsigned gm, int base) {
+__device__ __forceinline__ int advance_group(const TraceParams& p, const GroupFile& f, GLane& L,
+                                             int cc, unsigned gm, int base) {
   if (L.na >= p.max_steps || L.na + L.nr >= 4 * p.max_steps) return RAY_MAXSTEPS;
-  double yfull[6], t[6];
-  gather6(gm, base, L.yc, yfull);
   bool clipped = false;
   double h = L.h;
   {
-    double fx[6];
-    gather6(gm, base, L.f0c, fx);
-    const double v2 = fx[0] * fx[0] + fx[1] * fx[1] + fx[2] * fx[2];
-    const double r2 = yfull[0] * yfull[0] + yfull[1] * yfull[1] + yfull[2] * yfull[2];
-    if (h * h * v2 > STEP_REACH * STEP_REACH * r2) h = STEP_REACH * sqrt(r2 / v2);
+    // |f_x|^2: the three position lanes' squares
+    const double q = L.f0c * L.f0c;
+    const double v2 = __shfl_sync(gm, q, base) + __shfl_sync(gm, q, base + 1) +
+                      __shfl_sync(gm, q, base + 2);
+    if (h * h * v2 > STEP_REACH * STEP_REACH * L.r2) h = STEP_REACH * sqrt(L.r2 / v2);
   }
   if (p.lambda_max > 0.0 && L.lam + h >= p.lambda_max) {
     h = p.lambda_max - L.lam;
     clipped = true;
   }
   const double y = L.yc;
-  double K1 = L.f0c, K2, K3, K4, K5, K6, K7;
-  gather6(gm, base, y + h * (DP::a21 * K1), t);
-  K2 = rhs_comp(L.c, t, cc, gm, base);
-  gather6(gm, base, y + h * (DP::a31 * K1 + DP::a32 * K2), t);
-  K3 = rhs_comp(L.c, t, cc, gm, base);
-  gather6(gm, base, y + h * (DP::a41 * K1 + DP::a42 * K2 + DP::a43 * K3), t);
-  K4 = rhs_comp(L.c, t, cc, gm, base);
-  gather6(gm, base, y + h * (DP::a51 * K1 + DP::a52 * K2 + DP::a53 * K3 + DP::a54 * K4), t);
-  K5 = rhs_comp(L.c, t, cc, gm, base);
-  gather6(gm, base,
-          y + h * (DP::a61 * K1 + DP::a62 * K2 + DP::a63 * K3 + DP::a64 * K4 + DP::a65 * K5),
-          t);
-  K6 = rhs_comp(L.c, t, cc, gm, base);
+  double K1 = L.f0c, K2, K3, K4, K5, K6, K7, r2s, Fs;
+  K2 = rhs_group(f, L.c, y + h * (DP::a21 * K1), &r2s, &Fs);
+  K3 = rhs_group(f, L.c, y + h * (DP::a31 * K1 + DP::a32 * K2), &r2s, &Fs);
+  K4 = rhs_group(f, L.c, y + h * (DP::a41 * K1 + DP::a42 * K2 + DP::a43 * K3), &r2s, &Fs);
+  K5 = rhs_group(f, L.c, y + h * (DP::a51 * K1 + DP::a52 * K2 + DP::a53 * K3 + DP::a54 * K4), &r2s,
+                 &Fs);
+  K6 = rhs_group(
+      f, L.c, y + h * (DP::a61 * K1 + DP::a62 * K2 + DP::a63 * K3 + DP::a64 * K4 + DP::a65 * K5),
+      &r2s, &Fs);
   const double yn = y + h * (DP::b1 * K1 + DP::b3 * K3 + DP::b4 * K4 + DP::b5 * K5 + DP::b6 * K6);
-  double ynf[6];
-  gather6(gm, base, yn, ynf);
-  K7 = rhs_comp(L.c, ynf, cc, gm, base);
+  double rnew2, Fnew;
+  K7 = rhs_group(f, L.c, yn, &rnew2, &Fnew);
   const double e = h * (DP::e1 * K1 + DP::e3 * K3 + DP::e4 * K4 + DP::e5 * K5 + DP::e6 * K6 +
                         DP::e7 * K7);
-  const double sc = p.atol + p.rtol * fmax(fabs(y), fabs(yn));
-  double q6[6];
-  gather6(gm, base, (e / sc) * (e / sc), q6);
-  const double en = sqrt((q6[0] + q6[1] + q6[2] + q6[3] + q6[4] + q6[5]) / 6.0);
-  if (!isfinite(en)) {
+  const double eq = e * recip_series(p.atol + p.rtol * max_abs(y, yn));
+  // the sum over the group: lanes c and c + 3 form the same pair sum, so every
+  // lane holds the same bits
+  const double pair = eq * eq + __shfl_sync(gm, eq * eq, base + (cc < 3 ? cc + 3 : cc - 3));
+  const double en2 = (__shfl_sync(gm, pair, base) + __shfl_sync(gm, pair, base + 1) +
+                      __shfl_sync(gm, pair, base + 2)) * (1.0 / 6.0);
+  if ((__double2hiint(en2) & 0x7ff00000) == 0x7ff00000) {   // infinite or NaN
     ++L.nr;
     L.h = h * 0.2;
     L.last_rej = true;
     return (L.h < 1e-12) ? RAY_NAN : -1;
   }
+  const bool ok = en2 <= 1.0;
   const bool gj = (L.c.plasma == PLASMA_GJ);
-  // continuous extension, own component
-  const double r2c = yn - y;
-  const double r3c = h * K1 - r2c;
-  const double r4c = r2c - h * K7 - r3c;
-  const double r5c = h * (DP::d1 * K1 + DP::d3 * K3 + DP::d4 * K4 + DP::d5 * K5 + DP::d6 * K6 +
-                          DP::d7 * K7);
-  if (en <= 1.0 && gj && !L.switching &&
-      L.c.sig * gj_side<double>(L.c.m0, L.c.m1, L.c.m2, ynf[0], ynf[1], ynf[2]) < 0.0) {
-    // Illinois on the side function along the continuous extension
+  const bool across = ok && gj && (Fnew < 0.0) != (L.c.sig < 0.0);
+  const bool out = ok && rnew2 >= p.r_out * p.r_out;
+  // continuous extension, own component (and the position's, in FP32)
+  double r2c = 0.0, r3c = 0.0, r4c = 0.0, r5c = 0.0;
+  float yx[3], r2x[3], r3x[3], r4x[3], r5x[3];
+  if ((across && !L.switching) || out) {
+    r2c = yn - y;
+    r3c = h * K1 - r2c;
+    r4c = r2c - h * K7 - r3c;
+    r5c = h * (DP::d1 * K1 + DP::d3 * K3 + DP::d4 * K4 + DP::d5 * K5 + DP::d6 * K6 + DP::d7 * K7);
+    gather3(gm, base, r2c, r2x);
+    gather3(gm, base, r3c, r3x);
+    gather3(gm, base, r4c, r4x);
+    gather3(gm, base, r5c, r5x);
+    gather3(gm, base, y, yx);
+  }
+  if (across && !L.switching) {
+    // root of the side function along the continuous extension, as advance()
     const double sgn = L.c.sig;
     auto side_val = [&](double th) {
-      double xd[6];
-      gather6(gm, base, y + th * (r2c + (1.0 - th) * (r3c + th * (r4c + (1.0 - th) * r5c))), xd);
+      double xd[3];
+      gather3d(gm, base, y + th * (r2c + (1.0 - th) * (r3c + th * (r4c + (1.0 - th) * r5c))), xd);
       const double mx = L.c.m0 * xd[0] + L.c.m1 * xd[1] + L.c.m2 * xd[2];
       const double rr = xd[0] * xd[0] + xd[1] * xd[1] + xd[2] * xd[2];
       return sgn * (3.0 * xd[2] * mx - L.c.m2 * rr);
     };
-    double lo = 0.0, hi = 1.0;
     double flo = side_val(0.0), fhi = side_val(1.0);
+    ConeModel32 m32;
+    m32.init(narrow(sgn), narrow(sgn * flo), narrow(L.c.m0), narrow(L.c.m1), narrow(L.c.m2), yx,
+             r2x, r3x, r4x, r5x);
     if (!(flo >= 0.0)) flo = 0.0;
     if (!(fhi < 0.0)) fhi = -1e-300;
-    int last = 0;
-    double width = 1.0;
-    for (int it = 0; it < 200; ++it) {
-      double mid = (lo * fhi - hi * flo) / (fhi - flo);
-      if ((it & 1) && hi - lo > 0.5 * width) mid = 0.5 * (lo + hi);
-      if (!(mid > lo && mid < hi)) mid = 0.5 * (lo + hi);
-      if (mid <= lo || mid >= hi) break;
-      if (it & 1) width = hi - lo;
-      const double fm = side_val(mid);
-      if (fm >= 0.0) {
-        lo = mid;
-        flo = fm;
-        if (last > 0) fhi *= 0.5;
-        last = 1;
-      } else {
-        hi = mid;
-        fhi = fm;
-        if (last < 0) flo *= 0.5;
-        last = -1;
-      }
-    }
+    const double lo = event_root(side_val, m32, flo, fhi);
     ++L.nr;
     if (lo < SWITCH_MIN_FRACTION) {
-      L.c.sig = -L.c.sig;
-      L.f0c = rhs_comp(L.c, yfull, cc, gm, base);
+      flip_side(f, L);
       L.h = h;
     } else {
       L.h_resume = h;
@@ -262,52 +379,54 @@ __device__ int advance_group(const TraceParams& p, GLane& L, int cc, unsigned gm
     }
     return -1;
   }
-  if (en <= 1.0) {
+  if (ok) {
     ++L.na;
-    const double rnew2 = ynf[0] * ynf[0] + ynf[1] * ynf[1] + ynf[2] * ynf[2];
-    if (rnew2 >= p.r_out * p.r_out) {
-      // |x(th)| = r_out on the continuous extension: Illinois, as advance()
+    if (out) {
+      // |x(th)| = r_out on the continuous extension, as advance()
       const double ro2 = p.r_out * p.r_out;
       auto inside = [&](double th) {
-        double xd[6];
-        gather6(gm, base, y + th * (r2c + (1.0 - th) * (r3c + th * (r4c + (1.0 - th) * r5c))),
+        double xd[3];
+        gather3d(gm, base, y + th * (r2c + (1.0 - th) * (r3c + th * (r4c + (1.0 - th) * r5c))),
                 xd);
         return ro2 - (xd[0] * xd[0] + xd[1] * xd[1] + xd[2] * xd[2]);
       };
-      double flo = ro2 - (yfull[0] * yfull[0] + yfull[1] * yfull[1] + yfull[2] * yfull[2]);
+      double flo = ro2 - L.r2;
       if (!(flo >= 0.0)) flo = 0.0;
       double fhi = ro2 - rnew2;
       if (!(fhi < 0.0)) fhi = -1e-300;
-      double hi;
-      const double lo = last_nonneg(inside, flo, fhi, &hi);
-      const double th = 0.5 * (lo + hi);
+      EscapeModel32 e32;
+      e32.init(narrow(flo), yx, r2x, r3x, r4x, r5x);
+      const double th = event_root(inside, e32, flo, fhi);
       L.yc = y + th * (r2c + (1.0 - th) * (r3c + th * (r4c + (1.0 - th) * r5c)));
       L.lam += th * h;
       return RAY_ESCAPED;
     }
     L.yc = yn;
     L.f0c = K7;
+    L.r2 = rnew2;
     L.lam += h;
     if (rnew2 <= p.r_capture * p.r_capture) return RAY_CAPTURED;
     if (clipped) return RAY_LAMBDA_END;
-    if (gj && L.c.sig * gj_side<double>(L.c.m0, L.c.m1, L.c.m2, ynf[0], ynf[1], ynf[2]) < 0.0) {
-      L.c.sig = -L.c.sig;
-      L.f0c = rhs_comp(L.c, ynf, cc, gm, base);
+    if (across) {
+      flip_side(f, L);
     }
     if (L.switching) {
       L.h = L.h_resume;
       L.switching = false;
     } else {
-      L.h = h * step_factor(en, true, L.last_rej);
+      L.h = h * step_factor_sq(en2, true, L.last_rej);
     }
     L.last_rej = false;
     return -1;
   }
   ++L.nr;
-  L.h = h * step_factor(en, false, L.last_rej);
+  L.h = h * step_factor_sq(en2, false, L.last_rej);
   L.last_rej = true;
   return (L.h < 1e-12) ? RAY_STIFF : -1;
 }
+
+// shared doubles of a block of up to four warps
+constexpr int GROUP_SLOTS = 4 * GROUPS_PER_WARP * SLOTS;
 
 // Counts of one warp's finished rays (lane c == 0 of each group holds its own).
 struct GroupCounts {
@@ -319,16 +438,19 @@ struct GroupCounts {
 // ray, lambda), e = 0, 1, ... claimed one per group with an atomic on *next,
 // while lo + e < hi.  ngroups (1 to GROUPS_PER_WARP) groups of the warp take
 // part: one group per warp keeps a ray's attempts free of the other groups'
-// divergent branches.  Every lane of the warp must call it.
+// divergent branches.  slots: shared memory of the block, GROUP_SLOTS doubles.
+// Every lane of the warp must call it.
 __device__ void tail_groups(const TraceParams& p, const double* recs, unsigned long long lo,
                             unsigned long long hi, unsigned long long* next, int ngroups,
-                            GroupCounts& cnt) {
+                            GroupCounts& cnt, double* slots) {
   const int lane = threadIdx.x & 31;
   const int g = lane / GROUP, cc = lane % GROUP;
   const bool in_group = g < ngroups && g < GROUPS_PER_WARP;
   const int base = g * GROUP;
   const unsigned gm = in_group ? (0x3Fu << base) : 0u;
   GLane L;
+  GroupFile f;
+  if (in_group) file_init(f, slots + ((threadIdx.x >> 5) * GROUPS_PER_WARP + g) * SLOTS, cc, gm);
   bool have = false, done = !in_group;
   int na0 = 0, nr0 = 0;
   for (;;) {
@@ -367,9 +489,9 @@ __device__ void tail_groups(const TraceParams& p, const double* recs, unsigned l
         L.c.disp = s.dispersion;
         L.c.plasma = s.plasma;
         L.c.sig = sig;
-        double yfull[6];
-        gather6(gm, base, L.yc, yfull);
-        L.f0c = rhs_comp(L.c, yfull, cc, gm, base);
+        file_ray(f, L.c);
+        double F;
+        L.f0c = rhs_group(f, L.c, L.yc, &L.r2, &F);
         na0 = L.na;
         nr0 = L.nr;
         have = true;
@@ -377,7 +499,7 @@ __device__ void tail_groups(const TraceParams& p, const double* recs, unsigned l
     }
     if (__ballot_sync(0xffffffffu, in_group && !done) == 0) break;
     if (have) {
-      const int st = advance_group(p, L, cc, gm, base);
+      const int st = advance_group(p, f, L, cc, gm, base);
       if (st >= 0) {
         const StarDev& s = p.stars[L.star];
         const int64_t n = p.n;

@@ -161,6 +161,7 @@ __global__ void __launch_bounds__(128) trace_fp64_kernel(TraceParams p) {
     const unsigned long long xs = express_sms(K);
     const unsigned long long S = express_solo(K);
     __shared__ int role;
+    __shared__ double slots[GROUP_SLOTS];
     if (threadIdx.x == 0) {
       const unsigned sm = sm_id();
       role = (sm < xs && sm < (unsigned)XSLOTS) ? atomicAdd(p.xslot + sm, 1) : -1;
@@ -168,8 +169,8 @@ __global__ void __launch_bounds__(128) trace_fp64_kernel(TraceParams p) {
     __syncthreads();
     if (role == 0) {
       GroupCounts gc;
-      if ((threadIdx.x >> 5) < 2) tail_groups(p, p.xrec, 0, S, p.xcount + 2, 1, gc);
-      tail_groups(p, p.xrec, S, K, p.xcount + 1, GROUPS_PER_WARP, gc);
+      if ((threadIdx.x >> 5) < 2) tail_groups(p, p.xrec, 0, S, p.xcount + 2, 1, gc, slots);
+      tail_groups(p, p.xrec, S, K, p.xcount + 1, GROUPS_PER_WARP, gc, slots);
       acc += gc.acc;
       rej += gc.rej;
       traced += gc.traced;
