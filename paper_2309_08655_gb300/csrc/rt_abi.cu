@@ -115,6 +115,7 @@ struct rt_star {
   rtk::StarDev h;               // host copy of the descriptor
   rtk::StarDev* d = nullptr;    // device copy
   unsigned long long* d_queue = nullptr;  // trace work-queue counter (scratch)
+  unsigned long long* d_guided = nullptr; // guided rays (rt_guided.cuh; scratch)
   long long* d_bins = nullptr;  // binning accumulator (scratch)
   size_t bins_cap = 0;
   int device = 0;
@@ -200,7 +201,9 @@ rt_status rt_init_star(const rt_star_params* p, rt_star** out) {
     return cuda_fail(e, "cudaGetDevice");
   }
   void* blk = nullptr;
-  e = cudaMalloc(&blk, 256 + sizeof(rtk::StarDev));
+  // [queue counter | descriptor | guided rays]
+  const size_t desc = (sizeof(rtk::StarDev) + 255) / 256 * 256;
+  e = cudaMalloc(&blk, 256 + desc + rtk::guided_bytes());
   if (e != cudaSuccess) {
     delete s;
     return (e == cudaErrorMemoryAllocation) ? fail(RT_ENOMEM, "cudaMalloc failed")
@@ -208,6 +211,7 @@ rt_status rt_init_star(const rt_star_params* p, rt_star** out) {
   }
   s->d_queue = (unsigned long long*)blk;
   s->d = (rtk::StarDev*)((char*)blk + 256);
+  s->d_guided = (unsigned long long*)((char*)blk + 256 + desc);
   e = cudaMemcpy(s->d, &h, sizeof(h), cudaMemcpyHostToDevice);
   if (e != cudaSuccess) {
     cudaFree(blk);
@@ -402,6 +406,7 @@ rt_status rt_trace_forward(const rt_star* s, int64_t n, double* d_state, uint8_t
   p.nrej = d_nrej;
   p.counters = d_counters;
   p.queue = s->d_queue;
+  if (o->precision != RT_PREC_FP64 || rigid) p.guided = s->d_guided;
   p.ts = (unsigned long long*)o->timestamps;
   if (o->tail != 1 && o->lambda_max == 0.0 && !rigid && o->precision != RT_PREC_DF) {
     rt_star* sm = const_cast<rt_star*>(s);
@@ -861,6 +866,7 @@ struct rt_batch {
   rtk::StarDev* d_stars = nullptr;    // device table
   int64_t* d_off = nullptr;           // device offsets
   unsigned long long* d_queue = nullptr;
+  unsigned long long* d_guided = nullptr;  // guided rays (rt_guided.cuh; scratch)
   long long* d_bins = nullptr;        // nstars x per-star binning accumulators
   size_t bins_per_star = 0;
   int device = 0;
@@ -916,7 +922,8 @@ rt_status rt_init_batch(const rt_star* const* stars, int32_t nstars, const int64
   cudaGetDevice(&b->device);
   const size_t tbl = sizeof(rtk::StarDev) * nstars, offb = sizeof(int64_t) * (nstars + 1);
   void* blk = nullptr;
-  cudaError_t e = cudaMalloc(&blk, 256 + tbl + 256 + offb);
+  const size_t tblp = (tbl + 255) / 256 * 256, offp = (offb + 255) / 256 * 256;
+  cudaError_t e = cudaMalloc(&blk, 256 + tblp + offp + rtk::guided_bytes());
   if (e != cudaSuccess) {
     cudaGetLastError();
     delete b;
@@ -924,7 +931,8 @@ rt_status rt_init_batch(const rt_star* const* stars, int32_t nstars, const int64
   }
   b->d_queue = (unsigned long long*)blk;
   b->d_stars = (rtk::StarDev*)((char*)blk + 256);
-  b->d_off = (int64_t*)((char*)blk + 256 + ((tbl + 255) / 256) * 256);
+  b->d_off = (int64_t*)((char*)blk + 256 + tblp);
+  b->d_guided = (unsigned long long*)((char*)blk + 256 + tblp + offp);
   e = cudaMemcpy(b->d_stars, table.data(), tbl, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(b->d_off, b->off.data(), offb, cudaMemcpyHostToDevice);
   if (e != cudaSuccess) {
@@ -1121,6 +1129,7 @@ rt_status rt_trace_batch(rt_batch* b, double* d_state, uint8_t* d_status, int32_
   p.nrej = d_nrej;
   p.counters = d_counters;
   p.queue = b->d_queue;
+  if (o->precision != RT_PREC_FP64 || b->rigid) p.guided = b->d_guided;
   p.ts = (unsigned long long*)o->timestamps;
   if (o->tail != 1 && o->lambda_max == 0.0 && !b->rigid && o->precision != RT_PREC_DF) {
     if ((st = ensure_park(&b->d_park, &b->park_cap)) != RT_OK) return st;
@@ -1168,8 +1177,17 @@ rt_status rt_trace_batch(rt_batch* b, double* d_state, uint8_t* d_status, int32_
       e = cudaMemsetAsync(b->d_promo_n, 0, sizeof(unsigned long long), (cudaStream_t)stream);
       if (e == cudaSuccess) e = rtk::launch_batch_mixed(p, t, blk, bps, (cudaStream_t)stream);
       if (e != cudaSuccess) return cuda_fail(e, "mixed batch kernel");
-      // FP64: the promoted rays from where they stopped, the listed pixels anew
+      // FP64: the promoted rays from where they stopped, in tail mode (rays guided
+      // along the null cone are among them; one lane each they held the launch for
+      // 25 us an attempt), and the listed pixels anew
       p.claim_status = rtk::RAY_PROMOTED;
+      if (p.park && p.n > 0) {
+        rtk::TraceParams r = p;
+        r.refill_min = r.claim_size = 1;
+        e = rtk::launch_trace_fp64(r, 0, 0, (cudaStream_t)stream);
+        if (e != cudaSuccess) return cuda_fail(e, "trace kernel (promoted rays)");
+        p.n = 0;
+      }
       p.refill_min = p.claim_size = 1;
       t.list = b->d_promo;
       t.list_n = b->d_promo_n;

@@ -70,7 +70,23 @@ struct TraceParams {
   // a lane claims claim_size consecutive queue entries at a time
   int refill_min = 1;
   int claim_size = 1;
+  // lanes of a warp that take rays (spread_lanes)
+  int lanes = 32;
+  // guided rays (rt_guided.cuh): [0] found, then (key, ray) pairs, then the list;
+  // the first guided_max of the list have left the queue
+  unsigned long long* guided = nullptr;
+  int64_t guided_max = 0;
 };
+// The guided rays' scratch: a counter, GUIDED_CAP (key, ray) pairs and the list.
+constexpr int64_t GUIDED_CAP = 8192;
+inline size_t guided_bytes() { return 256 + (size_t)GUIDED_CAP * 3 * sizeof(unsigned long long); }
+// Lanes per warp of a persistent launch over n rays: with fewer than 32 rays for
+// each warp of one block of four per SM, every scheduler gets a warp and each warp
+// its share.  A warp's attempt costs the branches that any of its lanes takes.
+inline int spread_lanes(int64_t n, int nsm) {
+  const int64_t l = (n + (int64_t)nsm * 4 - 1) / ((int64_t)nsm * 4);
+  return l < 1 ? 1 : l > 32 ? 32 : (int)l;
+}
 constexpr int64_t XPARK_MIN_RAYS = (int64_t)4 << 20;
 constexpr int COST_BUCKETS = 3;
 constexpr int PARKREC = 14;   // y[6], h, h_resume, sig, flags, na, nr, ray, lambda
@@ -138,6 +154,9 @@ cudaError_t launch_trace_fp64(const TraceParams& p, int block, int blocks_per_sm
                               cudaStream_t stream);
 cudaError_t launch_trace_mixed(const TraceParams& p, int block, int blocks_per_sm,
                                cudaStream_t stream);
+// Lists the guided rays for a launch of the given number of warps (p.guided set;
+// sets p.guided_max).
+cudaError_t launch_guided(TraceParams& p, int64_t warps, cudaStream_t stream);
 cudaError_t launch_tail_fp64(const TraceParams& p, cudaStream_t stream);
 // Binning: launch_bin = clear p.acc, then the three phases; the phases alone
 // serve the sharded binning (rt_bin_part_*), whose callers reduce p.acc

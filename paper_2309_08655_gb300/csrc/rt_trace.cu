@@ -129,6 +129,40 @@ __global__ void express_rank_kernel(TraceParams p) {
   }
 }
 
+// Guided rays of the lane-per-ray kernels (rt_guided.cuh): the READY rays of cost
+// bucket 0 as (key, ray) pairs, then into the list by rank, nearest the cone first;
+// the first guided_max leave the queue (RAY_EXPRESS).
+__global__ void guided_select_kernel(TraceParams p) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < p.n;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    if (p.status[i] != RAY_READY) continue;
+    const double d2 = cone_dist2(p.stars[find_star(p, i)], p.state, p.n, i);
+    if (!(d2 < 1e-6)) continue;
+    const unsigned long long slot = atomicAdd(p.guided, 1ull);
+    if (slot < (unsigned long long)GUIDED_CAP) {
+      p.guided[32 + 2 * slot] = (unsigned long long)__double_as_longlong(d2);
+      p.guided[32 + 2 * slot + 1] = (unsigned long long)i;
+    }
+  }
+}
+
+__global__ void guided_rank_kernel(TraceParams p) {
+  const unsigned long long K = *p.guided < (unsigned long long)GUIDED_CAP
+                                   ? *p.guided : (unsigned long long)GUIDED_CAP;
+  const unsigned long long* cand = p.guided + 32;
+  for (unsigned long long k = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; k < K;
+       k += (unsigned long long)gridDim.x * blockDim.x) {
+    const unsigned long long key = cand[2 * k], ray = cand[2 * k + 1];
+    unsigned long long rank = 0;
+    for (unsigned long long j = 0; j < K; ++j) {
+      const unsigned long long kj = cand[2 * j], rj = cand[2 * j + 1];
+      rank += (kj < key || (kj == key && rj < ray)) ? 1ull : 0ull;
+    }
+    p.guided[32 + 2 * GUIDED_CAP + rank] = ray;
+    if (rank < (unsigned long long)p.guided_max) p.status[ray] = RAY_EXPRESS;
+  }
+}
+
 __device__ __forceinline__ unsigned sm_id() {
   unsigned r;
   asm volatile("mov.u32 %0, %%smid;" : "=r"(r));
@@ -141,7 +175,7 @@ constexpr int XWAIT_MAX = 1000000;
 
 __global__ void __launch_bounds__(128) trace_fp64_kernel(TraceParams p) {
   const int lane = threadIdx.x & 31;
-  int64_t ray = -1;   // -1: needs a ray, -2: queue exhausted
+  int64_t ray = lane < p.lanes ? -1 : -2;   // -1: needs a ray, -2: queue exhausted
   Lane L;
   long long acc = 0, rej = 0, traced = 0, esc = 0;
   int na0 = 0, nr0 = 0;   // steps a resumed ray had already taken in FP32
@@ -576,6 +610,23 @@ cudaError_t occupancy_batch_fp64(int block, int* occ) {
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, batch_fp64_kernel, block, 0);
 }
 
+cudaError_t launch_guided(TraceParams& p, int64_t warps, cudaStream_t stream) {
+  p.guided_max = 32 * (warps / 4 > 0 ? warps / 4 : 1);
+  int dev = 0, nsm = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  e = cudaMemsetAsync(p.guided, 0, sizeof(unsigned long long), stream);
+  if (e != cudaSuccess) return e;
+  const int64_t need = (p.n + 255) / 256, cap = (int64_t)nsm * 8;
+  guided_select_kernel<<<(unsigned)(need < cap ? (need > 0 ? need : 1) : cap), 256, 0, stream>>>(p);
+  e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  guided_rank_kernel<<<(unsigned)((GUIDED_CAP + 127) / 128), 128, 0, stream>>>(p);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_trace_fp64(const TraceParams& p, int block, int blocks_per_sm,
                               cudaStream_t stream) {
   int dev = 0, nsm = 0;
@@ -593,7 +644,9 @@ cudaError_t launch_trace_fp64(const TraceParams& p, int block, int blocks_per_sm
     if (e != cudaSuccess) return e;
     blocks_per_sm = occ > 0 ? occ : 1;
   }
-  const int64_t warps_needed = (p.n + 31) / 32;
+  TraceParams q = p;
+  q.lanes = spread_lanes(p.n, nsm);
+  const int64_t warps_needed = (p.n + q.lanes - 1) / q.lanes;
   int64_t grid = (int64_t)nsm * blocks_per_sm;
   const int64_t max_useful = (warps_needed * 32 + block - 1) / block;
   if (grid > max_useful) grid = max_useful;
@@ -604,7 +657,6 @@ cudaError_t launch_trace_fp64(const TraceParams& p, int block, int blocks_per_sm
     e = cudaMemsetAsync(p.park_count, 0, 2 * sizeof(unsigned long long), stream);
     if (e != cudaSuccess) return e;
   }
-  TraceParams q = p;
   if (p.xrec) {
     // express lane: select and rank the bucket-0 rays; the persistent launch
     // then traces the rest one lane per ray, parking only when xpark is set

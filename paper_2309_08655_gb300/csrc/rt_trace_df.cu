@@ -15,6 +15,7 @@
 
 #include "rt_df.cuh"
 #include "rt_device.cuh"
+#include "rt_guided.cuh"
 #include "rt_integrator.cuh"
 #include "rt_internal.h"
 
@@ -501,7 +502,9 @@ __device__ __forceinline__ int finish_df(const TraceParams& p, LaneD& L, DF h, D
 
 __global__ void __launch_bounds__(256) trace_df_kernel(TraceParams p) {
   const int lane = threadIdx.x & 31;
-  int64_t ray = -1;
+  int64_t ray = lane < p.lanes ? -1 : -2;
+  const GuidedShare share = guided_share(p);
+  bool guided = share.mine > 0;
   LaneD L;
   long long acc = 0, rej = 0, traced = 0, esc = 0;
   if (p.ts && threadIdx.x == 0) atomicMin(p.ts, global_ns());
@@ -511,9 +514,17 @@ __global__ void __launch_bounds__(256) trace_df_kernel(TraceParams p) {
   // one pass over the rays, or COST_BUCKETS passes (cost-ordered claims: the
   // rays that start nearest the null cone first)
   const int64_t nq = p.order ? (int64_t)COST_BUCKETS * p.n : p.n;
+  if (lane < share.mine) {
+    ray = (int64_t)share.list[share.first + lane * share.stride];
+    load_lane_d(p, ray, L);
+  }
   ClaimChunk ch;
   for (;;) {
-    claim_items(p.queue, nq, p.refill_min, p.claim_size, ray, ch, [&](int64_t idx) -> int64_t {
+    if (guided && __ballot_sync(FULL, ray >= 0) == 0) {   // the share has ended
+      guided = false;
+      ray = lane < p.lanes ? -1 : -2;
+    }
+    if (!guided) claim_items(p.queue, nq, p.refill_min, p.claim_size, ray, ch, [&](int64_t idx) -> int64_t {
       const int pass = p.order ? (int)(idx / p.n) : 0;
       const int64_t i = idx - (int64_t)pass * p.n;
       if (p.status[i] != RAY_READY ||
@@ -579,14 +590,20 @@ cudaError_t launch_trace_df(const TraceParams& p, int block, int blocks_per_sm,
     if (e != cudaSuccess) return e;
     blocks_per_sm = (block >= 128 || occ < 1) ? 1 : (occ < 128 / block ? occ : 128 / block);
   }
-  const int64_t warps_needed = (p.n + 31) / 32;
+  TraceParams q = p;
+  q.lanes = spread_lanes(p.n, nsm);
+  const int64_t warps_needed = (p.n + q.lanes - 1) / q.lanes;
   int64_t grid = (int64_t)nsm * blocks_per_sm;
   const int64_t max_useful = (warps_needed * 32 + block - 1) / block;
   if (grid > max_useful) grid = max_useful;
   if (grid < 1) grid = 1;
   e = cudaMemsetAsync(p.queue, 0, sizeof(unsigned long long), stream);
   if (e != cudaSuccess) return e;
-  trace_df_kernel<<<(unsigned)grid, block, 0, stream>>>(p);
+  if (q.guided) {
+    e = launch_guided(q, grid * (block / 32), stream);
+    if (e != cudaSuccess) return e;
+  }
+  trace_df_kernel<<<(unsigned)grid, block, 0, stream>>>(q);
   return cudaGetLastError();
 }
 

@@ -23,6 +23,7 @@
 #include <stdint.h>
 
 #include "rt_device.cuh"
+#include "rt_guided.cuh"
 #include "rt_integrator.cuh"
 #include "rt_internal.h"
 
@@ -353,13 +354,23 @@ __device__ int advance_rot(const TraceParams& p, RotLane& L) {
 
 __global__ void __launch_bounds__(128) trace_rot_kernel(TraceParams p) {
   const int lane = threadIdx.x & 31;
-  int64_t ray = -1;   // -1: needs a ray, -2: queue exhausted
+  int64_t ray = lane < p.lanes ? -1 : -2;   // -1: needs a ray, -2: queue exhausted
+  const GuidedShare share = guided_share(p);
+  bool guided = share.mine > 0;
   RotLane L;
   long long acc = 0, rej = 0, traced = 0, esc = 0;
   const int64_t nq = p.order ? (int64_t)COST_BUCKETS * p.n : p.n;   // cost-ordered passes
   if (p.ts && threadIdx.x == 0) atomicMin(p.ts, global_ns());
+  if (lane < share.mine) {
+    ray = (int64_t)share.list[share.first + lane * share.stride];
+    load_rot(p, ray, L);
+  }
   for (;;) {
-    const bool need = (ray == -1);
+    if (guided && __ballot_sync(FULL, ray >= 0) == 0) {   // the share has ended
+      guided = false;
+      ray = lane < p.lanes ? -1 : -2;
+    }
+    const bool need = (ray == -1) && !guided;
     const unsigned mneed = __ballot_sync(FULL, need);
     if (mneed) {
       const int leader = __ffs(mneed) - 1;
@@ -432,14 +443,20 @@ cudaError_t launch_trace_rot(const TraceParams& p, int block, int blocks_per_sm,
     if (e != cudaSuccess) return e;
     blocks_per_sm = occ > 0 ? occ : 1;
   }
-  const int64_t warps_needed = (p.n + 31) / 32;
+  TraceParams q = p;
+  q.lanes = spread_lanes(p.n, nsm);
+  const int64_t warps_needed = (p.n + q.lanes - 1) / q.lanes;
   int64_t grid = (int64_t)nsm * blocks_per_sm;
   const int64_t max_useful = (warps_needed * 32 + block - 1) / block;
   if (grid > max_useful) grid = max_useful;
   if (grid < 1) grid = 1;
   e = cudaMemsetAsync(p.queue, 0, sizeof(unsigned long long), stream);
   if (e != cudaSuccess) return e;
-  trace_rot_kernel<<<(unsigned)grid, block, 0, stream>>>(p);
+  if (q.guided) {
+    e = launch_guided(q, grid * (block / 32), stream);
+    if (e != cudaSuccess) return e;
+  }
+  trace_rot_kernel<<<(unsigned)grid, block, 0, stream>>>(q);
   return cudaGetLastError();
 }
 
