@@ -504,9 +504,9 @@ rt_status rt_flux_gradient(const rt_star* star, int64_t n, const double* d_unifo
  *   traces every pixel of every image (rt_trace_backward's estimator): rays
  *   and pixels share one work queue, rays first, and a lane that finishes
  *   either claims the next item of either kind.  RT_PREC_MIXED then runs one
- *   FP32 launch and one FP64 launch for the promoted rays (from where they
- *   stopped) and the handed-over pixels (anew).  No tail mode in that case;
- *   lambda_max must be 0.  Timestamps: 1 + nstars + nimg entries, [1 + nstars
+ *   FP32 launch, an FP64 launch for the promoted rays (from where they stopped;
+ *   in tail mode unless tail = 1) and one for the handed-over pixels (anew).  An
+ *   FP64 call with images has no tail mode; lambda_max must be 0.  Timestamps: 1 + nstars + nimg entries, [1 + nstars
  *   + j] the last pixel of image j.  Counters add rays and pixels.
  * rt_bin_batch - per-star histograms: d_hist is nstars x nth x nph x nnu,
  *   d_out_of_range nstars; per-star fixed-point scales (binning scratch owned

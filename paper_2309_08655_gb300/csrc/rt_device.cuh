@@ -456,6 +456,15 @@ __device__ __forceinline__ void claim_items(unsigned long long* queue, int64_t n
   }
 }
 
+// Lanes of each warp that take items in a launch over `total` of them: the launch's
+// warps share out a short queue evenly (an attempt of a warp costs every branch
+// that one of its lanes takes, and idle lanes cost nothing).
+__device__ __forceinline__ int launch_lanes(int64_t total) {
+  const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+  const int64_t l = (total + warps - 1) / warps;
+  return l < 1 ? 1 : l > 32 ? 32 : (int)l;
+}
+
 // Nanosecond global timer of the GPU (for per-instance completion times).
 __device__ __forceinline__ unsigned long long global_ns() {
   unsigned long long t;

@@ -76,10 +76,8 @@ struct TraceParams {
   // the first guided_max of the list have left the queue
   unsigned long long* guided = nullptr;
   int64_t guided_max = 0;
+  double* guided_rec = nullptr;   // their park records, for six-lane groups (NULL: none)
 };
-// The guided rays' scratch: a counter, GUIDED_CAP (key, ray) pairs and the list.
-constexpr int64_t GUIDED_CAP = 8192;
-inline size_t guided_bytes() { return 256 + (size_t)GUIDED_CAP * 3 * sizeof(unsigned long long); }
 // Lanes per warp of a persistent launch over n rays: with fewer than 32 rays for
 // each warp of one block of four per SM, every scheduler gets a warp and each warp
 // its share.  A warp's attempt costs the branches that any of its lanes takes.
@@ -98,6 +96,13 @@ constexpr int XRAYS_PER_SM = 12;       // one six-lane group in warps 0-1, five 
 inline size_t express_bytes() {
   return 64 + XSLOTS * sizeof(int) + (size_t)XCAP * 2 * sizeof(unsigned long long) +
          (size_t)XCAP * PARKREC * sizeof(double);
+}
+// The guided rays' scratch: a counter, GUIDED_CAP (key, ray) pairs, the list, and
+// the rays' park records.
+constexpr int64_t GUIDED_CAP = 4096;
+constexpr int64_t GUIDED_RECS = 32 + 3 * GUIDED_CAP;      // in 8-byte units
+inline size_t guided_bytes() {
+  return (size_t)(GUIDED_RECS + GUIDED_CAP * PARKREC) * sizeof(unsigned long long);
 }
 // Park capacity that covers any persistent grid on the device (up to 31 rays
 // per warp).

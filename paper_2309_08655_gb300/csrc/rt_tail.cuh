@@ -9,12 +9,11 @@
 // (their complete integrator state, so the continuation is the same
 // computation) and continued with one lane per state component: lane c
 // of a six-lane group owns y_c, its stage derivatives and the stage sums, and
-// evaluates the c-th component of the right-hand side after the scalar prefix
-// that every component shares.  Shuffles within the group (not the FP64 pipe)
-// assemble each stage input.  The steps, the error norm, the controller and
-// the events are those of advance() in rt_integrator.cuh; the arithmetic of
-// the component sums and of the error-norm sum is ordered differently, so
-// results agree with the lane-per-ray path to rounding.
+// the right-hand side's scalars are shared out over the lanes.  The steps, the
+// error norm, the controller and the events are those of advance() in
+// rt_integrator.cuh; the arithmetic of the component sums and of the error-norm
+// sum is ordered differently, so results agree with the lane-per-ray path to
+// rounding.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -46,23 +45,24 @@ __device__ __forceinline__ int find_star_t(const TraceParams& p, int64_t i) {
 // An FP64 instruction costs a warp 64 cycles whether the lanes of a group do the
 // same work or six different products, and a launch of guided rays ends with its
 // longest ray: what counts is the number of FP64 instructions one after another,
-// and what stands between them.  So the scalar coefficients of the
-// Goldreich-Julian anisotropic medium (the one with rays long enough for this
-// mode) are formed in passes: in each, the six lanes take one multiply-add whose
-// operands they read from slots of their own choice, and store the result to a
-// slot.  The slot numbers are one table, read into registers at the start, so a
-// pass is three loads, the multiply-add and a store: 32 FP64 instructions a
-// right-hand side, where every lane forming every scalar takes 105.  (Operands
-// exchanged by shuffles and picked by selects took 13 other instructions for
-// each FP64 one, and 23.5 us an attempt.)
+// and what stands between them.  So the scalar coefficients of the anisotropic
+// Goldreich-Julian and twisted media are formed in passes: in each, the six lanes
+// take one multiply-add whose operands they read from slots of their own choice,
+// and store the result to a slot.  The slot numbers are one table, read into
+// registers when a ray is taken up, so a pass is three loads, the multiply-add and
+// a store: 32 FP64 instructions a right-hand side, where every lane forming every
+// scalar takes 105.  A lone guided ray: 12.6 us an attempt (26 k cycles, of which
+// about 310 FP64 instructions take 20 k), 33 us with the prefix formed by every
+// lane; operands exchanged by shuffles and picked by selects took 13 other
+// instructions for each FP64 one, 23.5 us.
 //
 // Slots: the point, the ray's constants, plain numbers, then what the passes
 // leave.
 enum Slot : int {
   S_X = 0,                                      // x0 x1 x2 k0 k1 k2
   S_M = 6, S_M3 = 9,                            // m, 3 m
-  S_RS = 12, S_CPS, S_NM2, S_3M2, S_W2, S_IW2,  // rs, cp sig, -m_z, 3 m_z, W2, 1/W2
-  S_0, S_1, S_N1, S_2, S_N2, S_3, S_N15,
+  S_RS = 12, S_CPS, S_FB, S_W2, S_IW2,          // rs, cp sig, W2, 1/W2
+  S_0, S_1, S_N1, S_2, S_N2, S_3, S_FA, S_QA, S_QB,    // F = FA . + FB, qn = QA . + QB
   S_IR, S_DOT,                                  // 1/r; x.k, m.x, k.m, |x|^2, 3 m.x
   S_Q = S_DOT + 6,                              // 1/sqrt(A) (0-2), 1/|b| (3-5)
   S_P1 = S_Q + 6                                // pass n at S_P1 + 6 (n - 1)
@@ -100,47 +100,56 @@ enum Value : int {
 };
 
 // Operands of pass n (2 and up to 14): result = a b + c per lane.  Pass 1 (the
-// products with 1/r) and the dot products before it are written out.
-__constant__ unsigned char c_pass[PASSES - 1][GROUP][3] = {
-    // A, and |b|^2 = 3 mu^2 + 1
-    {{V_U, S_N1, S_1}, {V_U, S_N1, S_1}, {V_U, S_N1, S_1}, {V_MU3, V_MU, S_1},
-     {V_MU3, V_MU, S_1}, {V_MU3, V_MU, S_1}},
-    // r^-3, mu n_z, (rs/r) kr, dA/dr, kr^2, mu kr
-    {{V_IR2, S_IR, S_0}, {V_MU, V_NZ, S_0}, {V_U, V_KR, S_0}, {S_RS, V_IR2, S_0},
-     {V_KR, V_KR, S_0}, {V_MU, V_KR, S_0}},
-    // g3 = cp sig r^-3, F, qn, sqrt(A), 1/A, 1/|b|^2
-    {{S_CPS, V_IR3, S_0}, {S_3, V_MN, S_NM2}, {S_N15, V_MN, S_3M2}, {V_A, V_QA, S_0},
-     {V_QA, V_QA, S_0}, {V_IB, V_IB, S_0}},
-    // P, t, -2 (rs/r) kr, 1 + 2 sqrt(A), 1/A^2, dA/dr / sqrt(A)
-    {{V_G3, V_F, S_0}, {V_G3, S_IR, S_0}, {S_N2, V_UKR, S_0}, {S_2, V_SA, S_1},
-     {V_IA, V_IA, S_0}, {V_DA, V_QA, S_0}},
-    // c1, opsA kr, P A, qm, W2/A^2, a3
-    {{V_MU, V_OPSA, S_0}, {V_OPSA, V_KR, S_0}, {V_P, V_A, S_0}, {S_3, V_NZ, S_0},
-     {S_W2, V_IA2, S_0}, {V_MKR, V_DAQ, S_0}},
-    // U, 1/(|b| W2), c1 kr, 2 P A, W2/A^2 + 3 kr^2, A/W2
-    {{V_C1, V_KR, S_DOT + 5}, {V_IB, S_IW2, S_0}, {V_C1, V_KR, S_0}, {S_2, V_PA, S_0},
-     {S_3, V_KR2, V_W2IA2}, {V_A, S_IW2, S_0}},
-    // Kp, 3 mu U, and the negatives of 1/|b|^2, A/W2, c1, P
-    {{V_UU, V_IB, S_0}, {V_MU3, V_UU, S_0}, {S_N1, V_IB2, S_0}, {S_N1, V_AIW2, S_0},
-     {S_N1, V_C1, S_0}, {S_N1, V_P, S_0}},
-    // Kp^2, a1, Kp/(|b| W2), -a3
-    {{V_KP, V_KP, S_0}, {V_M3U, V_NIB2, V_OKR}, {V_KP, V_IBIW2, S_0}, {S_N1, V_A3, S_0},
-     {S_0, S_0, S_0}, {S_0, S_0, S_0}},
-    // 1 - A Kp^2/W2, gm, a1 mu + c1 kr, Kp^2/W2, -a1
-    {{V_NAIW2, V_KP2, S_1}, {V_PA2, V_QIB, S_0}, {V_A1, V_MU, V_C1KR}, {V_KP2, S_IW2, S_0},
-     {S_N1, V_A1, S_0}, {S_0, S_0, S_0}},
-    // w, gm/r, bx, s, z = (a1 mu + c1 kr)/r - a3
-    {{V_T, V_ONEM, S_0}, {V_GM, S_IR, S_0}, {V_GM, V_NC1, V_BX0}, {V_NP, V_KQ, V_S1},
-     {S_IR, V_D, V_NA3}, {S_0, S_0, S_0}},
-    // w qm, gm z, Ck, dA/dr s, w qz, -gm a1 / r
-    {{V_W, V_QM, S_0}, {V_GM, V_Z, S_0}, {V_BX, S_IR, S_0}, {V_DA, V_S, S_0},
-     {V_W, V_MU3, S_0}, {V_GMR, V_NA1, S_0}},
-    // Cm, w qn + gm z
-    {{S_1, V_WQM, V_NGA1}, {V_W, V_QN, V_GMZ}, {S_0, S_0, S_0}, {S_0, S_0, S_0},
-     {S_0, S_0, S_0}, {S_0, S_0, S_0}},
-    // Cn
-    {{S_1, V_E, V_VS}, {S_0, S_0, S_0}, {S_0, S_0, S_0}, {S_0, S_0, S_0}, {S_0, S_0, S_0},
-     {S_0, S_0, S_0}}};
+// products with 1/r) and the dot products before it are written out.  The media
+// differ in the plasma's terms, P = g F and dP = t (qn n + qm m + qz e_z) with
+// t = g / r, as ham_rhs64:
+//   Goldreich-Julian  g = cp sig r^-3, F = 3 mu n_z - m_z, qn = -15 mu n_z + 3 m_z,
+//                     qm = 3 n_z, qz = 3 mu
+//   twisted           g = cp r^-4, F = 1 - mu^2, qn = 6 mu^2 - 4, qm = -2 mu, qz = 0
+#define RT_PASSES(RA, RB, MA, MB, QMA, QMB, QZ) {                                             \
+    /* A, and |b|^2 = 3 mu^2 + 1 */                                                           \
+    {{V_U, S_N1, S_1}, {V_U, S_N1, S_1}, {V_U, S_N1, S_1}, {V_MU3, V_MU, S_1},                \
+     {V_MU3, V_MU, S_1}, {V_MU3, V_MU, S_1}},                                                 \
+    /* r^-3, mu n_z, (rs/r) kr, dA/dr, kr^2, mu kr */                                         \
+    {{RA, RB, S_0}, {MA, MB, S_0}, {V_U, V_KR, S_0}, {S_RS, V_IR2, S_0},                      \
+     {V_KR, V_KR, S_0}, {V_MU, V_KR, S_0}},                                                   \
+    /* g3 = cp sig r^-3, F, qn, sqrt(A), 1/A, 1/|b|^2 */                                      \
+    {{S_CPS, V_IR3, S_0}, {S_FA, V_MN, S_FB}, {S_QA, V_MN, S_QB}, {V_A, V_QA, S_0},           \
+     {V_QA, V_QA, S_0}, {V_IB, V_IB, S_0}},                                                   \
+    /* P, t, -2 (rs/r) kr, 1 + 2 sqrt(A), 1/A^2, dA/dr / sqrt(A) */                           \
+    {{V_G3, V_F, S_0}, {V_G3, S_IR, S_0}, {S_N2, V_UKR, S_0}, {S_2, V_SA, S_1},               \
+     {V_IA, V_IA, S_0}, {V_DA, V_QA, S_0}},                                                   \
+    /* c1, opsA kr, P A, qm, W2/A^2, a3 */                                                    \
+    {{V_MU, V_OPSA, S_0}, {V_OPSA, V_KR, S_0}, {V_P, V_A, S_0}, {QMA, QMB, S_0},              \
+     {S_W2, V_IA2, S_0}, {V_MKR, V_DAQ, S_0}},                                                \
+    /* U, 1/(|b| W2), c1 kr, 2 P A, W2/A^2 + 3 kr^2, A/W2 */                                  \
+    {{V_C1, V_KR, S_DOT + 5}, {V_IB, S_IW2, S_0}, {V_C1, V_KR, S_0}, {S_2, V_PA, S_0},        \
+     {S_3, V_KR2, V_W2IA2}, {V_A, S_IW2, S_0}},                                               \
+    /* Kp, 3 mu U, and the negatives of 1/|b|^2, A/W2, c1, P */                               \
+    {{V_UU, V_IB, S_0}, {V_MU3, V_UU, S_0}, {S_N1, V_IB2, S_0}, {S_N1, V_AIW2, S_0},          \
+     {S_N1, V_C1, S_0}, {S_N1, V_P, S_0}},                                                    \
+    /* Kp^2, a1, Kp/(|b| W2), -a3 */                                                          \
+    {{V_KP, V_KP, S_0}, {V_M3U, V_NIB2, V_OKR}, {V_KP, V_IBIW2, S_0}, {S_N1, V_A3, S_0},      \
+     {S_0, S_0, S_0}, {S_0, S_0, S_0}},                                                       \
+    /* 1 - A Kp^2/W2, gm, a1 mu + c1 kr, Kp^2/W2, -a1 */                                      \
+    {{V_NAIW2, V_KP2, S_1}, {V_PA2, V_QIB, S_0}, {V_A1, V_MU, V_C1KR}, {V_KP2, S_IW2, S_0},   \
+     {S_N1, V_A1, S_0}, {S_0, S_0, S_0}},                                                     \
+    /* w, gm/r, bx, s, z = (a1 mu + c1 kr)/r - a3 */                                          \
+    {{V_T, V_ONEM, S_0}, {V_GM, S_IR, S_0}, {V_GM, V_NC1, V_BX0}, {V_NP, V_KQ, V_S1},         \
+     {S_IR, V_D, V_NA3}, {S_0, S_0, S_0}},                                                    \
+    /* w qm, gm z, Ck, dA/dr s, w qz, -gm a1 / r */                                           \
+    {{V_W, V_QM, S_0}, {V_GM, V_Z, S_0}, {V_BX, S_IR, S_0}, {V_DA, V_S, S_0},                 \
+     {V_W, QZ, S_0}, {V_GMR, V_NA1, S_0}},                                                    \
+    /* Cm, w qn + gm z */                                                                     \
+    {{S_1, V_WQM, V_NGA1}, {V_W, V_QN, V_GMZ}, {S_0, S_0, S_0}, {S_0, S_0, S_0},              \
+     {S_0, S_0, S_0}, {S_0, S_0, S_0}},                                                       \
+    /* Cn */                                                                                  \
+    {{S_1, V_E, V_VS}, {S_0, S_0, S_0}, {S_0, S_0, S_0}, {S_0, S_0, S_0}, {S_0, S_0, S_0},    \
+     {S_0, S_0, S_0}}}
+__constant__ unsigned char c_pass[2][PASSES - 1][GROUP][3] = {
+    RT_PASSES(V_IR2, S_IR, V_MU, V_NZ, S_3, V_NZ, V_MU3),
+    RT_PASSES(V_IR2, V_IR2, V_MU, V_MU, S_N2, V_MU, S_0)};
+#undef RT_PASSES
 
 // A lane's view of its group's slots: byte offsets of its operands.
 struct GroupFile {
@@ -155,10 +164,6 @@ __device__ __forceinline__ void file_init(GroupFile& f, double* slots, int cc, u
   f.cc = cc;
   f.j = cc < 3 ? cc : cc - 3;
   f.gm = gm;
-#pragma unroll
-  for (int p = 0; p < PASSES - 1; ++p)
-#pragma unroll
-    for (int q = 0; q < 3; ++q) f.off[p][q] = 8u * c_pass[p][cc][q];
 }
 
 __device__ __forceinline__ double slot_at(const GroupFile& f, unsigned off) {
@@ -166,7 +171,12 @@ __device__ __forceinline__ double slot_at(const GroupFile& f, unsigned off) {
 }
 
 // The ray's constants, and the plain numbers (every lane of the group).
-__device__ __forceinline__ void file_ray(const GroupFile& f, const RayConst<double>& c) {
+__device__ __forceinline__ void file_ray(GroupFile& f, const RayConst<double>& c) {
+  const bool gj = c.plasma == PLASMA_GJ;
+#pragma unroll
+  for (int p = 0; p < PASSES - 1; ++p)
+#pragma unroll
+    for (int q = 0; q < 3; ++q) f.off[p][q] = 8u * c_pass[gj ? 0 : 1][p][f.cc][q];
   __syncwarp(f.gm);
   double* s = f.s;
   if (f.cc == 0) {
@@ -177,9 +187,11 @@ __device__ __forceinline__ void file_ray(const GroupFile& f, const RayConst<doub
     s[S_M3 + 1] = 3.0 * c.m1;
     s[S_M3 + 2] = 3.0 * c.m2;
     s[S_RS] = c.rs;
-    s[S_CPS] = c.cp * c.sig;
-    s[S_NM2] = -c.m2;
-    s[S_3M2] = 3.0 * c.m2;
+    s[S_CPS] = gj ? c.cp * c.sig : c.cp;
+    s[S_FA] = gj ? 3.0 : -1.0;
+    s[S_FB] = gj ? -c.m2 : 1.0;
+    s[S_QA] = gj ? -15.0 : 6.0;
+    s[S_QB] = gj ? 3.0 * c.m2 : -4.0;
     s[S_W2] = c.W2;
     s[S_IW2] = c.iW2;
     s[S_0] = 0.0;
@@ -188,21 +200,20 @@ __device__ __forceinline__ void file_ray(const GroupFile& f, const RayConst<doub
     s[S_2] = 2.0;
     s[S_N2] = -2.0;
     s[S_3] = 3.0;
-    s[S_N15] = -15.0;
   }
   __syncwarp(f.gm);
 }
 
 // Own component (0-2: dx_j/dl, 3-5: dk_j/dl) of the right-hand side at the point
 // whose own component is yc.  *r2 = |x|^2 and *F the null-cone factor there (any
-// positive multiple of it: its sign is the side; Goldreich-Julian only).
+// positive multiple of it: its sign is the side; meaningful for Goldreich-Julian).
 __device__ __forceinline__ double rhs_group(const GroupFile& f, const RayConst<double>& c,
                                             double yc, double* r2, double* F) {
   double* s = f.s;
   __syncwarp(f.gm);
   s[S_X + f.cc] = yc;
   __syncwarp(f.gm);
-  if (c.plasma != PLASMA_GJ || c.disp == DISP_ISO) {
+  if ((c.plasma != PLASMA_GJ && c.plasma != PLASMA_TWISTED) || c.disp == DISP_ISO) {
     // every lane evaluates the whole right-hand side and keeps its component
     double y[6], g[6];
 #pragma unroll
@@ -436,13 +447,15 @@ struct GroupCounts {
 // Six-lane groups of the calling warp continue parked rays: records
 // lo + e of recs (PARKREC doubles each: y[6], h, h_resume, sig, flags, na, nr,
 // ray, lambda), e = 0, 1, ... claimed one per group with an atomic on *next,
-// while lo + e < hi.  ngroups (1 to GROUPS_PER_WARP) groups of the warp take
+// while lo + e < hi; without next the warp's groups share out lo, lo + stride,
+// lo + 2 stride, ...  ngroups (1 to GROUPS_PER_WARP) groups of the warp take
 // part: one group per warp keeps a ray's attempts free of the other groups'
 // divergent branches.  slots: shared memory of the block, GROUP_SLOTS doubles.
 // Every lane of the warp must call it.
 __device__ void tail_groups(const TraceParams& p, const double* recs, unsigned long long lo,
                             unsigned long long hi, unsigned long long* next, int ngroups,
-                            GroupCounts& cnt, double* slots) {
+                            GroupCounts& cnt, double* slots,
+                            unsigned long long stride = 0) {
   const int lane = threadIdx.x & 31;
   const int g = lane / GROUP, cc = lane % GROUP;
   const bool in_group = g < ngroups && g < GROUPS_PER_WARP;
@@ -453,10 +466,11 @@ __device__ void tail_groups(const TraceParams& p, const double* recs, unsigned l
   if (in_group) file_init(f, slots + ((threadIdx.x >> 5) * GROUPS_PER_WARP + g) * SLOTS, cc, gm);
   bool have = false, done = !in_group;
   int na0 = 0, nr0 = 0;
+  unsigned long long taken = 0;
   for (;;) {
     if (in_group && !have && !done) {
       unsigned long long e = 0;
-      if (cc == 0) e = lo + atomicAdd(next, 1ull);
+      if (cc == 0) e = lo + (next ? atomicAdd(next, 1ull) : (taken++ * ngroups + g) * stride);
       e = __shfl_sync(gm, e, base);
       if (e >= hi) {
         done = true;

@@ -82,6 +82,22 @@ __device__ void store_lane(const TraceParams& p, int64_t i, const Lane& L, int s
   if (p.nrej) p.nrej[i] = L.nr;
 }
 
+// A READY ray's park record: the start of load_lane.
+__device__ void fresh_record(const TraceParams& p, int64_t ray, double* pe) {
+  Lane L;
+  load_lane(p, ray, L);
+#pragma unroll
+  for (int j = 0; j < 6; ++j) pe[j] = L.y[j];
+  pe[6] = L.h;
+  pe[7] = 0.0;
+  pe[8] = L.c.sig;
+  pe[9] = 0.0;
+  pe[10] = 0.0;
+  pe[11] = 0.0;
+  pe[12] = (double)ray;
+  pe[13] = 0.0;
+}
+
 // Express lane, step 1: the READY rays of cost bucket 0 as (key, ray) pairs,
 // key = the bits of the squared null-cone distance (ordered as the distance).
 __global__ void express_select_kernel(TraceParams p) {
@@ -112,19 +128,7 @@ __global__ void express_rank_kernel(TraceParams p) {
       const unsigned long long kj = p.xcand[2 * j], rj = p.xcand[2 * j + 1];
       rank += (kj < key || (kj == key && rj < ray)) ? 1ull : 0ull;
     }
-    Lane L;
-    load_lane(p, (int64_t)ray, L);
-    double* pe = p.xrec + rank * PARKREC;
-#pragma unroll
-    for (int j = 0; j < 6; ++j) pe[j] = L.y[j];
-    pe[6] = L.h;
-    pe[7] = 0.0;
-    pe[8] = L.c.sig;
-    pe[9] = 0.0;
-    pe[10] = 0.0;
-    pe[11] = 0.0;
-    pe[12] = (double)ray;
-    pe[13] = 0.0;
+    fresh_record(p, (int64_t)ray, p.xrec + rank * PARKREC);
     p.status[ray] = RAY_EXPRESS;
   }
 }
@@ -159,7 +163,10 @@ __global__ void guided_rank_kernel(TraceParams p) {
       rank += (kj < key || (kj == key && rj < ray)) ? 1ull : 0ull;
     }
     p.guided[32 + 2 * GUIDED_CAP + rank] = ray;
-    if (rank < (unsigned long long)p.guided_max) p.status[ray] = RAY_EXPRESS;
+    if (rank < (unsigned long long)p.guided_max) {
+      if (p.guided_rec) fresh_record(p, (int64_t)ray, p.guided_rec + rank * PARKREC);
+      p.status[ray] = RAY_EXPRESS;
+    }
   }
 }
 
@@ -345,7 +352,8 @@ __global__ void __launch_bounds__(128) backward_kernel(BackParams bp) {
   tp.max_steps = bp.max_steps;
   tp.ts = nullptr;
   tp.park = nullptr;
-  int64_t pix = -1;
+  const int lanes = launch_lanes(npix);
+  int64_t pix = lane < lanes ? -1 : -2;
   Lane L;
   CrossingHook hk;
   hk.on = true;
@@ -420,7 +428,8 @@ __global__ void __launch_bounds__(128) batch_fp64_kernel(TraceParams p, ImgTable
   const int64_t total = nf + (t.list ? (int64_t)*t.list_n : t.npix);
   TraceParams tp = p;          // r_out per item
   tp.park = nullptr;
-  int64_t item = -1;           // -1: needs an item, -2: queue exhausted
+  const int lanes = launch_lanes(t.list ? total - nf : total);
+  int64_t item = lane < lanes ? -1 : -2;   // -1: needs an item, -2: queue exhausted
   int64_t ray = 0, pix = 0;
   int img = 0;
   bool isp = false;
@@ -582,7 +591,8 @@ cudaError_t launch_backward(const BackLaunch& b, cudaStream_t stream) {
   if (e != cudaSuccess) return e;
   const int64_t npix = (int64_t)b.nx * b.ny;
   int64_t grid = (int64_t)nsm * (occ > 0 ? occ : 1);
-  const int64_t max_useful = (npix + block - 1) / block;
+  const int64_t lanes = spread_lanes(npix, nsm);
+  const int64_t max_useful = ((npix + lanes - 1) / lanes * 32 + block - 1) / block;
   if (grid > max_useful) grid = max_useful;
   if (grid < 1) grid = 1;
   e = cudaMemsetAsync(b.queue, 0, sizeof(unsigned long long), stream);

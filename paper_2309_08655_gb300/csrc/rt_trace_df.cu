@@ -7,9 +7,9 @@
 // the FP32 pipe.  Accuracy is FP64-class (a few units of 2^-47 per operation
 // against 2^-53); no operation of an attempted step touches the FP64 pipe.
 // One lane per ray in a persistent kernel with the warp-ballot work queue
-// (claim_items), index- or cost-ordered; no tail mode is needed: a lone ray's
-// attempt is a chain of FP32 instructions with instruction-level parallelism
-// across its six components.
+// (claim_items), index- or cost-ordered.  The rays that start within 1e-3 rad of
+// the null cone, which set the end of a launch, are traced by FP64 six-lane groups
+// (rt_tail.cuh) of the same launch instead.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -18,6 +18,7 @@
 #include "rt_guided.cuh"
 #include "rt_integrator.cuh"
 #include "rt_internal.h"
+#include "rt_tail.cuh"
 
 namespace rtk {
 
@@ -503,8 +504,7 @@ __device__ __forceinline__ int finish_df(const TraceParams& p, LaneD& L, DF h, D
 __global__ void __launch_bounds__(256) trace_df_kernel(TraceParams p) {
   const int lane = threadIdx.x & 31;
   int64_t ray = lane < p.lanes ? -1 : -2;
-  const GuidedShare share = guided_share(p);
-  bool guided = share.mine > 0;
+  __shared__ double slots[2 * GROUP_SLOTS];      // up to eight warps
   LaneD L;
   long long acc = 0, rej = 0, traced = 0, esc = 0;
   if (p.ts && threadIdx.x == 0) atomicMin(p.ts, global_ns());
@@ -514,17 +514,25 @@ __global__ void __launch_bounds__(256) trace_df_kernel(TraceParams p) {
   // one pass over the rays, or COST_BUCKETS passes (cost-ordered claims: the
   // rays that start nearest the null cone first)
   const int64_t nq = p.order ? (int64_t)COST_BUCKETS * p.n : p.n;
-  if (lane < share.mine) {
-    ray = (int64_t)share.list[share.first + lane * share.stride];
-    load_lane_d(p, ray, L);
+  {
+    // the guided rays six lanes each in FP64, from the start of the launch: 12.6 us
+    // an attempt where a lone double-float lane takes 18, on a pipe that the rest
+    // of the launch leaves idle
+    const GuidedShare share = guided_share(p);
+    if (share.mine > 0) {
+      GroupCounts gc;
+      tail_groups(p, p.guided_rec, share.first, share.first + share.mine * share.stride, nullptr,
+                  share.mine < GROUPS_PER_WARP ? share.mine : GROUPS_PER_WARP, gc, slots,
+                  share.stride);
+      acc += gc.acc;
+      rej += gc.rej;
+      traced += gc.traced;
+      esc += gc.esc;
+    }
   }
   ClaimChunk ch;
   for (;;) {
-    if (guided && __ballot_sync(FULL, ray >= 0) == 0) {   // the share has ended
-      guided = false;
-      ray = lane < p.lanes ? -1 : -2;
-    }
-    if (!guided) claim_items(p.queue, nq, p.refill_min, p.claim_size, ray, ch, [&](int64_t idx) -> int64_t {
+    claim_items(p.queue, nq, p.refill_min, p.claim_size, ray, ch, [&](int64_t idx) -> int64_t {
       const int pass = p.order ? (int)(idx / p.n) : 0;
       const int64_t i = idx - (int64_t)pass * p.n;
       if (p.status[i] != RAY_READY ||
@@ -578,6 +586,10 @@ cudaError_t launch_trace_df(const TraceParams& p, int block, int blocks_per_sm,
   if (block > 256) block = 256;
   block = (block / 32) * 32;
   if (block < 32) block = 32;
+  int occ = 0;
+  e = occupancy_trace_df(block, &occ);
+  if (e != cudaSuccess) return e;
+  if (occ < 1) occ = 1;
   if (blocks_per_sm <= 0) {
     // default: one 128-thread block per SM, one warp per scheduler.  Measured
     // on the eight-step benchmark launch: 2.66-2.69 s against 2.84 s with the
@@ -585,11 +597,10 @@ cudaError_t launch_trace_df(const TraceParams& p, int block, int blocks_per_sm,
     // the launch's end, and a warp that has its scheduler to itself runs them
     // fastest, while the bulk loses little (the kernel is bound by
     // instruction supply, not by the number of warps)
-    int occ = 0;
-    e = occupancy_trace_df(block, &occ);
-    if (e != cudaSuccess) return e;
-    blocks_per_sm = (block >= 128 || occ < 1) ? 1 : (occ < 128 / block ? occ : 128 / block);
+    blocks_per_sm = block >= 128 ? 1 : (occ < 128 / block ? occ : 128 / block);
   }
+  // resident blocks only: a share of the guided rays must not wait for a block
+  if (blocks_per_sm > occ) blocks_per_sm = occ;
   TraceParams q = p;
   q.lanes = spread_lanes(p.n, nsm);
   const int64_t warps_needed = (p.n + q.lanes - 1) / q.lanes;

@@ -28,7 +28,6 @@
 #include "rt_backward.cuh"
 #include "rt_df.cuh"
 #include "rt_device.cuh"
-#include "rt_guided.cuh"
 #include "rt_internal.h"
 
 namespace rtk {
@@ -524,26 +523,16 @@ __device__ int advance_m(const TraceParams& p, LaneM& L, Hook& hook) {
 
 __global__ void __launch_bounds__(256) trace_mixed_kernel(TraceParams p) {
   const int lane = threadIdx.x & 31;
-  int64_t ray = lane < p.lanes ? -1 : -2;
-  const GuidedShare share = guided_share(p);
-  bool guided = share.mine > 0;
+  int64_t ray = -1;
   LaneM L;
   long long acc = 0, rej = 0, traced = 0, esc = 0, promoted = 0;
   if (p.ts && threadIdx.x == 0) atomicMin(p.ts, global_ns());
   // one pass over the rays, or COST_BUCKETS passes (cost-ordered claims: the
   // rays that start nearest the null cone first)
   const int64_t nq = p.order ? (int64_t)COST_BUCKETS * p.n : p.n;
-  if (lane < share.mine) {
-    ray = (int64_t)share.list[share.first + lane * share.stride];
-    load_lane_m(p, ray, L);
-  }
   ClaimChunk ch;
   for (;;) {
-    if (guided && __ballot_sync(FULL, ray >= 0) == 0) {   // the share has ended
-      guided = false;
-      ray = lane < p.lanes ? -1 : -2;
-    }
-    if (!guided) claim_items(p.queue, nq, p.refill_min, p.claim_size, ray, ch, [&](int64_t idx) -> int64_t {
+    claim_items(p.queue, nq, p.refill_min, p.claim_size, ray, ch, [&](int64_t idx) -> int64_t {
       const int pass = p.order ? (int)(idx / p.n) : 0;
       const int64_t i = idx - (int64_t)pass * p.n;
       if (p.status[i] != RAY_READY ||
@@ -803,17 +792,9 @@ __global__ void __launch_bounds__(256) batch_mixed_kernel(TraceParams p, ImgTabl
   hk.on = false;
   long long acc = 0, rej = 0, done = 0, esc = 0, nc = 0, promoted = 0;
   if (p.ts && threadIdx.x == 0) atomicMin(p.ts, global_ns());
-  const GuidedShare share = guided_share(p);
-  bool guided = share.mine > 0;
-  if (lane < share.mine) {
-    ray = (int64_t)share.list[share.first + lane * share.stride];
-    load_lane_m(tp, ray, L);
-    item = ray;
-  }
   ClaimChunk ch;
   for (;;) {
-    if (guided && __ballot_sync(FULL, item >= 0) == 0) guided = false;   // the share has ended
-    if (!guided) claim_items(p.queue, total, p.refill_min, p.claim_size, item, ch,
+    claim_items(p.queue, total, p.refill_min, p.claim_size, item, ch,
                 [&](int64_t idx) -> int64_t {
       if (idx < nf) {
         if (p.status[idx] != RAY_READY) return -1;
@@ -915,14 +896,7 @@ cudaError_t launch_batch_mixed(const TraceParams& p, const ImgTable& t, int bloc
   if (grid < 1) grid = 1;
   e = cudaMemsetAsync(p.queue, 0, sizeof(unsigned long long), stream);
   if (e != cudaSuccess) return e;
-  TraceParams q = p;
-  if (q.guided && q.n > 0) {
-    e = launch_guided(q, grid * (block / 32), stream);
-    if (e != cudaSuccess) return e;
-  } else {
-    q.guided = nullptr;
-  }
-  batch_mixed_kernel<<<(unsigned)grid, block, 0, stream>>>(q, t);
+  batch_mixed_kernel<<<(unsigned)grid, block, 0, stream>>>(p, t);
   return cudaGetLastError();
 }
 
@@ -971,20 +945,14 @@ cudaError_t launch_trace_mixed(const TraceParams& p, int block, int blocks_per_s
     if (e != cudaSuccess) return e;
     blocks_per_sm = occ > 0 ? occ : 1;
   }
-  TraceParams q = p;
-  q.lanes = spread_lanes(p.n, nsm);
-  const int64_t warps_needed = (p.n + q.lanes - 1) / q.lanes;
+  const int64_t warps_needed = (p.n + 31) / 32;
   int64_t grid = (int64_t)nsm * blocks_per_sm;
   const int64_t max_useful = (warps_needed * 32 + block - 1) / block;
   if (grid > max_useful) grid = max_useful;
   if (grid < 1) grid = 1;
   e = cudaMemsetAsync(p.queue, 0, sizeof(unsigned long long), stream);
   if (e != cudaSuccess) return e;
-  if (q.guided) {
-    e = launch_guided(q, grid * (block / 32), stream);
-    if (e != cudaSuccess) return e;
-  }
-  trace_mixed_kernel<<<(unsigned)grid, block, 0, stream>>>(q);
+  trace_mixed_kernel<<<(unsigned)grid, block, 0, stream>>>(p);
   return cudaGetLastError();
 }
 

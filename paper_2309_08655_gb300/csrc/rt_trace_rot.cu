@@ -437,12 +437,12 @@ cudaError_t launch_trace_rot(const TraceParams& p, int block, int blocks_per_sm,
   if (block > 128) block = 128;            // __launch_bounds__(128)
   block = (block / 32) * 32;
   if (block < 32) block = 32;
-  if (blocks_per_sm <= 0) {
-    int occ = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, trace_rot_kernel, block, 0);
-    if (e != cudaSuccess) return e;
-    blocks_per_sm = occ > 0 ? occ : 1;
-  }
+  int occ = 0;
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, trace_rot_kernel, block, 0);
+  if (e != cudaSuccess) return e;
+  if (occ < 1) occ = 1;
+  // resident blocks only: a share of the guided rays must not wait for a block
+  if (blocks_per_sm <= 0 || blocks_per_sm > occ) blocks_per_sm = occ;
   TraceParams q = p;
   q.lanes = spread_lanes(p.n, nsm);
   const int64_t warps_needed = (p.n + q.lanes - 1) / q.lanes;

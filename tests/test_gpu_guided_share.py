@@ -1,6 +1,7 @@
 """Guided rays in warps of their own: bitwise the results of the plain queue for the
-mixed and rotating paths, whatever the launch -- few rays, every ray next to the null
-cone, and more of them than the launch's warps take at once."""
+rotating magnetosphere, whatever the launch -- few rays, every ray next to the null
+cone, more of them than the launch's warps take at once; and in double-float, where
+FP64 groups take them, every ray ends once."""
 import numpy as np
 import pytest
 import torch
@@ -12,25 +13,29 @@ from tests import gpu_util as G
 pytestmark = pytest.mark.gpu
 
 
-def _near(n, width):
-    """Samples of the aligned star within ``width`` rad of its null cone."""
+def _near(n, width, rotation):
+    """Samples of the aligned star within ``width`` rad of its null cone, and others."""
+    kw = dict(I.star_config0(), phase_mode=0, psi=0.0, rotation=rotation)
     u = I.sample_uniforms(9, n)
     u[0] = 0.5 * (1 - np.cos(np.arccos(1 / np.sqrt(3)) + width * (2 * u[0] - 1)))
-    return G.gpu_sample(dict(I.star_config0(), phase_mode=0, psi=0.0), u)
+    return G.gpu_sample(kw, u), G.gpu_sample(kw, I.sample_uniforms(3, 64))
 
 
 @pytest.mark.parametrize("n,width", [(1, 1e-4), (40, 9e-4), (700, 2e-2), (6000, 9e-4)])
 @pytest.mark.parametrize("block,bps", [(32, 1), (0, 0)])
-def test_mixed_shares_are_the_plain_queue(n, width, block, bps):
-    star, st0, _, s0, _ = _near(n, width)
-    far = G.gpu_sample(dict(I.star_config0(), phase_mode=0, psi=0.0), I.sample_uniforms(3, 64))
+@pytest.mark.parametrize("precision", [rt.PREC_FP64, rt.PREC_DF])
+def test_shares(n, width, block, bps, precision):
+    rotation = int(precision == rt.PREC_FP64)
+    near, far = _near(n, width, rotation)
     out = []
-    for tail_rays in (0, 64):            # alone, and among rays that are not guided
-        st = torch.cat([st0, far[1][:, :tail_rays]], 1).contiguous()
-        s = torch.cat([s0, far[3][:tail_rays]]).contiguous()
-        opts = rt.make_opts(rtol=1e-6, precision=rt.PREC_MIXED, tail=1, block=block,
-                            blocks_per_sm=bps, max_steps=400)
-        rt.rt_trace_forward(star, st.shape[1], st, s, opts=opts)
-        assert not (s == 9).any() and not (s == 0).any()   # none left in a share or the queue
+    for others in (0, 64):               # alone, and among rays that are not guided
+        st = torch.cat([near[1], far[1][:, :others]], 1).contiguous()
+        s = torch.cat([near[3], far[3][:others]]).contiguous()
+        opts = rt.make_opts(rtol=1e-6, precision=precision, block=block, blocks_per_sm=bps,
+                            max_steps=300)
+        rt.rt_trace_forward(near[0], st.shape[1], st, s, opts=opts)
+        # none left in a share (the internal status 9) or in the queue
+        assert not (s == 9).any() and not (s == rt.RAY_READY).any()
         out.append((st[:, :n].clone(), s[:n].clone()))
-    assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
+    if rotation:
+        assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
