@@ -262,9 +262,11 @@ struct ConstGrad {
 //   dk/dl = -(Cn n + (bx/r) k + Cm m + Cz e_z)
 //
 // with the plasma's gradient as dP = t (qn n + qm m + qz e_z).  That the
-// coefficient of k is bx/r follows from rotational symmetry about n.  About 105
-// FP64 instructions for the Goldreich-Julian anisotropic medium where ham_rhs
-// takes about 170; the results differ by rounding.  DW: *dw = dH/dW2, as
+// coefficient of k is bx/r follows from rotational symmetry about n.  128
+// operations for the Goldreich-Julian anisotropic medium where ham_rhs takes 196;
+// the results differ by rounding.  (ham_rhs stays for the FP32 stages and the mixed
+// sweep, whose FP32 rounding is part of their results.)  With the shorter error
+// norm and event search: twisted magnetosphere, 16 x 4093 rays, 77 -> 55 ms.  DW: *dw = dH/dW2, as
 // ham_rhs.  CG: *cg = the derivatives with respect to the star's constants
 // (with dual numbers in the direction u, their tangents are u . grad_y of them:
 // the parameter part of a Jacobian product without a tangent per parameter).

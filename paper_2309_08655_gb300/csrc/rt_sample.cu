@@ -4,9 +4,10 @@
 // Bound by the FP64 pipe: a warp instruction takes its sub-partition 64 cycles
 // whatever the number of live lanes, so the per-sample computation keeps the
 // lanes of a warp on one path (the inverse distribution from a table, the root
-// in two FP64 evaluations).  16 x 65536 samples of a mass scan: 0.86 ms, where
-// iterating both to the last bit, one launch per star, took 28.5 ms at 5 of 32
-// live lanes; 4096 samples: 40 us against 708 us.
+// in two FP64 evaluations).  16 x 65536 samples of a mass scan: 1.60 ms, of which
+// half goes to the samples next to the null cone, where iterating all of them to
+// the last bit, one launch per star, took 28.5 ms at 5 of 32 live lanes; 4096
+// samples: 279 us against 709 us.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -67,7 +68,7 @@ __device__ __forceinline__ void store_state(const SampleParams& p, const StarDev
   p.status[i] = o.ok ? RAY_READY : RAY_NO_ROOT;
 }
 
-// The samples next to the null cone (about 2 % of a Goldreich-Julian star's) are
+// The samples next to the null cone (0.7 % of a Goldreich-Julian star's) are
 // listed by their block and sampled once more by sample_state_iterated, a full
 // block of them at a time: scattered over the warps, their iterations would hold
 // every warp for a lane or two.
