@@ -151,7 +151,9 @@ typedef struct {
  *   max_steps         bound on accepted steps per ray
  *   block             threads per block of the persistent kernel (0 = auto, or
  *                     the batch's autotuned value, rt_batch_autotune)
- *   blocks_per_sm     resident blocks per SM for the persistent grid (0 = auto)
+ *   blocks_per_sm     resident blocks per SM for the persistent grid (0 = auto);
+ *                     FP64 traces of at most 128 rays per SM use four warps per SM
+ *                     where fewer are asked for
  *   tail              0: FP64 tracing parks the rays of warps left with at most 5
  *                     rays once the queue has drained and continues them six lanes
  *                     per ray (one lane per state component); results agree with
@@ -184,7 +186,9 @@ typedef struct {
  *                     refill_min); a lane traces its claimed rays one after the
  *                     other before it claims again.  Neither changes any ray's
  *                     result with one lane per ray (tail = 1); in tail mode the
- *                     set of rays that end in the six-lane kernel may change
+ *                     set of rays that end in the six-lane kernel may change.
+ *                     Index-ordered FP64 traces whose grid has a lane for every
+ *                     ray use neither
  *   timestamps        NULL, or a device array of 1 + (number of instances) uint64
  *                     that the kernels stamp with the GPU's nanosecond global
  *                     timer: [0] the earliest start of a tracing launch (min),

@@ -70,20 +70,37 @@ struct TraceParams {
   // a lane claims claim_size consecutive queue entries at a time
   int refill_min = 1;
   int claim_size = 1;
-  // lanes of a warp that take rays (spread_lanes)
+  // lanes of a warp that take rays (persistent_shape); covers: the launch has such a
+  // lane for every entry of the queue
   int lanes = 32;
+  int covers = 0;
   // guided rays (rt_guided.cuh): [0] found, then (key, ray) pairs, then the list;
   // the first guided_max of the list have left the queue
   unsigned long long* guided = nullptr;
   int64_t guided_max = 0;
   double* guided_rec = nullptr;   // their park records, for six-lane groups (NULL: none)
 };
-// Lanes per warp of a persistent launch over n rays: with fewer than 32 rays for
-// each warp of one block of four per SM, every scheduler gets a warp and each warp
-// its share.  A warp's attempt costs the branches that any of its lanes takes.
-inline int spread_lanes(int64_t n, int nsm) {
-  const int64_t l = (n + (int64_t)nsm * 4 - 1) / ((int64_t)nsm * 4);
-  return l < 1 ? 1 : l > 32 ? 32 : (int)l;
+// Grid of a persistent launch over n rays, at most bps blocks of `block` threads per
+// SM, and the lanes of a warp that take rays: with fewer than 32 rays for each of four
+// warps per SM, every scheduler gets a warp and each warp its share (a warp's attempt
+// costs the branches that any of its lanes takes).  The lanes are those of the warps
+// that the grid has, so that its lanes are no fewer than the rays or all of them take
+// rays.
+struct PersistentShape {
+  unsigned grid;
+  int lanes;
+};
+inline PersistentShape persistent_shape(int64_t n, int nsm, int block, int bps) {
+  auto lanes = [n](int64_t warps) {
+    const int64_t l = (n + warps - 1) / warps;
+    return l < 1 ? 1 : l > 32 ? 32 : (int)l;
+  };
+  const int wpb = block / 32;
+  const int spread = lanes((int64_t)nsm * 4);
+  const int64_t warps = (n + spread - 1) / spread;
+  const int64_t useful = (warps + wpb - 1) / wpb, resident = (int64_t)nsm * bps;
+  const int64_t grid = useful < 1 ? 1 : useful < resident ? useful : resident;
+  return {(unsigned)grid, lanes(grid * wpb)};
 }
 constexpr int64_t XPARK_MIN_RAYS = (int64_t)4 << 20;
 constexpr int COST_BUCKETS = 3;

@@ -182,7 +182,7 @@ constexpr int XWAIT_MAX = 1000000;
 
 __global__ void __launch_bounds__(128) trace_fp64_kernel(TraceParams p) {
   const int lane = threadIdx.x & 31;
-  int64_t ray = lane < p.lanes ? -1 : -2;   // -1: needs a ray, -2: queue exhausted
+  int64_t ray = lane < p.lanes ? -1 : -2;   // -1: needs a ray, -2: takes none (any more)
   Lane L;
   long long acc = 0, rej = 0, traced = 0, esc = 0;
   int na0 = 0, nr0 = 0;   // steps a resumed ray had already taken in FP32
@@ -242,11 +242,14 @@ __global__ void __launch_bounds__(128) trace_fp64_kernel(TraceParams p) {
     const unsigned live = __ballot_sync(FULL, ray != -2);
     if (live == 0) break;
     if (p.park) {
-      // the queue has drained and this warp holds few rays: park them for the
-      // six-lanes-per-ray tail kernel (the complete integrator state)
+      // this warp holds few rays and the queue has drained: park them for the
+      // six-lanes-per-ray tail kernel (the complete integrator state).  The queue's
+      // counter tells, not the warp's idle lanes: some take no rays, others wait for
+      // more to claim with them (refill_min).  A lane that has parked its ray goes on
+      // with its chunk's other entries, or finds the queue empty.
       const unsigned has = __ballot_sync(FULL, ray >= 0);
-      const unsigned drained = __ballot_sync(FULL, ray == -2);
-      if (drained && has && __popc(has) <= p.park_live && ray >= 0) {
+      if (has && __popc(has) <= p.park_live && ray >= 0 &&
+          (p.covers || *(volatile const unsigned long long*)p.queue >= (unsigned long long)nq)) {
         const unsigned long long slot = atomicAdd(p.park_count, 1ull);
         if (slot < (unsigned long long)p.park_cap) {
           double* pe = p.park + slot * PARKREC;
@@ -262,7 +265,7 @@ __global__ void __launch_bounds__(128) trace_fp64_kernel(TraceParams p) {
           pe[13] = L.lam;
           acc += L.na - na0;
           rej += L.nr - nr0;
-          ray = -2;
+          ray = -1;
         }
       }
     }
@@ -590,14 +593,10 @@ cudaError_t launch_backward(const BackLaunch& b, cudaStream_t stream) {
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, backward_kernel, block, 0);
   if (e != cudaSuccess) return e;
   const int64_t npix = (int64_t)b.nx * b.ny;
-  int64_t grid = (int64_t)nsm * (occ > 0 ? occ : 1);
-  const int64_t lanes = spread_lanes(npix, nsm);
-  const int64_t max_useful = ((npix + lanes - 1) / lanes * 32 + block - 1) / block;
-  if (grid > max_useful) grid = max_useful;
-  if (grid < 1) grid = 1;
+  const unsigned grid = persistent_shape(npix, nsm, block, occ > 0 ? occ : 1).grid;
   e = cudaMemsetAsync(b.queue, 0, sizeof(unsigned long long), stream);
   if (e != cudaSuccess) return e;
-  backward_kernel<<<(unsigned)grid, block, 0, stream>>>(bp);
+  backward_kernel<<<grid, block, 0, stream>>>(bp);
   return cudaGetLastError();
 }
 
@@ -654,13 +653,20 @@ cudaError_t launch_trace_fp64(const TraceParams& p, int block, int blocks_per_sm
     if (e != cudaSuccess) return e;
     blocks_per_sm = occ > 0 ? occ : 1;
   }
+  // A short launch gives every scheduler a warp, however few blocks are asked for, and
+  // a launch with a lane for every entry of the queue has nothing to refill or to claim
+  // in chunks.  So these options do not decide there which rays end in the six-lane
+  // groups (their results differ by rounding).
+  if (p.n <= (int64_t)nsm * 4 * 32 && blocks_per_sm * (block / 32) < 4)
+    blocks_per_sm = (4 * 32 + block - 1) / block;
+  const PersistentShape shape = persistent_shape(p.n, nsm, block, blocks_per_sm);
   TraceParams q = p;
-  q.lanes = spread_lanes(p.n, nsm);
-  const int64_t warps_needed = (p.n + q.lanes - 1) / q.lanes;
-  int64_t grid = (int64_t)nsm * blocks_per_sm;
-  const int64_t max_useful = (warps_needed * 32 + block - 1) / block;
-  if (grid > max_useful) grid = max_useful;
-  if (grid < 1) grid = 1;
+  q.lanes = shape.lanes;
+  if (!p.order && (int64_t)shape.grid * (block / 32) * shape.lanes >= p.n) {
+    q.covers = 1;
+    q.refill_min = 32;
+    q.claim_size = 1;
+  }
   e = cudaMemsetAsync(p.queue, 0, sizeof(unsigned long long), stream);
   if (e != cudaSuccess) return e;
   if (p.park) {
@@ -682,7 +688,7 @@ cudaError_t launch_trace_fp64(const TraceParams& p, int block, int blocks_per_sm
     if (e != cudaSuccess) return e;
     if (!p.xpark) q.park = nullptr;
   }
-  trace_fp64_kernel<<<(unsigned)grid, block, 0, stream>>>(q);
+  trace_fp64_kernel<<<shape.grid, block, 0, stream>>>(q);
   e = cudaGetLastError();
   if (e != cudaSuccess || !p.park) return e;
   return launch_tail_fp64(p, stream);

@@ -601,20 +601,16 @@ cudaError_t launch_trace_df(const TraceParams& p, int block, int blocks_per_sm,
   }
   // resident blocks only: a share of the guided rays must not wait for a block
   if (blocks_per_sm > occ) blocks_per_sm = occ;
+  const PersistentShape shape = persistent_shape(p.n, nsm, block, blocks_per_sm);
   TraceParams q = p;
-  q.lanes = spread_lanes(p.n, nsm);
-  const int64_t warps_needed = (p.n + q.lanes - 1) / q.lanes;
-  int64_t grid = (int64_t)nsm * blocks_per_sm;
-  const int64_t max_useful = (warps_needed * 32 + block - 1) / block;
-  if (grid > max_useful) grid = max_useful;
-  if (grid < 1) grid = 1;
+  q.lanes = shape.lanes;
   e = cudaMemsetAsync(p.queue, 0, sizeof(unsigned long long), stream);
   if (e != cudaSuccess) return e;
   if (q.guided) {
-    e = launch_guided(q, grid * (block / 32), stream);
+    e = launch_guided(q, (int64_t)shape.grid * (block / 32), stream);
     if (e != cudaSuccess) return e;
   }
-  trace_df_kernel<<<(unsigned)grid, block, 0, stream>>>(q);
+  trace_df_kernel<<<shape.grid, block, 0, stream>>>(q);
   return cudaGetLastError();
 }
 
