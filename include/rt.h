@@ -292,10 +292,10 @@ rt_status rt_sample_conversion_surface_part(const rt_star* star, int64_t n, int6
  * operation in double-float arithmetic on the FP32 pipe (a value is the sum
  * of two floats, ~48 significant bits; an FP64 operation on this GPU issues
  * at 1/64 of the FP32 rate): FP64-class results at a fraction of the cost;
- * one lane per ray (tail ignored), except that the rays which start within 1e-3
- * rad of the Goldreich-Julian null cone (up to 4096 per call, nearest first, in
- * any claim order) are traced in FP64 six lanes per ray from the start of the
- * launch; the handle owns their list (0.6 MB, allocated on first use).
+ * one lane per ray (tail ignored), except that every ray which starts within 1e-3
+ * rad of the Goldreich-Julian null cone is traced in FP64 six lanes per ray from the
+ * start of the launch, in any claim order.  A ray's result depends on its own start
+ * and the tolerances alone: not on the other rays, the launch or the run.
  * claim_order honoured; lambda_max must be 0; not for rotating stars.
  * Calls sharing one handle must be serialised on one stream (the handle owns
  * the work-queue counter).

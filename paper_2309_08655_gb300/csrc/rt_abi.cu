@@ -115,7 +115,6 @@ struct rt_star {
   rtk::StarDev h;               // host copy of the descriptor
   rtk::StarDev* d = nullptr;    // device copy
   unsigned long long* d_queue = nullptr;  // trace work-queue counter (scratch)
-  unsigned long long* d_guided = nullptr; // guided rays (rt_guided.cuh; on first use)
   long long* d_bins = nullptr;  // binning accumulator (scratch)
   size_t bins_cap = 0;
   int device = 0;
@@ -227,7 +226,6 @@ void rt_destroy_star(rt_star* s) {
   if (s->d_bins) cudaFree(s->d_bins);
   if (s->d_queue) cudaFree(s->d_queue);
   if (s->d_park) cudaFree(s->d_park);
-  if (s->d_guided) cudaFree(s->d_guided);
   if (s->d_promo) cudaFree(s->d_promo);
   if (cur != s->device) cudaSetDevice(cur);
   delete s;
@@ -332,24 +330,6 @@ static void set_express(rtk::TraceParams& p) {
   p.xpark = (p.n >= rtk::XPARK_MIN_RAYS) ? 1 : 0;
 }
 
-// The guided rays' scratch (0.6 MB), allocated on first use; a call without it (its
-// first one captured into a graph, or no memory left) claims from the plain queue.
-static void set_guided(rtk::TraceParams& p, unsigned long long** buf, const rt_trace_opts* o,
-                       cudaStream_t stream) {
-  if (!*buf) {
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    void* g = nullptr;
-    if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone ||
-        cudaMalloc(&g, rtk::guided_bytes()) != cudaSuccess) {
-      cudaGetLastError();
-      return;
-    }
-    *buf = (unsigned long long*)g;
-  }
-  p.guided = *buf;
-  if (o->precision == RT_PREC_DF) p.guided_rec = (double*)(*buf + rtk::GUIDED_RECS);
-}
-
 static rt_status check_opts(const rt_trace_opts* o) {
   if (!o) return fail(RT_EINVAL, "opts is NULL");
   if (!(o->rtol > 0 && o->rtol < 1) || !(o->atol > 0 && o->atol < 1))
@@ -422,8 +402,6 @@ rt_status rt_trace_forward(const rt_star* s, int64_t n, double* d_state, uint8_t
   p.nrej = d_nrej;
   p.counters = d_counters;
   p.queue = s->d_queue;
-  if (o->precision == RT_PREC_DF || rigid)
-    set_guided(p, &const_cast<rt_star*>(s)->d_guided, o, (cudaStream_t)stream);
   p.ts = (unsigned long long*)o->timestamps;
   if (o->tail != 1 && o->lambda_max == 0.0 && !rigid && o->precision != RT_PREC_DF) {
     rt_star* sm = const_cast<rt_star*>(s);
@@ -883,7 +861,6 @@ struct rt_batch {
   rtk::StarDev* d_stars = nullptr;    // device table
   int64_t* d_off = nullptr;           // device offsets
   unsigned long long* d_queue = nullptr;
-  unsigned long long* d_guided = nullptr;  // guided rays (rt_guided.cuh; on first use)
   long long* d_bins = nullptr;        // nstars x per-star binning accumulators
   size_t bins_per_star = 0;
   int device = 0;
@@ -967,7 +944,6 @@ void rt_destroy_batch(rt_batch* b) {
   if (b->d_bins) cudaFree(b->d_bins);
   if (b->d_queue) cudaFree(b->d_queue);
   if (b->d_park) cudaFree(b->d_park);
-  if (b->d_guided) cudaFree(b->d_guided);
   if (b->d_img_block) cudaFree(b->d_img_block);
   if (cur != b->device) cudaSetDevice(cur);
   delete b;
@@ -1145,8 +1121,6 @@ rt_status rt_trace_batch(rt_batch* b, double* d_state, uint8_t* d_status, int32_
   p.nrej = d_nrej;
   p.counters = d_counters;
   p.queue = b->d_queue;
-  if (o->precision == RT_PREC_DF || b->rigid)
-    set_guided(p, &b->d_guided, o, (cudaStream_t)stream);
   p.ts = (unsigned long long*)o->timestamps;
   if (o->tail != 1 && o->lambda_max == 0.0 && !b->rigid && o->precision != RT_PREC_DF) {
     if ((st = ensure_park(&b->d_park, &b->park_cap)) != RT_OK) return st;

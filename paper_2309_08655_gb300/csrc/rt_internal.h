@@ -74,12 +74,10 @@ struct TraceParams {
   // lane for every entry of the queue
   int lanes = 32;
   int covers = 0;
-  // guided rays (rt_guided.cuh): [0] found, then (key, ray) pairs, then the list;
-  // the first guided_max of the list have left the queue
-  unsigned long long* guided = nullptr;
-  int64_t guided_max = 0;
-  double* guided_rec = nullptr;   // their park records, for six-lane groups (NULL: none)
 };
+// The words of TraceParams::queue: the claim counter, the number of marked guided
+// rays and the counter of the search for them (rt_guided.cuh).
+enum { QUEUE_CLAIM = 0, QUEUE_GUIDED = 1, QUEUE_SCAN = 2, QUEUE_WORDS = 3 };
 // Grid of a persistent launch over n rays, at most bps blocks of `block` threads per
 // SM, and the lanes of a warp that take rays: with fewer than 32 rays for each of four
 // warps per SM, every scheduler gets a warp and each warp its share (a warp's attempt
@@ -113,13 +111,6 @@ constexpr int XRAYS_PER_SM = 12;       // one six-lane group in warps 0-1, five 
 inline size_t express_bytes() {
   return 64 + XSLOTS * sizeof(int) + (size_t)XCAP * 2 * sizeof(unsigned long long) +
          (size_t)XCAP * PARKREC * sizeof(double);
-}
-// The guided rays' scratch: a counter, GUIDED_CAP (key, ray) pairs, the list, and
-// the rays' park records.
-constexpr int64_t GUIDED_CAP = 4096;
-constexpr int64_t GUIDED_RECS = 32 + 3 * GUIDED_CAP;      // in 8-byte units
-inline size_t guided_bytes() {
-  return (size_t)(GUIDED_RECS + GUIDED_CAP * PARKREC) * sizeof(unsigned long long);
 }
 // Park capacity that covers any persistent grid on the device (up to 31 rays
 // per warp).
@@ -176,9 +167,8 @@ cudaError_t launch_trace_fp64(const TraceParams& p, int block, int blocks_per_sm
                               cudaStream_t stream);
 cudaError_t launch_trace_mixed(const TraceParams& p, int block, int blocks_per_sm,
                                cudaStream_t stream);
-// Lists the guided rays for a launch of the given number of warps (p.guided set;
-// sets p.guided_max).
-cudaError_t launch_guided(TraceParams& p, int64_t warps, cudaStream_t stream);
+// Clears the queue's words, marks the guided rays (RAY_EXPRESS) and counts them.
+cudaError_t launch_guided(const TraceParams& p, cudaStream_t stream);
 cudaError_t launch_tail_fp64(const TraceParams& p, cudaStream_t stream);
 // Binning: launch_bin = clear p.acc, then the three phases; the phases alone
 // serve the sharded binning (rt_bin_part_*), whose callers reduce p.acc

@@ -26,8 +26,9 @@ __global__ void __launch_bounds__(128) tail_fp64_kernel(TraceParams p, int nsm) 
     const unsigned long long K = *p.xcount < (unsigned long long)p.xcap
                                      ? *p.xcount : (unsigned long long)p.xcap;
     const unsigned long long S = express_solo(K);
-    tail_groups(p, p.xrec, 0, S, p.xcount + 2, GROUPS_PER_WARP, gc, slots);
-    tail_groups(p, p.xrec, S, K, p.xcount + 1, GROUPS_PER_WARP, gc, slots);
+    ParkedRays solo = {p.xrec, 0, S, p.xcount + 2}, rest = {p.xrec, S, K, p.xcount + 1};
+    tail_groups(p, solo, GROUPS_PER_WARP, gc, slots);
+    tail_groups(p, rest, GROUPS_PER_WARP, gc, slots);
   }
   const unsigned long long nparked = *p.park_count < (unsigned long long)p.park_cap
                                          ? *p.park_count
@@ -35,8 +36,10 @@ __global__ void __launch_bounds__(128) tail_fp64_kernel(TraceParams p, int nsm) 
   const unsigned long long wave = 4ull * (unsigned)nsm;     // warps of one block per SM
   const unsigned long long per = (nparked + wave - 1) / wave;
   const int ngroups = per < GROUPS_PER_WARP ? (int)(per > 0 ? per : 1) : GROUPS_PER_WARP;
-  if ((int)blockIdx.x < nsm || per > GROUPS_PER_WARP)
-    tail_groups(p, p.park, 0, nparked, p.park_next, ngroups, gc, slots);
+  if ((int)blockIdx.x < nsm || per > GROUPS_PER_WARP) {
+    ParkedRays parked = {p.park, 0, nparked, p.park_next};
+    tail_groups(p, parked, ngroups, gc, slots);
+  }
   if (p.counters && (lane % GROUP) == 0 && lane / GROUP < GROUPS_PER_WARP) {
     atomicAdd((unsigned long long*)&p.counters[CTR_ACC], (unsigned long long)gc.acc);
     atomicAdd((unsigned long long*)&p.counters[CTR_REJ], (unsigned long long)gc.rej);

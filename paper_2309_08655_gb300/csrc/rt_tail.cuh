@@ -19,6 +19,7 @@
 #include <stdint.h>
 
 #include "rt_device.cuh"
+#include "rt_guided.cuh"
 #include "rt_integrator.cuh"
 #include "rt_internal.h"
 
@@ -29,14 +30,72 @@ namespace {
 constexpr int GROUP = 6;           // lanes per ray
 constexpr int GROUPS_PER_WARP = 5;
 
-__device__ __forceinline__ int find_star_t(const TraceParams& p, int64_t i) {
+__device__ __forceinline__ int find_star(const TraceParams& p, int64_t i) {
   if (p.nstars <= 1) return 0;
-  int lo = 0, hi = p.nstars - 1;
+  int lo = 0, hi = p.nstars - 1;   // offsets[s] <= i < offsets[s + 1]
   while (lo < hi) {
     const int mid = (lo + hi + 1) >> 1;
     if (p.offsets[mid] <= i) lo = mid; else hi = mid - 1;
   }
   return lo;
+}
+
+__device__ void load_lane(const TraceParams& p, int64_t i, Lane& L) {
+  const StarDev& s = p.stars[find_star(p, i)];
+  const int64_t n = p.n;
+  L.R_km = s.R_km;
+  L.ma_eV = s.ma_eV;
+  const double iR = 1.0 / s.R_km, im = 1.0 / s.ma_eV;
+  L.y[0] = p.state[i] * iR;
+  L.y[1] = p.state[n + i] * iR;
+  L.y[2] = p.state[2 * n + i] * iR;
+  L.y[3] = p.state[3 * n + i] * im;
+  L.y[4] = p.state[4 * n + i] * im;
+  L.y[5] = p.state[5 * n + i] * im;
+  const double om = 1.0 + p.state[6 * n + i];
+  const double psi = p.state[7 * n + i];
+  double sp, cpsi;
+  sincos(psi, &sp, &cpsi);
+  L.c.rs = s.rs_prop;
+  L.c.cp = s.cp;
+  L.c.pa = s.plasma_a;
+  L.c.W2 = om * om;
+  L.c.iW2 = 1.0 / (om * om);
+  L.c.m0 = s.sin_tm * cpsi;
+  L.c.m1 = s.sin_tm * sp;
+  L.c.m2 = s.cos_tm;
+  L.c.disp = s.dispersion;
+  L.c.plasma = s.plasma;
+  L.c.sig = gj_side<double>(L.c.m0, L.c.m1, L.c.m2, L.y[0], L.y[1], L.y[2]);
+  L.switching = false;
+  L.h_resume = 0.0;
+  rhs64(L.c, L.y, L.f0);
+  const double hmax = (p.lambda_max > 0.0) ? p.lambda_max : 1e30;
+  L.h = initial_step(L.c, L.y, L.f0, p.rtol, p.atol, hmax);
+  L.lam = 0.0;
+  L.na = 0;
+  L.nr = 0;
+  if (p.claim_status == RAY_PROMOTED) {   // resume a ray handed over by the FP32 pass
+    if (p.nacc) L.na = p.nacc[i];
+    if (p.nrej) L.nr = p.nrej[i];
+  }
+  L.last_rej = false;
+}
+
+// A READY ray's park record: the start of load_lane.
+__device__ void fresh_record(const TraceParams& p, int64_t ray, double* pe) {
+  Lane L;
+  load_lane(p, ray, L);
+#pragma unroll
+  for (int j = 0; j < 6; ++j) pe[j] = L.y[j];
+  pe[6] = L.h;
+  pe[7] = 0.0;
+  pe[8] = L.c.sig;
+  pe[9] = 0.0;
+  pe[10] = 0.0;
+  pe[11] = 0.0;
+  pe[12] = (double)ray;
+  pe[13] = 0.0;
 }
 
 // The group's right-hand side as passes over a small register file in shared
@@ -436,7 +495,7 @@ __device__ __forceinline__ int advance_group(const TraceParams& p, const GroupFi
   return (L.h < 1e-12) ? RAY_STIFF : -1;
 }
 
-// shared doubles of a block of up to four warps
+// shared doubles of four warps
 constexpr int GROUP_SLOTS = 4 * GROUPS_PER_WARP * SLOTS;
 
 // Counts of one warp's finished rays (lane c == 0 of each group holds its own).
@@ -444,18 +503,58 @@ struct GroupCounts {
   long long acc = 0, rej = 0, traced = 0, esc = 0;
 };
 
-// Six-lane groups of the calling warp continue parked rays: records
-// lo + e of recs (PARKREC doubles each: y[6], h, h_resume, sig, flags, na, nr,
-// ray, lambda), e = 0, 1, ... claimed one per group with an atomic on *next,
-// while lo + e < hi; without next the warp's groups share out lo, lo + stride,
-// lo + 2 stride, ...  ngroups (1 to GROUPS_PER_WARP) groups of the warp take
-// part: one group per warp keeps a ray's attempts free of the other groups'
-// divergent branches.  slots: shared memory of the block, GROUP_SLOTS doubles.
-// Every lane of the warp must call it.
-__device__ void tail_groups(const TraceParams& p, const double* recs, unsigned long long lo,
-                            unsigned long long hi, unsigned long long* next, int ngroups,
-                            GroupCounts& cnt, double* slots,
-                            unsigned long long stride = 0) {
+// Where a warp's groups get their rays: records lo + e of recs (PARKREC doubles each:
+// y[6], h, h_resume, sig, flags, na, nr, ray, lambda), e = 0, 1, ... claimed with an
+// atomic on *next, while lo + e < hi.
+struct ParkedRays {
+  const double* recs;
+  unsigned long long lo, hi;
+  unsigned long long* next;
+  // once an iteration, every lane of the warp (wants: the lane's group is free)
+  __device__ __forceinline__ void poll(const TraceParams&, bool, bool) {}
+  // the lanes of a free group: its next record, or NULL (*done: no more will come)
+  __device__ __forceinline__ const double* take(const TraceParams&, const GroupFile& f, int base,
+                                                bool* done) {
+    unsigned long long e = 0;
+    if (f.cc == 0) e = lo + atomicAdd(next, 1ull);
+    e = __shfl_sync(f.gm, e, base);
+    *done = e >= hi;
+    return *done ? nullptr : recs + e * PARKREC;
+  }
+};
+
+// The marked guided rays of a launch (rt_guided.cuh), from their start.
+struct FreshRays {
+  GuidedScan scan;
+  int64_t ray = -1;
+  __device__ __forceinline__ void poll(const TraceParams& p, bool wants, bool busy) {
+    const int lane = threadIdx.x & 31;
+    const unsigned w = __ballot_sync(0xffffffffu, wants && lane % GROUP == 0);
+    const unsigned b = __ballot_sync(0xffffffffu, busy);
+    ray = -1;
+    if (w == 0 || !scan.more(p, b != 0)) return;
+    ray = scan.nth(__popc(w & ((1u << (lane - lane % GROUP)) - 1u)));
+    scan.drop(__popc(w));
+  }
+  __device__ __forceinline__ const double* take(const TraceParams& p, const GroupFile& f, int,
+                                                bool* done) {
+    *done = ray < 0 && !scan.open && scan.found == 0;
+    if (ray < 0) return nullptr;
+    double* pe = f.s + S_P1;              // the passes' slots are free between rays
+    __syncwarp(f.gm);
+    if (f.cc == 0) fresh_record(p, ray, pe);
+    __syncwarp(f.gm);
+    return pe;
+  }
+};
+
+// Six-lane groups of the calling warp continue the rays of src.  ngroups (1 to
+// GROUPS_PER_WARP) groups of the warp take part: one group per warp keeps a ray's
+// attempts free of the other groups' divergent branches.  slots: shared memory of the
+// block, GROUP_SLOTS doubles for every four warps.  Every lane of the warp must call it.
+template <class Source>
+__device__ void tail_groups(const TraceParams& p, Source& src, int ngroups, GroupCounts& cnt,
+                            double* slots) {
   const int lane = threadIdx.x & 31;
   const int g = lane / GROUP, cc = lane % GROUP;
   const bool in_group = g < ngroups && g < GROUPS_PER_WARP;
@@ -466,16 +565,11 @@ __device__ void tail_groups(const TraceParams& p, const double* recs, unsigned l
   if (in_group) file_init(f, slots + ((threadIdx.x >> 5) * GROUPS_PER_WARP + g) * SLOTS, cc, gm);
   bool have = false, done = !in_group;
   int na0 = 0, nr0 = 0;
-  unsigned long long taken = 0;
   for (;;) {
+    src.poll(p, in_group && !have && !done, have);
     if (in_group && !have && !done) {
-      unsigned long long e = 0;
-      if (cc == 0) e = lo + (next ? atomicAdd(next, 1ull) : (taken++ * ngroups + g) * stride);
-      e = __shfl_sync(gm, e, base);
-      if (e >= hi) {
-        done = true;
-      } else {
-        const double* pe = recs + e * PARKREC;
+      const double* pe = src.take(p, f, base, &done);
+      if (pe) {
         L.yc = pe[cc];
         L.h = pe[6];
         L.h_resume = pe[7];
@@ -487,7 +581,7 @@ __device__ void tail_groups(const TraceParams& p, const double* recs, unsigned l
         L.nr = (int)pe[11];
         L.ray = (int64_t)pe[12];
         L.lam = pe[13];
-        L.star = find_star_t(p, L.ray);
+        L.star = find_star(p, L.ray);
         const StarDev& s = p.stars[L.star];
         const double om = 1.0 + p.state[6 * p.n + L.ray];
         double sp, cpsi;

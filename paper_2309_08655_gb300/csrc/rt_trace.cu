@@ -17,58 +17,6 @@ namespace rtk {
 
 namespace {
 
-__device__ __forceinline__ int find_star(const TraceParams& p, int64_t i) {
-  if (p.nstars <= 1) return 0;
-  int lo = 0, hi = p.nstars - 1;   // offsets[s] <= i < offsets[s + 1]
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (p.offsets[mid] <= i) lo = mid; else hi = mid - 1;
-  }
-  return lo;
-}
-
-__device__ void load_lane(const TraceParams& p, int64_t i, Lane& L) {
-  const StarDev& s = p.stars[find_star(p, i)];
-  const int64_t n = p.n;
-  L.R_km = s.R_km;
-  L.ma_eV = s.ma_eV;
-  const double iR = 1.0 / s.R_km, im = 1.0 / s.ma_eV;
-  L.y[0] = p.state[i] * iR;
-  L.y[1] = p.state[n + i] * iR;
-  L.y[2] = p.state[2 * n + i] * iR;
-  L.y[3] = p.state[3 * n + i] * im;
-  L.y[4] = p.state[4 * n + i] * im;
-  L.y[5] = p.state[5 * n + i] * im;
-  const double om = 1.0 + p.state[6 * n + i];
-  const double psi = p.state[7 * n + i];
-  double sp, cpsi;
-  sincos(psi, &sp, &cpsi);
-  L.c.rs = s.rs_prop;
-  L.c.cp = s.cp;
-  L.c.pa = s.plasma_a;
-  L.c.W2 = om * om;
-  L.c.iW2 = 1.0 / (om * om);
-  L.c.m0 = s.sin_tm * cpsi;
-  L.c.m1 = s.sin_tm * sp;
-  L.c.m2 = s.cos_tm;
-  L.c.disp = s.dispersion;
-  L.c.plasma = s.plasma;
-  L.c.sig = gj_side<double>(L.c.m0, L.c.m1, L.c.m2, L.y[0], L.y[1], L.y[2]);
-  L.switching = false;
-  L.h_resume = 0.0;
-  rhs64(L.c, L.y, L.f0);
-  const double hmax = (p.lambda_max > 0.0) ? p.lambda_max : 1e30;
-  L.h = initial_step(L.c, L.y, L.f0, p.rtol, p.atol, hmax);
-  L.lam = 0.0;
-  L.na = 0;
-  L.nr = 0;
-  if (p.claim_status == RAY_PROMOTED) {   // resume a ray handed over by the FP32 pass
-    if (p.nacc) L.na = p.nacc[i];
-    if (p.nrej) L.nr = p.nrej[i];
-  }
-  L.last_rej = false;
-}
-
 __device__ void store_lane(const TraceParams& p, int64_t i, const Lane& L, int st) {
   const int64_t n = p.n;
   p.state[i] = L.y[0] * L.R_km;
@@ -80,22 +28,6 @@ __device__ void store_lane(const TraceParams& p, int64_t i, const Lane& L, int s
   status_after_state(p, i, st);
   if (p.nacc) p.nacc[i] = L.na;
   if (p.nrej) p.nrej[i] = L.nr;
-}
-
-// A READY ray's park record: the start of load_lane.
-__device__ void fresh_record(const TraceParams& p, int64_t ray, double* pe) {
-  Lane L;
-  load_lane(p, ray, L);
-#pragma unroll
-  for (int j = 0; j < 6; ++j) pe[j] = L.y[j];
-  pe[6] = L.h;
-  pe[7] = 0.0;
-  pe[8] = L.c.sig;
-  pe[9] = 0.0;
-  pe[10] = 0.0;
-  pe[11] = 0.0;
-  pe[12] = (double)ray;
-  pe[13] = 0.0;
 }
 
 // Express lane, step 1: the READY rays of cost bucket 0 as (key, ray) pairs,
@@ -133,41 +65,20 @@ __global__ void express_rank_kernel(TraceParams p) {
   }
 }
 
-// Guided rays of the lane-per-ray kernels (rt_guided.cuh): the READY rays of cost
-// bucket 0 as (key, ray) pairs, then into the list by rank, nearest the cone first;
-// the first guided_max leave the queue (RAY_EXPRESS).
-__global__ void guided_select_kernel(TraceParams p) {
+// Marks the guided rays of the double-float and rotating kernels (rt_guided.cuh): the
+// READY rays of cost bucket 0.
+__global__ void guided_mark_kernel(TraceParams p) {
+  unsigned marked = 0;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < p.n;
        i += (int64_t)gridDim.x * blockDim.x) {
     if (p.status[i] != RAY_READY) continue;
-    const double d2 = cone_dist2(p.stars[find_star(p, i)], p.state, p.n, i);
-    if (!(d2 < 1e-6)) continue;
-    const unsigned long long slot = atomicAdd(p.guided, 1ull);
-    if (slot < (unsigned long long)GUIDED_CAP) {
-      p.guided[32 + 2 * slot] = (unsigned long long)__double_as_longlong(d2);
-      p.guided[32 + 2 * slot + 1] = (unsigned long long)i;
-    }
+    if (!(cone_dist2(p.stars[find_star(p, i)], p.state, p.n, i) < 1e-6)) continue;
+    p.status[i] = RAY_EXPRESS;
+    ++marked;
   }
-}
-
-__global__ void guided_rank_kernel(TraceParams p) {
-  const unsigned long long K = *p.guided < (unsigned long long)GUIDED_CAP
-                                   ? *p.guided : (unsigned long long)GUIDED_CAP;
-  const unsigned long long* cand = p.guided + 32;
-  for (unsigned long long k = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; k < K;
-       k += (unsigned long long)gridDim.x * blockDim.x) {
-    const unsigned long long key = cand[2 * k], ray = cand[2 * k + 1];
-    unsigned long long rank = 0;
-    for (unsigned long long j = 0; j < K; ++j) {
-      const unsigned long long kj = cand[2 * j], rj = cand[2 * j + 1];
-      rank += (kj < key || (kj == key && rj < ray)) ? 1ull : 0ull;
-    }
-    p.guided[32 + 2 * GUIDED_CAP + rank] = ray;
-    if (rank < (unsigned long long)p.guided_max) {
-      if (p.guided_rec) fresh_record(p, (int64_t)ray, p.guided_rec + rank * PARKREC);
-      p.status[ray] = RAY_EXPRESS;
-    }
-  }
+  marked = __reduce_add_sync(FULL, marked);
+  if ((threadIdx.x & 31) == 0 && marked)
+    atomicAdd(p.queue + QUEUE_GUIDED, (unsigned long long)marked);
 }
 
 __device__ __forceinline__ unsigned sm_id() {
@@ -210,8 +121,9 @@ __global__ void __launch_bounds__(128) trace_fp64_kernel(TraceParams p) {
     __syncthreads();
     if (role == 0) {
       GroupCounts gc;
-      if ((threadIdx.x >> 5) < 2) tail_groups(p, p.xrec, 0, S, p.xcount + 2, 1, gc, slots);
-      tail_groups(p, p.xrec, S, K, p.xcount + 1, GROUPS_PER_WARP, gc, slots);
+      ParkedRays solo = {p.xrec, 0, S, p.xcount + 2}, rest = {p.xrec, S, K, p.xcount + 1};
+      if ((threadIdx.x >> 5) < 2) tail_groups(p, solo, 1, gc, slots);
+      tail_groups(p, rest, GROUPS_PER_WARP, gc, slots);
       acc += gc.acc;
       rej += gc.rej;
       traced += gc.traced;
@@ -619,20 +531,16 @@ cudaError_t occupancy_batch_fp64(int block, int* occ) {
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, batch_fp64_kernel, block, 0);
 }
 
-cudaError_t launch_guided(TraceParams& p, int64_t warps, cudaStream_t stream) {
-  p.guided_max = 32 * (warps / 4 > 0 ? warps / 4 : 1);
+cudaError_t launch_guided(const TraceParams& p, cudaStream_t stream) {
   int dev = 0, nsm = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
-  e = cudaMemsetAsync(p.guided, 0, sizeof(unsigned long long), stream);
+  e = cudaMemsetAsync(p.queue, 0, QUEUE_WORDS * sizeof(unsigned long long), stream);
   if (e != cudaSuccess) return e;
   const int64_t need = (p.n + 255) / 256, cap = (int64_t)nsm * 8;
-  guided_select_kernel<<<(unsigned)(need < cap ? (need > 0 ? need : 1) : cap), 256, 0, stream>>>(p);
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  guided_rank_kernel<<<(unsigned)((GUIDED_CAP + 127) / 128), 128, 0, stream>>>(p);
+  guided_mark_kernel<<<(unsigned)(need < cap ? (need > 0 ? need : 1) : cap), 256, 0, stream>>>(p);
   return cudaGetLastError();
 }
 

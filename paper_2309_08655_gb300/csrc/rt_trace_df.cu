@@ -518,12 +518,11 @@ __global__ void __launch_bounds__(256) trace_df_kernel(TraceParams p) {
     // the guided rays six lanes each in FP64, from the start of the launch: 12.6 us
     // an attempt where a lone double-float lane takes 18, on a pipe that the rest
     // of the launch leaves idle
-    const GuidedShare share = guided_share(p);
-    if (share.mine > 0) {
+    const int quota = guided_quota(p);
+    if (quota > 0) {
       GroupCounts gc;
-      tail_groups(p, p.guided_rec, share.first, share.first + share.mine * share.stride, nullptr,
-                  share.mine < GROUPS_PER_WARP ? share.mine : GROUPS_PER_WARP, gc, slots,
-                  share.stride);
+      FreshRays rays;
+      tail_groups(p, rays, quota < GROUPS_PER_WARP ? quota : GROUPS_PER_WARP, gc, slots);
       acc += gc.acc;
       rej += gc.rej;
       traced += gc.traced;
@@ -604,12 +603,8 @@ cudaError_t launch_trace_df(const TraceParams& p, int block, int blocks_per_sm,
   const PersistentShape shape = persistent_shape(p.n, nsm, block, blocks_per_sm);
   TraceParams q = p;
   q.lanes = shape.lanes;
-  e = cudaMemsetAsync(p.queue, 0, sizeof(unsigned long long), stream);
+  e = launch_guided(q, stream);
   if (e != cudaSuccess) return e;
-  if (q.guided) {
-    e = launch_guided(q, (int64_t)shape.grid * (block / 32), stream);
-    if (e != cudaSuccess) return e;
-  }
   trace_df_kernel<<<shape.grid, block, 0, stream>>>(q);
   return cudaGetLastError();
 }

@@ -355,20 +355,30 @@ __device__ int advance_rot(const TraceParams& p, RotLane& L) {
 __global__ void __launch_bounds__(128) trace_rot_kernel(TraceParams p) {
   const int lane = threadIdx.x & 31;
   int64_t ray = lane < p.lanes ? -1 : -2;   // -1: needs a ray, -2: queue exhausted
-  const GuidedShare share = guided_share(p);
-  bool guided = share.mine > 0;
+  const int quota = guided_quota(p);
+  bool guided = quota > 0;
+  GuidedScan scan;
   RotLane L;
   long long acc = 0, rej = 0, traced = 0, esc = 0;
   const int64_t nq = p.order ? (int64_t)COST_BUCKETS * p.n : p.n;   // cost-ordered passes
   if (p.ts && threadIdx.x == 0) atomicMin(p.ts, global_ns());
-  if (lane < share.mine) {
-    ray = (int64_t)share.list[share.first + lane * share.stride];
-    load_rot(p, ray, L);
-  }
   for (;;) {
-    if (guided && __ballot_sync(FULL, ray >= 0) == 0) {   // the share has ended
-      guided = false;
-      ray = lane < p.lanes ? -1 : -2;
+    if (guided) {
+      // marked rays to the free lanes, up to the quota at a time
+      unsigned busy = __ballot_sync(FULL, ray >= 0);
+      while (__popc(busy) < quota && scan.more(p, busy != 0)) {
+        const int64_t i = scan.nth(__popc(~busy & ((1u << lane) - 1u)));
+        if (ray < 0 && i >= 0) {
+          ray = i;
+          load_rot(p, i, L);
+        }
+        scan.drop(32 - __popc(busy));
+        busy = __ballot_sync(FULL, ray >= 0);
+      }
+      if (busy == 0) {   // none is left
+        guided = false;
+        ray = lane < p.lanes ? -1 : -2;
+      }
     }
     const bool need = (ray == -1) && !guided;
     const unsigned mneed = __ballot_sync(FULL, need);
@@ -446,12 +456,8 @@ cudaError_t launch_trace_rot(const TraceParams& p, int block, int blocks_per_sm,
   const PersistentShape shape = persistent_shape(p.n, nsm, block, blocks_per_sm);
   TraceParams q = p;
   q.lanes = shape.lanes;
-  e = cudaMemsetAsync(p.queue, 0, sizeof(unsigned long long), stream);
+  e = launch_guided(q, stream);
   if (e != cudaSuccess) return e;
-  if (q.guided) {
-    e = launch_guided(q, (int64_t)shape.grid * (block / 32), stream);
-    if (e != cudaSuccess) return e;
-  }
   trace_rot_kernel<<<shape.grid, block, 0, stream>>>(q);
   return cudaGetLastError();
 }
