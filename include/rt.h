@@ -442,8 +442,10 @@ rt_status rt_trace_backward(const rt_star* star, int32_t nx, int32_t ny, double 
  *   the FP64 integrator, at the star's parameters, for the n samples drawn
  *   from d_uniforms (RT_UNIFORM_ROWS x n, as rt_sample_conversion_surface)
  *   and traced with opts (lambda_max 0).  Each ray is re-integrated in FP64
- *   (the same steps as the forward rt_trace_forward run with the same opts,
- *   whose accepted steps per ray d_nacc sizes the store) and swept
+ *   (from the sampling kernel's own states and with the integrator of the forward
+ *   rt_trace_forward run with the same opts, whose accepted steps per ray d_nacc
+ *   sizes the store; the two round some sums differently, and a ray guided along
+ *   the null cone may take a few steps more or less) and swept
  *   backwards: the discrete adjoint of each Dormand-Prince step
  *   (Jacobian-vector products of the analytic right-hand side by forward-mode
  *   dual numbers), the saltation jump where the Goldreich-Julian branch
@@ -478,7 +480,7 @@ rt_status rt_trace_backward(const rt_star* star, int32_t nx, int32_t ny, double 
  *                allocation fails falls back to the checkpoints
  *     store_bytes out (host, may be NULL): bytes of the tape or checkpoint store
  *   Needs RT_PLASMA_GJ, M_sun > 0 and B0_G > 0.  Synchronous: allocates the
- *   store and 69 B per ray, and frees them before returning; RT_ENOMEM if
+ *   store and 141 B per ray, and frees them before returning; RT_ENOMEM if
  *   that fails.  Deterministic (fixed-order sums of per-ray terms).
  */
 rt_status rt_flux_value(const rt_star* star, int64_t n, const double* d_state,

@@ -673,7 +673,7 @@ rt_status rt_flux_gradient(const rt_star* s, int64_t n, const double* d_uniforms
   // under tape_max_bytes, else the checkpoints and the segment records
   int64_t* off = nullptr;
   double *ck = nullptr, *seg = nullptr, *Fr = nullptr, *Gr = nullptr, *tape = nullptr,
-         *head = nullptr;
+         *head = nullptr, *smp = nullptr;
   int64_t* order = nullptr;
   unsigned long long* bucket = nullptr;
   uint8_t* stt = nullptr;
@@ -684,6 +684,7 @@ rt_status rt_flux_gradient(const rt_star* s, int64_t n, const double* d_uniforms
     cudaFree(seg);
     cudaFree(Fr);
     cudaFree(Gr);
+    cudaFree(smp);
     cudaFree(tape);
     cudaFree(head);
     cudaFree(order);
@@ -699,6 +700,7 @@ rt_status rt_flux_gradient(const rt_star* s, int64_t n, const double* d_uniforms
   if ((e = cudaMalloc(&off, (n + 1) * sizeof(int64_t))) != cudaSuccess ||
       (e = cudaMalloc(&Fr, n * sizeof(double))) != cudaSuccess ||
       (e = cudaMalloc(&Gr, (size_t)rtk::NPARAMS * n * sizeof(double))) != cudaSuccess ||
+      (e = cudaMalloc(&smp, (size_t)(RT_STATE_ROWS + 1) * n * sizeof(double))) != cudaSuccess ||
       (e = cudaMalloc(&flg, n * sizeof(int32_t))) != cudaSuccess ||
       (!d_status && (e = cudaMalloc(&stt, n)) != cudaSuccess))
     return alloc_fail(e, "adjoint scratch allocation failed");
@@ -708,6 +710,22 @@ rt_status rt_flux_gradient(const rt_star* s, int64_t n, const double* d_uniforms
   a.status = stt;
   a.flags = flg;
   a.nacc = d_nacc;
+  // the samples themselves, by the kernel that made the forward run's
+  rtk::SampleParams sp;
+  sp.stars = s->d;
+  sp.nstars = 1;
+  sp.begin[0] = 0;
+  sp.begin[1] = sp.norm[0] = sp.ld = n;
+  sp.u = d_uniforms;
+  sp.state = smp;
+  sp.weight = smp + (size_t)RT_STATE_ROWS * n;
+  sp.status = stt;
+  a.state = sp.state;
+  a.weight = sp.weight;
+  if ((e = rtk::launch_sample(sp, cs)) != cudaSuccess) {
+    cleanup();
+    return cuda_fail(e, "sample kernel");
+  }
   // the tape's size from the forward step counts
   int64_t total = 0;
   if ((e = rtk::launch_tape_offsets(d_nacc, n, off, cs)) != cudaSuccess ||

@@ -85,7 +85,8 @@ enum { FL_FLIP_BEFORE = 1, FL_FLIP_AFTER = 2, FL_ESCAPE = 4 };
 
 struct AdjParams {
   SampConst<Dual<NSAMP_TANGENTS>> sc;
-  SampConst<double> scv;
+  const double* state;    // the samples (rt_sample.cu), 8 x n, and their weights
+  const double* weight;
   double R_km, ma_eV, rs_prop, cp, plasma_a, cos_tm, sin_tm;
   int dispersion, plasma;
   double drsp_dM, drsp_dR, dcp_dma, dcp_dB0;
@@ -628,33 +629,39 @@ __device__ __forceinline__ TraceParams replay_params(const AdjParams& P) {
   return tp;
 }
 
-// Samples ray i with its parameter tangents (so) and its plain values (sv,
-// exactly as the sampling kernel computes them) and sets up the lane exactly
-// as the forward trace loads it from the state.  false: no conversion point;
-// the ray's outputs are zeroed.
-__device__ bool begin_ray(const AdjParams& P, int64_t i, SampOut<Dual<NSAMP_TANGENTS>>& so,
-                          SampOut<double>& sv, Lane& L, double& cps, double& sps) {
+// Sets up the lane of ray i from the sampling kernel's state, as the forward trace
+// loads it (so the two start from the same bits), and samples it once more with its
+// parameter tangents (so).  false: no conversion point; the ray's outputs are zeroed.
+// Out of line: one copy for the kernels of every sweep precision, so that their replays
+// start alike.
+__device__ __noinline__ bool begin_ray(const AdjParams& P, int64_t i,
+                                       SampOut<Dual<NSAMP_TANGENTS>>& so, double& w, Lane& L,
+                                       double& cps, double& sps) {
   const int64_t n = P.n;
-  double u[6];
-#pragma unroll
-  for (int j = 0; j < 6; ++j) u[j] = P.u[j * n + i];
-  sample_core(P.sc, u, (double)n, so);
-  sample_core(P.scv, u, (double)n, sv);
   P.flags[i] = 0;
-  if (!sv.ok || !so.ok) {
+  bool ok = P.status[i] == RAY_READY;
+  if (ok) {
+    double u[6];
+#pragma unroll
+    for (int j = 0; j < 6; ++j) u[j] = P.u[j * n + i];
+    sample_core(P.sc, u, (double)n, so);
+    ok = so.ok;
+  }
+  if (!ok) {
     P.F_ray[i] = 0.0;
     for (int k = 0; k < NPARAMS; ++k) P.G_ray[k * n + i] = 0.0;
     P.status[i] = RAY_NO_ROOT;
     return false;
   }
+  w = P.weight[i];
   const double iR = 1.0 / P.R_km, im = 1.0 / P.ma_eV;
 #pragma unroll
   for (int j = 0; j < 3; ++j) {
-    L.y[j] = (sv.x[j] * P.R_km) * iR;
-    L.y[3 + j] = (sv.k[j] * P.ma_eV) * im;
+    L.y[j] = P.state[j * n + i] * iR;
+    L.y[3 + j] = P.state[(3 + j) * n + i] * im;
   }
-  const double om = 1.0 + sv.delta;
-  sincos(sv.psi, &sps, &cps);
+  const double om = 1.0 + P.state[6 * n + i];
+  sincos(P.state[7 * n + i], &sps, &cps);
   L.R_km = P.R_km;
   L.ma_eV = P.ma_eV;
   L.c.rs = P.rs_prop;
@@ -687,10 +694,9 @@ template <class T, bool HYB = false>
 __device__ void adjoint_ray(const AdjParams& P, int64_t i, double* seg, long long* steps) {
   const int64_t n = P.n;
   SampOut<Dual<NSAMP_TANGENTS>> so;
-  SampOut<double> sv;
   Lane L;
-  double sps, cps;
-  if (!begin_ray(P, i, so, sv, L, cps, sps)) return;
+  double w, sps, cps;
+  if (!begin_ray(P, i, so, w, L, cps, sps)) return;
   double G[NPARAMS];
   TraceParams tp = replay_params(P);
   // forward replay with a checkpoint every CK accepted steps
@@ -728,7 +734,6 @@ __device__ void adjoint_ray(const AdjParams& P, int64_t i, double* seg, long lon
   }
   // functional at the escape point
   double ybar[6], qbar[NQ] = {0, 0, 0}, rsb, dmu_di;
-  const double w = sv.w;
   double Kv;
   const double Fi = flux_kernel_value(P, L.y, w, ybar, &rsb, &dmu_di, &Kv);
   qbar[Q_RS] += rsb;
@@ -858,11 +863,10 @@ __global__ void __launch_bounds__(128) adjoint_sample_kernel(AdjParams P) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= P.n) return;
   SampOut<Dual<NSAMP_TANGENTS>> so;
-  SampOut<double> sv;
   Lane L;
-  double cps, sps;
+  double w, cps, sps;
   double* hd = P.head + i * HEADREC;
-  if (!begin_ray(P, i, so, sv, L, cps, sps)) {
+  if (!begin_ray(P, i, so, w, L, cps, sps)) {
     hd[HD_NREC] = -1.0;
     return;
   }
@@ -886,7 +890,7 @@ __global__ void __launch_bounds__(128) adjoint_sample_kernel(AdjParams P) {
   hd[HD_M + 2] = L.c.m2;
 #pragma unroll
   for (int j = 0; j < 6; ++j) hd[HD_Y0 + j] = L.y[j];
-  hd[HD_W] = sv.w;
+  hd[HD_W] = w;
 }
 
 // The lane of ray i from its head record, exactly as begin_ray leaves it.
@@ -1278,30 +1282,8 @@ cudaError_t adjoint_grid(int prec, int* grid, int* block) {
 static AdjParams adj_params(const AdjLaunch& a) {
   AdjParams P;
   P.sc = a.sc;
-  {
-    const auto& d = a.sc;
-    SampConst<double>& v = P.scv;
-    v.rs = d.rs.v;
-    v.cp = d.cp.v;
-    v.sin_tm = d.sin_tm.v;
-    v.cos_tm = d.cos_tm.v;
-    v.B0_eV2 = d.B0_eV2.v;
-    v.R_eV = d.R_eV.v;
-    v.n_inf = d.n_inf.v;
-    v.ma_eV = d.ma_eV.v;
-    v.v0 = d.v0;
-    v.psi_fixed = d.psi_fixed;
-    v.plasma_a = d.plasma_a;
-    v.rlc = d.rlc;
-    v.g_eV = d.g_eV;
-    v.w_unit = d.w_unit;
-    v.disp = d.disp;
-    v.plasma = d.plasma;
-    v.fa_model = d.fa_model;
-    v.phase_mode = d.phase_mode;
-    v.weight_mode = d.weight_mode;
-    v.per_cm3 = d.per_cm3;
-  }
+  P.state = a.state;
+  P.weight = a.weight;
   P.R_km = a.star->R_km;
   P.ma_eV = a.star->ma_eV;
   P.rs_prop = a.star->rs_prop;

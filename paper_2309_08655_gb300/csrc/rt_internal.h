@@ -257,6 +257,8 @@ struct AdjLaunch {
   // doubles per ray; order: the rays, longest first (n), built from nacc with
   // the 32 counters of bucket
   const int64_t* tape_off;
+  const double* state;    // the samples of u (launch_sample): 8 x n, weights; the
+  const double* weight;   // statuses in `status`
   double* tape;
   double* head;
   const int32_t* nacc;
