@@ -429,19 +429,18 @@ struct CrossingAcc {
   }
 
   // A piece [a, b] whose ends have the same sign of g (negative iff neg)
-  // while g turns toward zero inside: the extremum is located by FP64
-  // bisection on the sign of dg/dth; if g has the other sign there, the two
-  // roots on either side are located and counted.
+  // while g turns toward zero inside: the extremum is located in FP64 by Illinois on
+  // dg/dth.  Whether g has the other sign there (*te): two roots, on either side.
   template <class Dense64>
-  __device__ void graze(const RayConst<double>& c, double a, double b, bool neg,
-                        Dense64& dense64) {
+  __device__ bool graze(const RayConst<double>& c, double a, double b, bool neg,
+                        Dense64& dense64, double* te) {
     double yd[6], yp[6], g, ga, gb;
     dense64(a, yd, yp);
     crossing_g_slope(c, W, yd, yp, &g, &ga);
     dense64(b, yd, yp);
     crossing_g_slope(c, W, yd, yp, &g, &gb);
     // a minimum of |g| on the side of neg: g' < 0 then > 0 for g > 0
-    if (neg ? !(ga > 0.0 && gb < 0.0) : !(ga < 0.0 && gb > 0.0)) return;
+    if (neg ? !(ga > 0.0 && gb < 0.0) : !(ga < 0.0 && gb > 0.0)) return false;
     // Illinois (regula falsi with halving of the stale end) on dg/dth
     double lo = a, hi = b, flo = ga, fhi = gb;
     int side = 0;
@@ -463,11 +462,9 @@ struct CrossingAcc {
         side = 1;
       }
     }
-    const double te = 0.5 * (lo + hi);
-    dense64(te, yd, nullptr);
-    if ((crossing_g(c, W, yd) < 0.0) == neg) return;      // the dip stays on its side
-    root(c, a, te, neg, dense64);
-    root(c, te, b, !neg, dense64);
+    *te = 0.5 * (lo + hi);
+    dense64(*te, yd, nullptr);
+    return (crossing_g(c, W, yd) < 0.0) != neg;           // else the dip stays on its side
   }
 
   // One accepted step from y to yn with the continuous extension y(th): the
@@ -494,8 +491,9 @@ struct CrossingAcc {
     double th0 = 0.0;
     bool negA = neg_prev;
     float NA, slA;
-    // pieces whose dip is searched after the loop (bit q - 1), and their sign
-    unsigned dips = 0u, dip_neg = 0u;
+    // pieces with a sign change, and pieces whose dip is searched (bit q - 1), both
+    // after the loop; the signs at their starts
+    unsigned roots = 0u, dips = 0u, negs = 0u;
     {
       const float d[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
       float xs[3], ks[3];
@@ -558,8 +556,9 @@ struct CrossingAcc {
         dense64(th1, yd, nullptr);
         negB = crossing_g(c, W, yd) < 0.0;
       }
+      if (negA) negs |= 1u << (q - 1);
       if (negA != negB) {
-        root(c, th0, th1, negA, dense64);
+        roots |= 1u << (q - 1);
       } else {
         // s N decreasing at th0 and increasing at th1 (s = sign of g): a dip
         // toward zero between them; the tangent lines at both ends meet at
@@ -574,7 +573,6 @@ struct CrossingAcc {
           const float margin = 0.05f * (2.0f + fabsf(NA) + fabsf(NB));
           if (!(L > margin)) {
             dips |= 1u << (q - 1);
-            if (negA) dip_neg |= 1u << (q - 1);
           }
         }
       }
@@ -585,11 +583,29 @@ struct CrossingAcc {
     }
     neg_prev = negA;
     nsearch += __popc(dips);
-    while (dips) {
-      const int q = __ffs(dips);                   // piece q: [(q - 1), q] / BACK_SUBDIV
-      dips &= dips - 1u;
-      graze(c, (double)(q - 1) / BACK_SUBDIV, (double)q / BACK_SUBDIV,
-            ((dip_neg >> (q - 1)) & 1u) != 0u, dense64);
+    // One root at a time, from a single place: the search and the contribution are much of
+    // the kernels' code, and the mixed kernels wait for instructions, not for FP64.  Three
+    // places took the joint mixed launch of 64 forward and 64 image instances from 1029
+    // to 1720 ms when the search grew by four evaluations of g; from one place it takes
+    // 900 ms, and a 512 x 512 mixed image 38 ms against 55.
+    unsigned todo = roots | dips;
+    double te = 0.0;
+    bool second = false;                           // the root past a dip's extremum
+    while (todo) {
+      const int q = __ffs(todo);                   // piece q: [(q - 1), q] / BACK_SUBDIV
+      const unsigned bit = 1u << (q - 1);
+      double lo = (double)(q - 1) / BACK_SUBDIV, hi = (double)q / BACK_SUBDIV;
+      bool neg = (negs & bit) != 0u, cross = true;
+      if (second) {
+        lo = te;
+        neg = !neg;
+        second = false;
+      } else if (dips & bit) {
+        cross = second = graze(c, lo, hi, neg, dense64, &te);
+        hi = te;
+      }
+      if (!second) todo &= ~bit;
+      if (cross) root(c, lo, hi, neg, dense64);
     }
   }
 
