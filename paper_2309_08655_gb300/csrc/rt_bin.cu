@@ -9,9 +9,9 @@
 //                      (shared memory, flushed once per block) and the sky map
 //                      (global atomics); 2^e is the largest power of two with
 //                      n * wmax * 2^e < 2^62;
-//   3. finalize_kernel q / 2^e to float64, one warp per sky cell, which sums
-//                      its row for the sky map (integer sums: the same whether
-//                      the rays or the bins are added).
+//   3. finalize_kernel q / 2^e to float64, one warp per sky cell (or part of its
+//                      row), which sums the row for the sky map (integer sums: the
+//                      same whether the rays or the bins are added).
 // n in the bound is BinParams::n_scale: the rays of this call, or of all shards
 // of a sharded binning (rt_bin_part_*), whose int64 sums add exactly.
 //
@@ -256,32 +256,47 @@ __global__ void __launch_bounds__(256) accum_kernel(BinParams p, Bins b) {
   }
 }
 
-__global__ void __launch_bounds__(256) finalize_kernel(BinParams p) {
+// One warp per segment of a sky cell's row (segs segments of len bins).  A whole row's
+// sum is the sky map's entry; of a row in segments the parts are added to the sums
+// behind the cube, for sky_kernel, unless the rays were (sum false).
+__global__ void __launch_bounds__(256) finalize_kernel(BinParams p, int segs, int len, bool sum) {
   const double inv = fixed_unit(p.acc[0], p.n_scale);
   const int nsky = p.nth * p.nph, nnu = p.nnu;
   const long long* g_hist = p.acc + 2;
-  const long long* g_spec = g_hist + (int64_t)nsky * nnu + nsky;
+  unsigned long long* g_sky = (unsigned long long*)p.acc + 2 + (int64_t)nsky * nnu;
+  const long long* g_spec = (const long long*)g_sky + nsky;
   const int lane = threadIdx.x & 31;
   const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int64_t threads = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t s = tid >> 5; s < nsky; s += threads >> 5) {
+  for (int64_t g = tid >> 5; g < (int64_t)nsky * segs; g += threads >> 5) {
+    const int64_t s = g / segs, lo = (g - s * segs) * len;
+    const int64_t hi = lo + len < nnu ? lo + len : nnu;
     const long long* row = g_hist + s * nnu;
     double* out = p.hist + s * nnu;
-    long long sum = 0;
-    for (int j = lane; j < nnu; j += 32) {
+    long long q_sum = 0;
+    for (int64_t j = lo + lane; j < hi; j += 32) {
       const long long q = row[j];
       out[j] = (double)q * inv;
-      sum += q;
+      q_sum += q;
     }
-    if (p.sky) {
+    if (p.sky && sum) {
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, o);
-      if (lane == 0) p.sky[s] = (double)sum * inv;
+      for (int o = 16; o > 0; o >>= 1) q_sum += __shfl_down_sync(0xffffffffu, q_sum, o);
+      if (lane == 0 && segs == 1) p.sky[s] = (double)q_sum * inv;
+      if (lane == 0 && segs > 1) atomicAdd(g_sky + s, (unsigned long long)q_sum);
     }
   }
   if (p.spec)
     for (int64_t j = tid; j < nnu; j += threads) p.spec[j] = (double)g_spec[j] * inv;
   if (tid == 0) *p.oor = (double)p.acc[1] * inv;
+}
+
+__global__ void __launch_bounds__(256) sky_kernel(BinParams p) {
+  const double inv = fixed_unit(p.acc[0], p.n_scale);
+  const int64_t nsky = (int64_t)p.nth * p.nph;
+  const long long* g_sky = p.acc + 2 + nsky * p.nnu;
+  const int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (s < nsky) p.sky[s] = (double)g_sky[s] * inv;
 }
 
 }  // namespace
@@ -330,24 +345,43 @@ cudaError_t launch_bin_accum(const BinParams& p, cudaStream_t stream) {
   return launch_accum<true, true>(p, stream);
 }
 
-cudaError_t launch_bin_finalize(const BinParams& p, cudaStream_t stream) {
+namespace {
+
+// marg: p.acc holds the sky map's sums already.
+cudaError_t launch_finalize(const BinParams& p, bool marg, cudaStream_t stream) {
   int nsm = 0;
   cudaError_t e = sm_count(&nsm);
   if (e != cudaSuccess) return e;
-  // one warp per sky cell, at least enough threads for the spectrum's entries
-  int64_t warps = (int64_t)p.nth * p.nph;
+  // One warp per row, or, with fewer rows than warps that the GPU holds, per segment of
+  // at least 256 bins (a spectrum alone is one row: 2^22 bins in one warp took 60 ms,
+  // shared out the whole call takes 87 us); at least enough threads for the spectrum's entries.
+  const int64_t nsky = (int64_t)p.nth * p.nph, warps_held = (int64_t)nsm * 64;
+  int64_t segs = nsky < warps_held ? warps_held / nsky : 1;
+  if (segs > (p.nnu + 255) / 256) segs = (p.nnu + 255) / 256;
+  const int len = (int)(((p.nnu + segs - 1) / segs + 31) / 32 * 32);
+  segs = (p.nnu + len - 1) / len;
+  int64_t warps = nsky * segs;
   if (p.spec && warps < (p.nnu + 31) / 32) warps = (p.nnu + 31) / 32;
   int64_t gf = (warps + BIN_BLOCK / 32 - 1) / (BIN_BLOCK / 32);
   if (gf > (int64_t)nsm * 8) gf = (int64_t)nsm * 8;
-  finalize_kernel<<<(unsigned)gf, BIN_BLOCK, 0, stream>>>(p);
+  finalize_kernel<<<(unsigned)gf, BIN_BLOCK, 0, stream>>>(p, (int)segs, len, segs == 1 || !marg);
+  e = cudaGetLastError();
+  if (e != cudaSuccess || segs == 1 || !p.sky) return e;
+  sky_kernel<<<(unsigned)((nsky + BIN_BLOCK - 1) / BIN_BLOCK), BIN_BLOCK, 0, stream>>>(p);
   return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_bin_finalize(const BinParams& p, cudaStream_t stream) {
+  return launch_finalize(p, true, stream);
 }
 
 cudaError_t launch_bin(const BinParams& p, cudaStream_t stream) {
   cudaError_t e = launch_bin_max(p, stream);
   if (e == cudaSuccess)
     e = p.spec ? launch_accum<false, true>(p, stream) : launch_accum<false, false>(p, stream);
-  if (e == cudaSuccess) e = launch_bin_finalize(p, stream);
+  if (e == cudaSuccess) e = launch_finalize(p, false, stream);
   return e;
 }
 
