@@ -343,7 +343,8 @@ __global__ void __launch_bounds__(128) batch_fp64_kernel(TraceParams p, ImgTable
   const int64_t total = nf + (t.list ? (int64_t)*t.list_n : t.npix);
   TraceParams tp = p;          // r_out per item
   tp.park = nullptr;
-  const int lanes = launch_lanes(t.list ? total - nf : total);
+  // (rays that are not of claim_status count, too: all of them are looked at here)
+  const int lanes = launch_lanes(total);
   int64_t item = lane < lanes ? -1 : -2;   // -1: needs an item, -2: queue exhausted
   int64_t ray = 0, pix = 0;
   int img = 0;
