@@ -1109,6 +1109,29 @@ rt_status rt_batch_set_norm(rt_batch* b, const int64_t* n_norm) {
   return RT_OK;
 }
 
+// The FP64 pass of a mixed launch (p and t as of its FP32 pass): the promoted rays from
+// where they stopped, in tail mode (rays guided along the null cone are among them; one
+// lane each they held the launch for 25 us an attempt), and with images (t) the pixels
+// that the FP32 pass listed, anew.
+static cudaError_t launch_promoted(rtk::TraceParams p, const rtk::ImgTable* t,
+                                   cudaStream_t stream) {
+  p.claim_status = rtk::RAY_PROMOTED;
+  p.refill_min = p.claim_size = 1;
+  p.order = 0;
+  p.xrec = nullptr;
+  p.sample_of = 0;
+  cudaError_t e = cudaSuccess;
+  if (p.n > 0 && (p.park || !t)) {
+    e = rtk::launch_trace_fp64(p, 0, 0, stream);
+    p.n = 0;
+  }
+  if (e != cudaSuccess || !t) return e;
+  rtk::ImgTable list = *t;
+  list.list = t->promo;
+  list.list_n = t->promo_n;
+  return rtk::launch_batch_fp64(p, list, 0, 0, stream);
+}
+
 rt_status rt_trace_batch(rt_batch* b, double* d_state, uint8_t* d_status, int32_t* d_nacc,
                          int32_t* d_nrej, int64_t* d_counters, const rt_trace_opts* o,
                          void* stream) {
@@ -1186,21 +1209,7 @@ rt_status rt_trace_batch(rt_batch* b, double* d_state, uint8_t* d_status, int32_
       e = cudaMemsetAsync(b->d_promo_n, 0, sizeof(unsigned long long), (cudaStream_t)stream);
       if (e == cudaSuccess) e = rtk::launch_batch_mixed(p, t, blk, bps, (cudaStream_t)stream);
       if (e != cudaSuccess) return cuda_fail(e, "mixed batch kernel");
-      // FP64: the promoted rays from where they stopped, in tail mode (rays guided
-      // along the null cone are among them; one lane each they held the launch for
-      // 25 us an attempt), and the listed pixels anew
-      p.claim_status = rtk::RAY_PROMOTED;
-      if (p.park && p.n > 0) {
-        rtk::TraceParams r = p;
-        r.refill_min = r.claim_size = 1;
-        e = rtk::launch_trace_fp64(r, 0, 0, (cudaStream_t)stream);
-        if (e != cudaSuccess) return cuda_fail(e, "trace kernel (promoted rays)");
-        p.n = 0;
-      }
-      p.refill_min = p.claim_size = 1;
-      t.list = b->d_promo;
-      t.list_n = b->d_promo_n;
-      e = rtk::launch_batch_fp64(p, t, 0, 0, (cudaStream_t)stream);
+      e = launch_promoted(p, &t, (cudaStream_t)stream);
       if (e != cudaSuccess) return cuda_fail(e, "batch kernel (promoted rays and pixels)");
       return RT_OK;
     }
@@ -1216,11 +1225,7 @@ rt_status rt_trace_batch(rt_batch* b, double* d_state, uint8_t* d_status, int32_
   if (o->precision == RT_PREC_MIXED) {
     e = rtk::launch_trace_mixed(p, blk, bps, (cudaStream_t)stream);
     if (e != cudaSuccess) return cuda_fail(e, "mixed trace kernel");
-    p.claim_status = rtk::RAY_PROMOTED;
-    p.refill_min = p.claim_size = 1;
-    p.order = 0;
-    p.xrec = nullptr;
-    e = rtk::launch_trace_fp64(p, 0, 0, (cudaStream_t)stream);
+    e = launch_promoted(p, nullptr, (cudaStream_t)stream);
     if (e != cudaSuccess) return cuda_fail(e, "trace kernel (promoted rays)");
     return RT_OK;
   }
@@ -1443,6 +1448,9 @@ rt_status rt_batch_autotune(rt_batch* b, const double* d_state, const uint8_t* d
   }
   const int64_t P = ioff[nimg];
   if (M + P == 0) return fail(RT_EINVAL, "nothing to tune on");
+  if (o->tail != 1 && o->lambda_max == 0.0 && !df &&
+      (st = ensure_park(&b->d_park, &b->park_cap)) != RT_OK)
+    return st;
   cudaStream_t cs = (cudaStream_t)stream;
   auto al = [](size_t x) { return (x + 255) / 256 * 256; };
   const size_t b_st = al((size_t)RT_STATE_ROWS * M * sizeof(double));
@@ -1536,7 +1544,13 @@ rt_status rt_batch_autotune(rt_batch* b, const double* d_state, const uint8_t* d
   p.counters = nullptr;
   p.queue = queue;
   p.ts = nullptr;
-  set_park(p, nullptr, 0, o);
+  // the claim order and the tail mode of the launch that is tuned (rt_trace_batch)
+  const bool tail = o->tail != 1 && o->lambda_max == 0.0 && !df;
+  set_park(p, tail ? b->d_park : nullptr, b->park_cap, o);
+  p.order = (o->claim_order == RT_CLAIM_COST && !img) ? 1 : 0;
+  if (!mixed && !df) set_express(p);
+  p.claim_status = rtk::RAY_READY;
+  p.sample_of = b->N + b->npix;
   p.rtol = o->rtol;
   p.atol = o->atol;
   p.r_out = o->r_out_over_R;
@@ -1579,11 +1593,8 @@ rt_status rt_batch_autotune(rt_batch* b, const double* d_state, const uint8_t* d
     }
     if (r == cudaSuccess && img) r = cudaMemsetAsync(promo_n, 0, sizeof(unsigned long long), cs);
     if (r == cudaSuccess) r = cudaEventRecord(ev0, cs);
-    p.claim_status = rtk::RAY_READY;
     p.refill_min = refill;
     p.claim_size = claim;
-    t.list = nullptr;
-    t.list_n = nullptr;
     if (r == cudaSuccess) {
       if (img)
         r = mixed ? rtk::launch_batch_mixed(p, t, block, bps, cs)
@@ -1593,18 +1604,7 @@ rt_status rt_batch_autotune(rt_batch* b, const double* d_state, const uint8_t* d
             : df  ? rtk::launch_trace_df(p, block, bps, cs)
                   : rtk::launch_trace_fp64(p, block, bps, cs);
     }
-    if (r == cudaSuccess && mixed) {
-      // the FP64 pass over the promoted rays (and the handed-over pixels)
-      p.claim_status = rtk::RAY_PROMOTED;
-      p.refill_min = p.claim_size = 1;
-      if (img) {
-        t.list = promo;
-        t.list_n = promo_n;
-        r = rtk::launch_batch_fp64(p, t, 0, 0, cs);
-      } else {
-        r = rtk::launch_trace_fp64(p, 0, 0, cs);
-      }
-    }
+    if (r == cudaSuccess && mixed) r = launch_promoted(p, img ? &t : nullptr, cs);
     if (r == cudaSuccess) r = cudaEventRecord(ev1, cs);
     if (r == cudaSuccess) r = cudaEventSynchronize(ev1);
     if (r == cudaSuccess) r = cudaEventElapsedTime(ms, ev0, ev1);

@@ -74,11 +74,14 @@ struct TraceParams {
   // lane for every entry of the queue
   int lanes = 32;
   int covers = 0;
+  // rays (and pixels) of the launch that this one is a sample of (rt_batch_autotune):
+  // lanes and covers are those of that launch
+  int64_t sample_of = 0;
 };
 // The words of TraceParams::queue: the claim counter, the number of marked guided
 // rays and the counter of the search for them (rt_guided.cuh).
 enum { QUEUE_CLAIM = 0, QUEUE_GUIDED = 1, QUEUE_SCAN = 2, QUEUE_WORDS = 3 };
-// Grid of a persistent launch over n rays, at most bps blocks of `block` threads per
+// Grid of a persistent launch over p.n rays, at most bps blocks of `block` threads per
 // SM, and the lanes of a warp that take rays: with fewer than 32 rays for each of four
 // warps per SM, every scheduler gets a warp and each warp its share (a warp's attempt
 // costs the branches that any of its lanes takes).  The lanes are those of the warps
@@ -87,18 +90,22 @@ enum { QUEUE_CLAIM = 0, QUEUE_GUIDED = 1, QUEUE_SCAN = 2, QUEUE_WORDS = 3 };
 struct PersistentShape {
   unsigned grid;
   int lanes;
+  bool covers;   // a lane for every ray
 };
-inline PersistentShape persistent_shape(int64_t n, int nsm, int block, int bps) {
-  auto lanes = [n](int64_t warps) {
-    const int64_t l = (n + warps - 1) / warps;
+inline PersistentShape persistent_shape(int64_t n, int64_t sample_of, int nsm, int block,
+                                        int bps) {
+  const int64_t whole = sample_of > n ? sample_of : n;
+  auto lanes = [](int64_t rays, int64_t warps) {
+    const int64_t l = (rays + warps - 1) / warps;
     return l < 1 ? 1 : l > 32 ? 32 : (int)l;
   };
   const int wpb = block / 32;
-  const int spread = lanes((int64_t)nsm * 4);
+  const int spread = lanes(whole, (int64_t)nsm * 4);
   const int64_t warps = (n + spread - 1) / spread;
   const int64_t useful = (warps + wpb - 1) / wpb, resident = (int64_t)nsm * bps;
   const int64_t grid = useful < 1 ? 1 : useful < resident ? useful : resident;
-  return {(unsigned)grid, lanes(grid * wpb)};
+  const int l = lanes(n, grid * wpb);
+  return {(unsigned)grid, l, grid * wpb * l >= whole};
 }
 constexpr int64_t XPARK_MIN_RAYS = (int64_t)4 << 20;
 constexpr int COST_BUCKETS = 3;
@@ -250,6 +257,8 @@ struct AdjLaunch {
   int max_steps;
   int64_t n;
   const double* u;
+  const double* state;    // the samples of u (launch_sample): 8 x n, weights; the
+  const double* weight;   // statuses in `status`
   const int64_t* ck_off;
   double* ck;
   double* seg;
@@ -257,8 +266,6 @@ struct AdjLaunch {
   // doubles per ray; order: the rays, longest first (n), built from nacc with
   // the 32 counters of bucket
   const int64_t* tape_off;
-  const double* state;    // the samples of u (launch_sample): 8 x n, weights; the
-  const double* weight;   // statuses in `status`
   double* tape;
   double* head;
   const int32_t* nacc;

@@ -344,7 +344,7 @@ __global__ void __launch_bounds__(128) batch_fp64_kernel(TraceParams p, ImgTable
   TraceParams tp = p;          // r_out per item
   tp.park = nullptr;
   // (rays that are not of claim_status count, too: all of them are looked at here)
-  const int lanes = launch_lanes(total);
+  const int lanes = launch_lanes(p.sample_of > total ? p.sample_of : total);
   int64_t item = lane < lanes ? -1 : -2;   // -1: needs an item, -2: queue exhausted
   int64_t ray = 0, pix = 0;
   int img = 0;
@@ -506,7 +506,7 @@ cudaError_t launch_backward(const BackLaunch& b, cudaStream_t stream) {
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, backward_kernel, block, 0);
   if (e != cudaSuccess) return e;
   const int64_t npix = (int64_t)b.nx * b.ny;
-  const unsigned grid = persistent_shape(npix, nsm, block, occ > 0 ? occ : 1).grid;
+  const unsigned grid = persistent_shape(npix, 0, nsm, block, occ > 0 ? occ : 1).grid;
   e = cudaMemsetAsync(b.queue, 0, sizeof(unsigned long long), stream);
   if (e != cudaSuccess) return e;
   backward_kernel<<<grid, block, 0, stream>>>(bp);
@@ -566,12 +566,13 @@ cudaError_t launch_trace_fp64(const TraceParams& p, int block, int blocks_per_sm
   // a launch with a lane for every entry of the queue has nothing to refill or to claim
   // in chunks.  So these options do not decide there which rays end in the six-lane
   // groups (their results differ by rounding).
-  if (p.n <= (int64_t)nsm * 4 * 32 && blocks_per_sm * (block / 32) < 4)
+  const int64_t whole = p.sample_of > p.n ? p.sample_of : p.n;
+  if (whole <= (int64_t)nsm * 4 * 32 && blocks_per_sm * (block / 32) < 4)
     blocks_per_sm = (4 * 32 + block - 1) / block;
-  const PersistentShape shape = persistent_shape(p.n, nsm, block, blocks_per_sm);
+  const PersistentShape shape = persistent_shape(p.n, p.sample_of, nsm, block, blocks_per_sm);
   TraceParams q = p;
   q.lanes = shape.lanes;
-  if (!p.order && (int64_t)shape.grid * (block / 32) * shape.lanes >= p.n) {
+  if (!p.order && shape.covers) {
     q.covers = 1;
     q.refill_min = 32;
     q.claim_size = 1;

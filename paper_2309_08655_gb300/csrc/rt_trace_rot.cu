@@ -453,7 +453,7 @@ cudaError_t launch_trace_rot(const TraceParams& p, int block, int blocks_per_sm,
   if (occ < 1) occ = 1;
   // resident blocks only: a share of the guided rays must not wait for a block
   if (blocks_per_sm <= 0 || blocks_per_sm > occ) blocks_per_sm = occ;
-  const PersistentShape shape = persistent_shape(p.n, nsm, block, blocks_per_sm);
+  const PersistentShape shape = persistent_shape(p.n, p.sample_of, nsm, block, blocks_per_sm);
   TraceParams q = p;
   q.lanes = shape.lanes;
   e = launch_guided(q, stream);
