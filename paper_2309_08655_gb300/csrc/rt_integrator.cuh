@@ -46,23 +46,75 @@ __device__ __forceinline__ double max_abs(double a, double b) {
   const long long y = __double_as_longlong(b) & 0x7fffffffffffffffll;
   return __longlong_as_double(x > y ? x : y);
 }
-// 1/x to rounding for normal x: the hardware's coarse reciprocal r (about 2^-20
-// off) corrected by the geometric series in the residual d = 1 - x r,
-// r (1 + d + d^2); the rest is d^3 ~ 2^-60.
-__device__ __forceinline__ double recip_series(double x) {
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+// Reciprocal, quotient and inverse square root to rounding, for arguments in FP32's
+// range (in_fp32: 2^-100 <= x < 2^100) from the FP32 unit's estimate at the leading 21
+// bits and one iteration of order three in FP64, for all others by CUDA's functions (a
+// tolerance may be as small as the smallest double).  A division takes ten FP64
+// instructions of 64 cycles and rsqrt() has a longer path around its special values; an
+// attempt has six quotients, a group's attempt twelve inverse roots: 4096 rays of the
+// aligned star 372 ms, 382 ms with CUDA's functions throughout; 16 x 251 rays of the
+// rotating one 544 and 562 ms.
+__device__ __forceinline__ bool in_fp32(double x) {
+  return (unsigned)(__double2hiint(x) - 0x39b00000) < 0x0c800000u;
+}
+__device__ __forceinline__ float lead_in_fp32(double x) {
+  return __int_as_float((unsigned)__double2hiint(x) * 8u + 0x40000000u);
+}
+__device__ __forceinline__ double widen_normal(float v) {
+  const int b = __float_as_int(v);
+  return __hiloint2double((b >> 3) + 0x38000000, b << 29);
+}
+// The hyperpower iteration r (1 + d + d^2) with the residual d = 1 - x r (Altman, Pacific
+// J. Math. 10 (1960) 1107); the estimate is off by at most 2^-23 and its argument by
+// 2^-20, so |d| < 2^-19 and the rest, d^3, is below 2^-57.
+__device__ __forceinline__ double recip_in_fp32(double x) {
+  float v;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(v) : "f"(lead_in_fp32(x)));
+  const double r = widen_normal(v);
   const double d = fma(-x, r, 1.0);
   return fma(r, fma(d, d, d), r);
 }
-
-// 1/sqrt(x) to rounding for normal positive x (NaN for negative): the hardware's
-// coarse estimate y corrected by the binomial series in e = 1 - x y^2 (~2^-19),
-// y (1 + e/2 + 3 e^2/8); the rest is O(e^3) ~ 2^-58.  Five FP64 instructions and
-// no branch.
-__device__ __forceinline__ double rsqrt_series(double x) {
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+__device__ __forceinline__ double recip(double x) { return in_fp32(x) ? recip_in_fp32(x) : 1.0 / x; }
+static __device__ __noinline__ double quotient_any(double a, double b) { return a / b; }
+__device__ __forceinline__ double quotient(double a, double b) {
+  return in_fp32(b) ? a * recip_in_fp32(b) : quotient_any(a, b);
+}
+// The squared error norm's sum: (err(i) / sc_i)^2 over the six components, sc = atol +
+// rtol max(|y|, |yn|), with one test of the range for all six quotients.
+template <class Err>
+__device__ __forceinline__ double error_sum(double atol, double rtol, const double* y,
+                                            const double* yn, const Err& err) {
+  double sc[6], s = 0.0;
+  bool plain = true;
+#pragma unroll
+  for (int i = 0; i < 6; ++i) {
+    sc[i] = atol + rtol * max_abs(y[i], yn[i]);
+    plain = plain && in_fp32(sc[i]);
+  }
+  if (plain) {
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+      const double q = err(i) * recip_in_fp32(sc[i]);
+      s += q * q;
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+      const double q = err(i) / sc[i];
+      s += q * q;
+    }
+  }
+  return s;
+}
+// Householder's iteration of order three for x y^2 = 1, y (1 + e/2 + 3 e^2/8) with e = 1 -
+// x y^2 (The Numerical Treatment of a Single Nonlinear Equation, 1970, sec. 4.4); the
+// estimate is off by at most 2^-22 and its argument by 2^-20, so |e| < 2^-19 and the
+// rest, 5 e^3/16, is below 2^-58.
+__device__ __forceinline__ double inv_sqrt(double x) {
+  if (!in_fp32(x)) return rsqrt(x);
+  float v;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(v) : "f"(lead_in_fp32(x)));
+  const double y = widen_normal(v);
   const double e = fma(-x, y * y, 1.0);
   return fma(y * e, fma(0.375, e, 0.5), y);
 }
@@ -279,7 +331,7 @@ __device__ __forceinline__ double event_root(const S64& f64, const S32& f32, dou
   const double a = widen(fmaxf(0.0f, l - SEED_WIDEN)), b = widen(fminf(1.0f, u + SEED_WIDEN));
   const double fa = f64(a), fb = f64(b);
   if (fa >= 0.0 && fb < 0.0) {
-    const double slope = (b - a) * recip_series(fa - fb);      // -1 / f'
+    const double slope = (b - a) * recip(fa - fb);      // -1 / f'
     double th = fma(fa, slope, a);
     th = fma(f64(th), slope, th);
     if (th >= a && th <= b) return th;
@@ -402,14 +454,10 @@ __device__ int advance(const TraceParams& p, Lane& L, Hook& hook) {
     yn[i] = y[i] + h * (DP::b1 * k1[i] + DP::b3 * k3[i] + DP::b4 * k4[i] + DP::b5 * k5[i] +
                         DP::b6 * k6[i]);
   rhs64(L.c, yn, k7);
-  double s = 0.0;
-#pragma unroll
-  for (int i = 0; i < 6; ++i) {
-    const double e = h * (DP::e1 * k1[i] + DP::e3 * k3[i] + DP::e4 * k4[i] + DP::e5 * k5[i] +
-                          DP::e6 * k6[i] + DP::e7 * k7[i]);
-    const double q = e * recip_series(p.atol + p.rtol * max_abs(y[i], yn[i]));
-    s += q * q;
-  }
+  const double s = error_sum(p.atol, p.rtol, y, yn, [&](int i) {
+    return h * (DP::e1 * k1[i] + DP::e3 * k3[i] + DP::e4 * k4[i] + DP::e5 * k5[i] +
+                DP::e6 * k6[i] + DP::e7 * k7[i]);
+  });
   // the squared error norm; <= 1 accepts
   const double en2 = s * (1.0 / 6.0);
   if ((__double2hiint(en2) & 0x7ff00000) == 0x7ff00000) {   // infinite or NaN

@@ -293,7 +293,7 @@ __device__ __forceinline__ double rhs_group(const GroupFile& f, const RayConst<d
   s[S_DOT + f.cc] = f.cc == 5 ? -d : d;
   __syncwarp(f.gm);
   const double rr = s[S_DOT + 3];
-  const double ir = rsqrt_series(rr);
+  const double ir = inv_sqrt(rr);
   // kr, mu, n_z, r^-2, 3 mu, rs/r
   const double v1 = f.cc == 2 ? s[S_X + 2] : f.cc == 3 ? ir : f.cc == 5 ? s[S_RS] : d;
   s[S_P1 + f.cc] = ir * v1;
@@ -308,7 +308,7 @@ __device__ __forceinline__ double rhs_group(const GroupFile& f, const RayConst<d
   const double p2 = pass(2);
   out[6] = p2;
   out[12] = pass(3);
-  s[S_Q + f.cc] = rsqrt_series(p2);
+  s[S_Q + f.cc] = inv_sqrt(p2);
   __syncwarp(f.gm);
 #pragma unroll
   for (int n = 4; n <= PASSES; ++n) {
@@ -391,7 +391,7 @@ __device__ __forceinline__ int advance_group(const TraceParams& p, const GroupFi
   K7 = rhs_group(f, L.c, yn, &rnew2, &Fnew);
   const double e = h * (DP::e1 * K1 + DP::e3 * K3 + DP::e4 * K4 + DP::e5 * K5 + DP::e6 * K6 +
                         DP::e7 * K7);
-  const double eq = e * recip_series(p.atol + p.rtol * max_abs(y, yn));
+  const double eq = quotient(e, p.atol + p.rtol * max_abs(y, yn));
   // the sum over the group: lanes c and c + 3 form the same pair sum, so every
   // lane holds the same bits
   const double pair = eq * eq + __shfl_sync(gm, eq * eq, base + (cc < 3 ? cc + 3 : cc - 3));

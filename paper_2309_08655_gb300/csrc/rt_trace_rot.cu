@@ -48,7 +48,7 @@ __device__ __forceinline__ void rhs_rot(RotLane& L, const double* y, double* f) 
   L.c.m0 = L.sin_tm * cp;
   L.c.m1 = L.sin_tm * sp;
   L.c.W2 = y[7] * y[7];
-  L.c.iW2 = recip_series(L.c.W2);
+  L.c.iW2 = recip(L.c.W2);
   double dw;
   ham_rhs64<double, true>(L.c, y[0], y[1], y[2], y[3], y[4], y[5], f[0], f[1], f[2], f[3], f[4],
                           f[5], &dw);
@@ -215,14 +215,10 @@ __device__ int advance_rot(const TraceParams& p, RotLane& L) {
     yn[i] = y[i] + h * (DP::b1 * k1[i] + DP::b3 * k3[i] + DP::b4 * k4[i] + DP::b5 * k5[i] +
                         DP::b6 * k6[i]);
   rhs_rot(L, yn, k7);
-  double s = 0.0;
-#pragma unroll
-  for (int i = 0; i < 6; ++i) {
-    const double e = h * (DP::e1 * k1[i] + DP::e3 * k3[i] + DP::e4 * k4[i] + DP::e5 * k5[i] +
-                          DP::e6 * k6[i] + DP::e7 * k7[i]);
-    const double q = e * recip_series(p.atol + p.rtol * max_abs(y[i], yn[i]));
-    s += q * q;
-  }
+  const double s = error_sum(p.atol, p.rtol, y, yn, [&](int i) {
+    return h * (DP::e1 * k1[i] + DP::e3 * k3[i] + DP::e4 * k4[i] + DP::e5 * k5[i] +
+                DP::e6 * k6[i] + DP::e7 * k7[i]);
+  });
   // the squared error norm; <= 1 accepts
   const double en2 = s * (1.0 / 6.0);
   if ((__double2hiint(en2) & 0x7ff00000) == 0x7ff00000) {   // infinite or NaN
