@@ -206,7 +206,7 @@ def _flops_per_attempt(rt):
     return rt.rt_flops_per_step(0, 0)
 
 
-def _roofline(prec, fl, fl_df, attempts, rays, promoted_attempts, t):
+def _roofline(prec, fl, fl_mixed, fl_df, attempts, rays, promoted_attempts, t):
     """ALU roofline of one trace call of `t` seconds: counted operations per
     attempt (and per ray for the initial step) against the measured peak of
     the pipe that executes them."""
@@ -215,9 +215,9 @@ def _roofline(prec, fl, fl_df, attempts, rays, promoted_attempts, t):
         r = {"kernel": FP64_KERNELS, "peak": PEAK["fp64"], "peak_source": PEAK_SOURCE["fp64"],
              "flops_per_attempt": fl[1]}
     elif prec == "mixed":
-        flops = (attempts - promoted_attempts) * fl[1] + rays * fl[2]
+        flops = (attempts - promoted_attempts) * fl_mixed[1] + rays * (2 * fl_mixed[0] + 60)
         r = {"kernel": "trace_mixed_kernel (+ FP64 pass for promoted rays)", "peak": PEAK["fp32"],
-             "peak_source": PEAK_SOURCE["fp32"], "flops_per_attempt": fl[1]}
+             "peak_source": PEAK_SOURCE["fp32"], "flops_per_attempt": fl_mixed[1]}
     else:
         # the FP32 operations the double-float arithmetic executes; the FP64
         # operations they stand for reported beside them
@@ -442,6 +442,7 @@ def run_ours(args):
 
     res = {}
     fl = _flops_per_attempt(rt)
+    fl_mixed = rt.rt_flops_per_step_mixed(0, 0)
     fl_df = rt.rt_flops_per_step_df(0, 0)
     peaks = _measure_peaks(rt, stream)
     clocks = Clocks(local)
@@ -471,7 +472,7 @@ def run_ours(args):
         rays_launch = c_sum[2] / args.steps
         promoted_attempts = c_sum[5] / args.steps
         t_tr = statistics.mean(t_trace)
-        roof = _roofline(prec, fl, fl_df, attempts, rays_launch, promoted_attempts, t_tr)
+        roof = _roofline(prec, fl, fl_mixed, fl_df, attempts, rays_launch, promoted_attempts, t_tr)
         if prec == "mixed":
             roof.update({"promoted_rays_per_step": c_sum[4] / args.steps,
                          "promoted_fp64_attempts_per_step": promoted_attempts})
@@ -508,7 +509,7 @@ def run_ours(args):
         T, acc_all, rays_all = shard.reduce_totals(e0.elapsed_time(e1) / 1e3, c[0], c[2], dev)
         t_tr = P.ev[0].elapsed_time(P.ev[1]) / 1e3
         attempts = c[0] + c[1]
-        roof = _roofline(prec, fl, fl_df, attempts, c[2], c[5], t_tr)
+        roof = _roofline(prec, fl, fl_mixed, fl_df, attempts, c[2], c[5], t_tr)
         roof.update({"attempts_per_launch": attempts, "trace_ms_per_launch": 1e3 * t_tr,
                      "steps_per_launch": K})
         hp = P.hist.cpu().numpy()

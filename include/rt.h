@@ -689,6 +689,13 @@ rt_status rt_count_status(int64_t n, const uint8_t* d_status, int64_t* counts, v
 rt_status rt_flops_per_step(int32_t dispersion, int32_t plasma, double* out4);
 
 /*
+ * rt_flops_per_step_mixed - the same for the FP32 stages of RT_PREC_MIXED, whose
+ * right-hand side is another form of the same equations with more operations: out2[0]
+ * per evaluation, out2[1] per step attempt.
+ */
+rt_status rt_flops_per_step_mixed(int32_t dispersion, int32_t plasma, double* out2);
+
+/*
  * rt_flops_per_step_df - the same for RT_PREC_DF, in the FP32 operations the
  * double-float kernel executes (host only): out2[0] per right-hand side
  * evaluation, out2[1] per step attempt.  A double-float sum counts 11, a

@@ -111,15 +111,13 @@ RT_HD __forceinline__ T gj_side(const T m0, const T m1, const T m2, const T x0, 
 
 // dx/dl = dH/dk, dk/dl = -dH/dx (Eq. Hamilton), analytic.  With XCORR the
 // position derivative is returned without its flat-space part 2k (the caller
-// then adds 2k itself, in higher precision).  With DW also *dw = dH/dW2, the
-// derivative with respect to omega_inf^2 = k_t^2 (for a Hamiltonian in which
-// k_t evolves).  (Host-callable only for the flop-counting scalar of
-// rt_flops.cu.)
-template <class T, bool XCORR = false, bool FIN = false, bool DW = false>
+// then adds 2k itself, in higher precision).  (Host-callable only for the
+// flop-counting scalar of rt_flops.cu.)
+template <class T, bool XCORR = false, bool FIN = false>
 RT_HD __forceinline__ void ham_rhs(const RayConst<T>& c, const T x0, const T x1,
                                         const T x2, const T k0, const T k1, const T k2, T& dx0,
                                         T& dx1, T& dx2, T& dk0, T& dk1, T& dk2,
-                                        const T F_in = T(0), T* dw = nullptr) {
+                                        const T F_in = T(0)) {
   const T r2 = x0 * x0 + x1 * x1 + x2 * x2;
   const T ir = rt_rsqrt(r2);
   const T n0 = x0 * ir, n1 = x1 * ir, n2 = x2 * ir;
@@ -187,7 +185,6 @@ RT_HD __forceinline__ void ham_rhs(const RayConst<T>& c, const T x0, const T x1,
     gx0 += dP0;
     gx1 += dP1;
     gx2 += dP2;
-    if (DW) *dw = -iA;                            // d(-W2/A)/dW2
   } else {
     // anisotropic term H_a = P - P A Kp^2 / W2 with Kp = U / |b|,
     // U = k.b + (sqrt(A) - 1) (n.k)(n.b), n.b = 2 mu, |b|^2 = 3 mu^2 + 1
@@ -219,7 +216,6 @@ RT_HD __forceinline__ void ham_rhs(const RayConst<T>& c, const T x0, const T x1,
     const T one_m = T(1) - A * Kp2iW2;
     const T cdA = -P * Kp2iW2 * c.rs * ir2;
     const T m2f = T(-2) * fac;
-    if (DW) *dw = Kp2iW2 * P * A * c.iW2 - iA;    // d(-W2/A - P A Kp^2/W2)/dW2
     gx0 += dP0 * one_m + cdA * n0 + m2f * dK0;
     gx1 += dP1 * one_m + cdA * n1 + m2f * dK1;
     gx2 += dP2 * one_m + cdA * n2 + m2f * dK2;
@@ -266,8 +262,9 @@ struct ConstGrad {
 // operations for the Goldreich-Julian anisotropic medium where ham_rhs takes 196;
 // the results differ by rounding.  (ham_rhs stays for the FP32 stages and the mixed
 // sweep, whose FP32 rounding is part of their results.)  With the shorter error
-// norm and event search: twisted magnetosphere, 16 x 4093 rays, 77 -> 55 ms.  DW: *dw = dH/dW2, as
-// ham_rhs.  CG: *cg = the derivatives with respect to the star's constants
+// norm and event search: twisted magnetosphere, 16 x 4093 rays, 77 -> 55 ms.  DW: *dw =
+// dH/dW2, the derivative with respect to omega_inf^2 = k_t^2 (for a Hamiltonian in which
+// k_t evolves).  CG: *cg = the derivatives with respect to the star's constants
 // (with dual numbers in the direction u, their tangents are u . grad_y of them:
 // the parameter part of a Jacobian product without a tangent per parameter).
 // C: the type of the ray's constants (T, or the plain scalar under a dual T).

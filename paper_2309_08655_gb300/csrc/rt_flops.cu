@@ -63,17 +63,17 @@ inline CntD rt_rsqrt(CntD v) {
 #pragma nv_diag_suppress 177
 #include "rt_device.cuh"
 
-extern "C" rt_status rt_flops_per_step(int32_t dispersion, int32_t plasma, double* out4) {
-  if (!out4) return RT_EINVAL;
-  if (dispersion < 0 || dispersion > 1 || plasma < 0 || plasma > 4) return RT_EINVAL;
+namespace {
+
+rtk::RayConst<Cnt> count_const(int32_t dispersion, int32_t plasma) {
   rtk::RayConst<Cnt> c;
   c.rs = 0.4; c.cp = 4000.0; c.pa = 0.1; c.W2 = 1.0; c.iW2 = 1.0;
   c.m0 = 0.3; c.m1 = 0.1; c.m2 = 0.9; c.sig = 1.0; c.disp = dispersion; c.plasma = plasma;
-  g_t = Tally();
-  Cnt d[6];
-  rtk::ham_rhs64<Cnt>(c, Cnt(20.0), Cnt(3.0), Cnt(-5.0), Cnt(0.3), Cnt(-0.4), Cnt(0.8), d[0], d[1],
-                    d[2], d[3], d[4], d[5]);
-  const double rhs = g_t.flops, rhs_special = g_t.special;
+  return c;
+}
+
+// Operations of an attempt outside its right-hand sides.
+double step_sums() {
   // Stage inputs y + h * sum_j a_sj k_j for stages 2..6 with 1..5 nonzero
   // coefficients: (2 nnz + 1) flops per component; the 5th-order update uses
   // b_1, b_3..b_6 (nnz = 5); the error estimate h * sum e_j k_j uses 6 terms
@@ -87,10 +87,37 @@ extern "C" rt_status rt_flops_per_step(int32_t dispersion, int32_t plasma, doubl
   comb += 6.0 * (2 * 6);
   comb += 6.0 * (2 + 1 + 2) + 2;
   comb += 5;
+  return comb;
+}
+
+}  // namespace
+
+extern "C" rt_status rt_flops_per_step(int32_t dispersion, int32_t plasma, double* out4) {
+  if (!out4) return RT_EINVAL;
+  if (dispersion < 0 || dispersion > 1 || plasma < 0 || plasma > 4) return RT_EINVAL;
+  const rtk::RayConst<Cnt> c = count_const(dispersion, plasma);
+  g_t = Tally();
+  Cnt d[6];
+  rtk::ham_rhs64<Cnt>(c, Cnt(20.0), Cnt(3.0), Cnt(-5.0), Cnt(0.3), Cnt(-0.4), Cnt(0.8), d[0], d[1],
+                    d[2], d[3], d[4], d[5]);
+  const double rhs = g_t.flops, rhs_special = g_t.special;
   out4[0] = rhs;                        // flops of one right-hand side evaluation
-  out4[1] = 6.0 * rhs + comb;           // flops of one step attempt (FSAL: 6 evaluations)
+  out4[1] = 6.0 * rhs + step_sums();    // flops of one step attempt (FSAL: 6 evaluations)
   out4[2] = 2.0 * rhs + 60.0;           // flops of the initial step heuristic (2 evaluations)
   out4[3] = 6.0 * rhs_special + 6 + 3;  // divisions / square roots / powers per attempt
+  return RT_OK;
+}
+
+extern "C" rt_status rt_flops_per_step_mixed(int32_t dispersion, int32_t plasma, double* out2) {
+  if (!out2) return RT_EINVAL;
+  if (dispersion < 0 || dispersion > 1 || plasma < 0 || plasma > 5) return RT_EINVAL;
+  const rtk::RayConst<Cnt> c = count_const(dispersion, plasma);
+  g_t = Tally();
+  Cnt d[6];
+  rtk::ham_rhs<Cnt>(c, Cnt(20.0), Cnt(3.0), Cnt(-5.0), Cnt(0.3), Cnt(-0.4), Cnt(0.8), d[0], d[1],
+                    d[2], d[3], d[4], d[5]);
+  out2[0] = g_t.flops;                       // flops of one right-hand side evaluation
+  out2[1] = 6.0 * g_t.flops + step_sums();   // flops of one step attempt
   return RT_OK;
 }
 

@@ -113,6 +113,9 @@ def lib():
         L.rt_flops_per_step.restype = ctypes.c_int
         L.rt_flops_per_step.argtypes = [ctypes.c_int32, ctypes.c_int32,
                                         ctypes.POINTER(ctypes.c_double)]
+        L.rt_flops_per_step_mixed.restype = ctypes.c_int
+        L.rt_flops_per_step_mixed.argtypes = [ctypes.c_int32, ctypes.c_int32,
+                                              ctypes.POINTER(ctypes.c_double)]
         L.rt_flops_per_step_df.restype = ctypes.c_int
         L.rt_flops_per_step_df.argtypes = [ctypes.c_int32, ctypes.c_int32,
                                            ctypes.POINTER(ctypes.c_double)]
@@ -361,6 +364,12 @@ def rt_flops_per_step(dispersion: int, plasma: int) -> list[float]:
     return list(out)
 
 
+def rt_flops_per_step_mixed(dispersion: int, plasma: int) -> list[float]:
+    out = (ctypes.c_double * 2)()
+    _check(lib().rt_flops_per_step_mixed(int(dispersion), int(plasma), out))
+    return list(out)
+
+
 def rt_flops_per_step_df(dispersion: int, plasma: int) -> list[float]:
     out = (ctypes.c_double * 2)()
     _check(lib().rt_flops_per_step_df(int(dispersion), int(plasma), out))
@@ -568,4 +577,5 @@ EXPORTED = ["rt_init_star", "rt_destroy_star", "rt_star_info", "rt_sample_conver
             "rt_batch_graph_create", "rt_graph_launch", "rt_graph_destroy", "rt_batch_autotune",
             "rt_batch_set_images", "rt_sample_conversion_surface_part", "rt_bin_part_max",
             "rt_bin_part_accumulate", "rt_bin_part_finalize", "rt_batch_set_norm",
-            "rt_measure_alu_peak", "rt_hamilton_rhs", "rt_flops_per_step_df"]
+            "rt_measure_alu_peak", "rt_hamilton_rhs", "rt_flops_per_step_df",
+            "rt_flops_per_step_mixed"]
