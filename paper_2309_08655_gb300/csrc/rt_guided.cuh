@@ -5,12 +5,14 @@
 // attempts, and a launch lasts as long as its longest ray.  Among 31 other lanes
 // every attempt of that ray also costs their crossings, escapes and refills.  So
 // these rays leave the plain queue before the launch (launch_guided: status
-// RAY_EXPRESS, their number beside the queue's counter), and a quarter of the
-// launch's warps, the first of each block, look for them in the statuses and trace
-// nothing else until none is left.  A ray is marked for where it starts and for
-// nothing else, so the rays beside it, the launch's shape and their number do not
-// change a result: the rotating kernel's are those of the plain queue, bit for bit,
-// and the double-float kernel traces every marked ray in FP64 groups.
+// RAY_EXPRESS within 1e-4 rad, RAY_GUIDED beyond, their number beside the queue's
+// counter), and a quarter of the launch's warps, the first of each block, look for
+// them in the statuses, the nearest first, and trace nothing else until none is left
+// (half of the warps, or a warp to itself for each of the nearest, changed nothing
+// beyond noise).  A ray is marked for where it starts and for nothing else, so the
+// rays beside it, the launch's shape and their number do not change a result: the
+// rotating kernel's are those of the plain queue, bit for bit, and the double-float
+// kernel traces every marked ray in FP64 groups.
 //
 // Not in the mixed kernel: there a second place that loads a ray made the compiler
 // contract other multiply-adds of the FP32 start (5 % of the rays took another step
@@ -34,7 +36,8 @@ __device__ __forceinline__ int guided_quota(const TraceParams& p) {
 }
 
 // A warp's search for marked rays: the statuses in chunks of 32, claimed from the
-// counter beside the queue's.  Every lane of the warp calls the members together.
+// counter beside the queue's, once for each mark.  Every lane of the warp calls the
+// members together.
 struct GuidedScan {
   int64_t base = 0;        // the chunk
   unsigned found = 0;      // its marked rays not yet taken
@@ -47,9 +50,11 @@ struct GuidedScan {
     while (found == 0 && open) {
       unsigned long long b = 0;
       if (lane == 0) b = atomicAdd(p.queue + QUEUE_SCAN, 32ull);
-      base = (int64_t)__shfl_sync(0xffffffffu, b, 0);
-      open = base < p.n;
-      const bool hit = base + lane < p.n && p.status[base + lane] == RAY_EXPRESS;
+      const int64_t at = (int64_t)__shfl_sync(0xffffffffu, b, 0), pass = (p.n + 31) & ~31ll;
+      open = at < 2 * pass;
+      base = at < pass ? at : at - pass;
+      const int want = at < pass ? RAY_EXPRESS : RAY_GUIDED;
+      const bool hit = open && base + lane < p.n && p.status[base + lane] == want;
       found = __ballot_sync(0xffffffffu, hit);
       if (once) break;
     }

@@ -174,7 +174,7 @@ cudaError_t launch_trace_fp64(const TraceParams& p, int block, int blocks_per_sm
                               cudaStream_t stream);
 cudaError_t launch_trace_mixed(const TraceParams& p, int block, int blocks_per_sm,
                                cudaStream_t stream);
-// Clears the queue's words, marks the guided rays (RAY_EXPRESS) and counts them.
+// Clears the queue's words, marks the guided rays and counts them.
 cudaError_t launch_guided(const TraceParams& p, cudaStream_t stream);
 cudaError_t launch_tail_fp64(const TraceParams& p, cudaStream_t stream);
 // Binning: launch_bin = clear p.acc, then the three phases; the phases alone

@@ -510,7 +510,8 @@ struct ParkedRays {
   const double* recs;
   unsigned long long lo, hi;
   unsigned long long* next;
-  // once an iteration, every lane of the warp (wants: the lane's group is free)
+  // before a free group takes one, every lane of the warp (wants: the lane's group is
+  // free; busy: it holds a ray)
   __device__ __forceinline__ void poll(const TraceParams&, bool, bool) {}
   // the lanes of a free group: its next record, or NULL (*done: no more will come)
   __device__ __forceinline__ const double* take(const TraceParams&, const GroupFile& f, int base,
@@ -532,7 +533,7 @@ struct FreshRays {
     const unsigned w = __ballot_sync(0xffffffffu, wants && lane % GROUP == 0);
     const unsigned b = __ballot_sync(0xffffffffu, busy);
     ray = -1;
-    if (w == 0 || !scan.more(p, b != 0)) return;
+    if (!scan.more(p, b != 0)) return;
     ray = scan.nth(__popc(w & ((1u << (lane - lane % GROUP)) - 1u)));
     scan.drop(__popc(w));
   }
@@ -566,46 +567,49 @@ __device__ void tail_groups(const TraceParams& p, Source& src, int ngroups, Grou
   bool have = false, done = !in_group;
   int na0 = 0, nr0 = 0;
   for (;;) {
-    src.poll(p, in_group && !have && !done, have);
-    if (in_group && !have && !done) {
-      const double* pe = src.take(p, f, base, &done);
-      if (pe) {
-        L.yc = pe[cc];
-        L.h = pe[6];
-        L.h_resume = pe[7];
-        const double sig = pe[8];
-        const int fl = (int)pe[9];
-        L.last_rej = (fl & 1) != 0;
-        L.switching = (fl & 2) != 0;
-        L.na = (int)pe[10];
-        L.nr = (int)pe[11];
-        L.ray = (int64_t)pe[12];
-        L.lam = pe[13];
-        L.star = find_star(p, L.ray);
-        const StarDev& s = p.stars[L.star];
-        const double om = 1.0 + p.state[6 * p.n + L.ray];
-        double sp, cpsi;
-        sincos(p.state[7 * p.n + L.ray], &sp, &cpsi);
-        L.c.rs = s.rs_prop;
-        L.c.cp = s.cp;
-        L.c.pa = s.plasma_a;
-        L.c.W2 = om * om;
-        L.c.iW2 = 1.0 / (om * om);
-        L.c.m0 = s.sin_tm * cpsi;
-        L.c.m1 = s.sin_tm * sp;
-        L.c.m2 = s.cos_tm;
-        L.c.disp = s.dispersion;
-        L.c.plasma = s.plasma;
-        L.c.sig = sig;
-        file_ray(f, L.c);
-        double F;
-        L.f0c = rhs_group(f, L.c, L.yc, &L.r2, &F);
-        na0 = L.na;
-        nr0 = L.nr;
-        have = true;
+    const bool wants = in_group && !have && !done;
+    if (__ballot_sync(0xffffffffu, wants)) {
+      src.poll(p, wants, have);
+      if (wants) {
+        const double* pe = src.take(p, f, base, &done);
+        if (pe) {
+          L.yc = pe[cc];
+          L.h = pe[6];
+          L.h_resume = pe[7];
+          const double sig = pe[8];
+          const int fl = (int)pe[9];
+          L.last_rej = (fl & 1) != 0;
+          L.switching = (fl & 2) != 0;
+          L.na = (int)pe[10];
+          L.nr = (int)pe[11];
+          L.ray = (int64_t)pe[12];
+          L.lam = pe[13];
+          L.star = find_star(p, L.ray);
+          const StarDev& s = p.stars[L.star];
+          const double om = 1.0 + p.state[6 * p.n + L.ray];
+          double sp, cpsi;
+          sincos(p.state[7 * p.n + L.ray], &sp, &cpsi);
+          L.c.rs = s.rs_prop;
+          L.c.cp = s.cp;
+          L.c.pa = s.plasma_a;
+          L.c.W2 = om * om;
+          L.c.iW2 = 1.0 / (om * om);
+          L.c.m0 = s.sin_tm * cpsi;
+          L.c.m1 = s.sin_tm * sp;
+          L.c.m2 = s.cos_tm;
+          L.c.disp = s.dispersion;
+          L.c.plasma = s.plasma;
+          L.c.sig = sig;
+          file_ray(f, L.c);
+          double F;
+          L.f0c = rhs_group(f, L.c, L.yc, &L.r2, &F);
+          na0 = L.na;
+          nr0 = L.nr;
+          have = true;
+        }
       }
+      if (__ballot_sync(0xffffffffu, in_group && !done) == 0) break;
     }
-    if (__ballot_sync(0xffffffffu, in_group && !done) == 0) break;
     if (have) {
       const int st = advance_group(p, f, L, cc, gm, base);
       if (st >= 0) {

@@ -72,8 +72,9 @@ __global__ void guided_mark_kernel(TraceParams p) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < p.n;
        i += (int64_t)gridDim.x * blockDim.x) {
     if (p.status[i] != RAY_READY) continue;
-    if (!(cone_dist2(p.stars[find_star(p, i)], p.state, p.n, i) < 1e-6)) continue;
-    p.status[i] = RAY_EXPRESS;
+    const double d2 = cone_dist2(p.stars[find_star(p, i)], p.state, p.n, i);
+    if (!(d2 < 1e-6)) continue;
+    p.status[i] = d2 < 1e-8 ? RAY_EXPRESS : RAY_GUIDED;
     ++marked;
   }
   marked = __reduce_add_sync(FULL, marked);
