@@ -256,9 +256,10 @@ __global__ void __launch_bounds__(256) accum_kernel(BinParams p, Bins b) {
   }
 }
 
-// One warp per segment of a sky cell's row (segs segments of len bins).  A whole row's
-// sum is the sky map's entry; of a row in segments the parts are added to the sums
+// One warp per sky cell's row, whose sum is the sky map's entry, or, with SEG, per
+// segment of it (segs segments of len bins): the parts' sums are then added to those
 // behind the cube, for sky_kernel, unless the rays were (sum false).
+template <bool SEG>
 __global__ void __launch_bounds__(256) finalize_kernel(BinParams p, int segs, int len, bool sum) {
   const double inv = fixed_unit(p.acc[0], p.n_scale);
   const int nsky = p.nth * p.nph, nnu = p.nnu;
@@ -268,22 +269,23 @@ __global__ void __launch_bounds__(256) finalize_kernel(BinParams p, int segs, in
   const int lane = threadIdx.x & 31;
   const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int64_t threads = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t g = tid >> 5; g < (int64_t)nsky * segs; g += threads >> 5) {
-    const int64_t s = g / segs, lo = (g - s * segs) * len;
-    const int64_t hi = lo + len < nnu ? lo + len : nnu;
+  const int64_t parts = SEG ? (int64_t)nsky * segs : nsky;
+  for (int64_t g = tid >> 5; g < parts; g += threads >> 5) {
+    const int64_t s = SEG ? g / segs : g;
+    const int lo = SEG ? (int)(g - s * segs) * len : 0, hi = SEG ? min(lo + len, nnu) : nnu;
     const long long* row = g_hist + s * nnu;
     double* out = p.hist + s * nnu;
     long long q_sum = 0;
-    for (int64_t j = lo + lane; j < hi; j += 32) {
+    for (int j = lo + lane; j < hi; j += 32) {
       const long long q = row[j];
       out[j] = (double)q * inv;
       q_sum += q;
     }
-    if (p.sky && sum) {
+    if (p.sky && (!SEG || sum)) {
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) q_sum += __shfl_down_sync(0xffffffffu, q_sum, o);
-      if (lane == 0 && segs == 1) p.sky[s] = (double)q_sum * inv;
-      if (lane == 0 && segs > 1) atomicAdd(g_sky + s, (unsigned long long)q_sum);
+      if (lane == 0 && !SEG) p.sky[s] = (double)q_sum * inv;
+      if (lane == 0 && SEG) atomicAdd(g_sky + s, (unsigned long long)q_sum);
     }
   }
   if (p.spec)
@@ -364,7 +366,10 @@ cudaError_t launch_finalize(const BinParams& p, bool marg, cudaStream_t stream) 
   if (p.spec && warps < (p.nnu + 31) / 32) warps = (p.nnu + 31) / 32;
   int64_t gf = (warps + BIN_BLOCK / 32 - 1) / (BIN_BLOCK / 32);
   if (gf > (int64_t)nsm * 8) gf = (int64_t)nsm * 8;
-  finalize_kernel<<<(unsigned)gf, BIN_BLOCK, 0, stream>>>(p, (int)segs, len, segs == 1 || !marg);
+  if (segs == 1)
+    finalize_kernel<false><<<(unsigned)gf, BIN_BLOCK, 0, stream>>>(p, 1, p.nnu, true);
+  else
+    finalize_kernel<true><<<(unsigned)gf, BIN_BLOCK, 0, stream>>>(p, (int)segs, len, !marg);
   e = cudaGetLastError();
   if (e != cudaSuccess || segs == 1 || !p.sky) return e;
   sky_kernel<<<(unsigned)((nsky + BIN_BLOCK - 1) / BIN_BLOCK), BIN_BLOCK, 0, stream>>>(p);

@@ -598,7 +598,7 @@ cudaError_t launch_trace_df(const TraceParams& p, int block, int blocks_per_sm,
     // instruction supply, not by the number of warps)
     blocks_per_sm = block >= 128 ? 1 : (occ < 128 / block ? occ : 128 / block);
   }
-  // resident blocks only: a share of the guided rays must not wait for a block
+  // resident blocks only: the warps that look for the guided rays start with the launch
   if (blocks_per_sm > occ) blocks_per_sm = occ;
   const PersistentShape shape = persistent_shape(p.n, p.sample_of, nsm, block, blocks_per_sm);
   TraceParams q = p;

@@ -447,7 +447,7 @@ cudaError_t launch_trace_rot(const TraceParams& p, int block, int blocks_per_sm,
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, trace_rot_kernel, block, 0);
   if (e != cudaSuccess) return e;
   if (occ < 1) occ = 1;
-  // resident blocks only: a share of the guided rays must not wait for a block
+  // resident blocks only: the warps that look for the guided rays start with the launch
   if (blocks_per_sm <= 0 || blocks_per_sm > occ) blocks_per_sm = occ;
   const PersistentShape shape = persistent_shape(p.n, p.sample_of, nsm, block, blocks_per_sm);
   TraceParams q = p;
