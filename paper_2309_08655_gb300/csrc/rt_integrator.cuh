@@ -48,15 +48,19 @@ __device__ __forceinline__ double max_abs(double a, double b) {
 }
 // Reciprocal, quotient and inverse square root to rounding, for arguments in FP32's
 // range (in_fp32: 2^-100 <= x < 2^100) from the FP32 unit's estimate at the leading 21
-// bits and one iteration of order three in FP64, for all others by CUDA's functions (a
-// tolerance may be as small as the smallest double).  A division takes ten FP64
+// bits and one step of Chebyshev's iteration of order three in FP64 (Traub, Iterative
+// Methods for the Solution of Equations, 1964: t - f/f' - f^2 f''/(2 f'^3)), for all
+// others by CUDA's functions (a tolerance may be as small as the smallest double).  A division takes ten FP64
 // instructions of 64 cycles and rsqrt() has a longer path around its special values; an
 // attempt has six quotients, a group's attempt twelve inverse roots: 4096 rays of the
-// aligned star 372 ms, 382 ms with CUDA's functions throughout; 16 x 251 rays of the
-// rotating one 544 and 562 ms.
+// aligned star 371 ms, 382 ms with CUDA's functions throughout; 16 x 251 rays of the
+// rotating one 540 and 562 ms.  CUDA's functions stand in copies of their own: inlined
+// at every use they cost the double-float kernel, which waits for instructions, 2 %.
 __device__ __forceinline__ bool in_fp32(double x) {
   return (unsigned)(__double2hiint(x) - 0x39b00000) < 0x0c800000u;
 }
+static __device__ __noinline__ double quotient_any(double a, double b) { return a / b; }
+static __device__ __noinline__ double rsqrt_any(double x) { return rsqrt(x); }
 __device__ __forceinline__ float lead_in_fp32(double x) {
   return __int_as_float((unsigned)__double2hiint(x) * 8u + 0x40000000u);
 }
@@ -64,9 +68,8 @@ __device__ __forceinline__ double widen_normal(float v) {
   const int b = __float_as_int(v);
   return __hiloint2double((b >> 3) + 0x38000000, b << 29);
 }
-// The hyperpower iteration r (1 + d + d^2) with the residual d = 1 - x r (Altman, Pacific
-// J. Math. 10 (1960) 1107); the estimate is off by at most 2^-23 and its argument by
-// 2^-20, so |d| < 2^-19 and the rest, d^3, is below 2^-57.
+// f = 1/r - x: r (1 + d + d^2) with d = 1 - x r; the estimate is off by at most 2^-23 and
+// its argument by 2^-20, so |d| < 2^-19 and the rest, d^3, is below 2^-57.
 __device__ __forceinline__ double recip_in_fp32(double x) {
   float v;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(v) : "f"(lead_in_fp32(x)));
@@ -74,8 +77,9 @@ __device__ __forceinline__ double recip_in_fp32(double x) {
   const double d = fma(-x, r, 1.0);
   return fma(r, fma(d, d, d), r);
 }
-__device__ __forceinline__ double recip(double x) { return in_fp32(x) ? recip_in_fp32(x) : 1.0 / x; }
-static __device__ __noinline__ double quotient_any(double a, double b) { return a / b; }
+__device__ __forceinline__ double recip(double x) {
+  return in_fp32(x) ? recip_in_fp32(x) : quotient_any(1.0, x);
+}
 __device__ __forceinline__ double quotient(double a, double b) {
   return in_fp32(b) ? a * recip_in_fp32(b) : quotient_any(a, b);
 }
@@ -100,18 +104,16 @@ __device__ __forceinline__ double error_sum(double atol, double rtol, const doub
   } else {
 #pragma unroll
     for (int i = 0; i < 6; ++i) {
-      const double q = err(i) / sc[i];
+      const double q = quotient_any(err(i), sc[i]);
       s += q * q;
     }
   }
   return s;
 }
-// Householder's iteration of order three for x y^2 = 1, y (1 + e/2 + 3 e^2/8) with e = 1 -
-// x y^2 (The Numerical Treatment of a Single Nonlinear Equation, 1970, sec. 4.4); the
-// estimate is off by at most 2^-22 and its argument by 2^-20, so |e| < 2^-19 and the
-// rest, 5 e^3/16, is below 2^-58.
+// f = 1/y^2 - x: y (1 + e/2 + 3 e^2/8) with e = 1 - x y^2; the estimate is off by at most
+// 2^-22 and its argument by 2^-20, so |e| < 2^-19 and the rest, 5 e^3/16, is below 2^-58.
 __device__ __forceinline__ double inv_sqrt(double x) {
-  if (!in_fp32(x)) return rsqrt(x);
+  if (!in_fp32(x)) return rsqrt_any(x);
   float v;
   asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(v) : "f"(lead_in_fp32(x)));
   const double y = widen_normal(v);
