@@ -466,9 +466,10 @@ rt_status rt_trace_backward(const rt_star* star, int32_t nx, int32_t ny, double 
  *   RT_PREC_FP64 FP64; RT_PREC_MIXED the adjoint of the state and its
  *   Jacobian products in FP64, the tangents of the three constants of the
  *   ray equations (r_s, the omega_p^2 coefficient, the magnetic axis) and
- *   their products with the adjoint in FP32 (about 1e-5 from the FP64 sweep,
- *   in half the FP64 sweep's time); RT_PREC_DF double-float (FP64-class
- *   rounding on the FP32 pipe; slower than the FP64 sweep on GB300).
+ *   their products with the adjoint in FP32 (about 1e-5 from the FP64 sweep;
+ *   its three tangents now make it slower than that sweep's one: the whole
+ *   gradient takes 3.7 times the forward run against 2.9); RT_PREC_DF
+ *   double-float (FP64-class rounding on the FP32 pipe; 4.2 times).
  *     d_grad     out: 6 float64, dF/dp
  *     d_F        out: 1 float64, F recomputed by the adjoint's replay
  *     d_status   out (may be NULL): n final statuses of the replay

@@ -110,7 +110,7 @@ __device__ void fresh_record(const TraceParams& p, int64_t ray, double* pe) {
 // and store the result to a slot.  The slot numbers are one table, read into
 // registers when a ray is taken up, so a pass is three loads, the multiply-add and
 // a store: 32 FP64 instructions a right-hand side, where every lane forming every
-// scalar takes 105.  A lone guided ray: 12.6 us an attempt (26 k cycles, of which
+// scalar takes 105.  A lone guided ray: 12.8 us an attempt (26 k cycles, of which
 // about 310 FP64 instructions take 20 k), 33 us with the prefix formed by every
 // lane; operands exchanged by shuffles and picked by selects took 13 other
 // instructions for each FP64 one, 23.5 us.

@@ -515,7 +515,7 @@ __global__ void __launch_bounds__(256) trace_df_kernel(TraceParams p) {
   // rays that start nearest the null cone first)
   const int64_t nq = p.order ? (int64_t)COST_BUCKETS * p.n : p.n;
   {
-    // the guided rays six lanes each in FP64, from the start of the launch: 12.6 us
+    // the guided rays six lanes each in FP64, from the start of the launch: 12.8 us
     // an attempt where a lone double-float lane takes 18, on a pipe that the rest
     // of the launch leaves idle
     const int quota = guided_quota(p);
